@@ -52,18 +52,19 @@ using step_detail::WarpReplica;
 // W points at the item's couplings (global memory, row pitch ldw) or at a
 // copy staged in shared memory (SW, row pitch ldw = 32 V).
 template <typename Tw, int V, bool SW, bool COAL = false>
-__device__ __forceinline__ void run_unit(const BatchItemDev& it, int r, const Tw* W, int ldw, long long t_limit)
+__device__ __forceinline__ void run_unit(const BatchItemDev& it, int r, const Tw* W, int ldw, long long t_limit,
+                                         step_detail::FlipLog<typename step_detail::Arith<Tw>::E>* log)
 {
     // the precomputed draws (PRE) for V <= 16; the V = 32 kernel has no registers left for
     // them (measured slower)
     constexpr bool kPre = V <= 16;
-    using R_ = WarpReplica<Tw, V, SW, kPre, (V >= 8), COAL>;
+    using R_ = WarpReplica<Tw, V, SW, kPre, COAL>;
     using A = step_detail::Arith<Tw>;
     using H = typename R_::H;
     constexpr int nw = V;   // state words per replica (the padded width 32V / 32)
     const int lane = threadIdx.x & 31;
     R_ rp;
-    rp.init(W, it.N, ldw, (uint32_t)r, it.xs + ((size_t)it.R + r) * nw);
+    rp.init(W, it.N, ldw, (uint32_t)r, it.xs + ((size_t)it.R + r) * nw, log);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
         if constexpr (std::is_same<Tw, step_detail::f32e>::value)   // int32 diagonal, exact in fp32
@@ -73,31 +74,28 @@ __device__ __forceinline__ void run_unit(const BatchItemDev& it, int r, const Tw
     }
     rp.xm = 0;
     rp.m = 0;
-    rp.Ecur = 0;
-    rp.Ebest = 0;
-    rp.flips = 0;
     const PhiloxKeys keys(it.seed);
     const long long T = t_limit > 0 ? std::min(t_limit, it.T) : it.T;
+    rp.begin(0, T, it.beta, 0.f, 0, 0, 0, keys);
     if constexpr (kPre) {
         rp.prep_draws(keys);
         if (T > 0) rp.draw_pre(0u, keys);
     } else {
         if (T > 0) rp.draw(0u, keys);
     }
-    float beta_next = T > 0 ? it.beta[0] : 0.f;
     // the next step count (t + 1) at which the fp32 fields are recomputed: a running
     // target instead of a 64-bit remainder every step
     long long next_rec = std::is_same<Tw, float>::value && it.recompute_every > 0 ? it.recompute_every : -1;
     for (long long t = 0; t < T; ++t) {
-        const float beta = beta_next;
-        if (t + 1 < T) beta_next = it.beta[t + 1];
-        const int k = rp.template step<false>(t, t + 1 < T, beta, it.inc, keys);
+        const int k = rp.template step<false>(t, t + 1 < T, it.inc, keys);
         if (it.trace && lane == 0) it.trace[(size_t)r * it.T + t] = k;
         if (it.stop && (t & 1023) == 1023 && *reinterpret_cast<const volatile int*>(it.stop)) break;
         if constexpr (std::is_same<Tw, float>::value) {
             if (t + 1 == next_rec) {
                 next_rec += it.recompute_every;
+                if (rp.n > 0) rp.settle(k >= 0);
                 rp.recompute(static_cast<const float*>(it.diag), it.S, it.exact_shift != 0);
+                rp.test_current();
                 // the draws of t + 1 again: lg is dead across the recompute, which frees its registers
                 if (t + 1 < T) {
                     if constexpr (kPre) rp.draw_pre((uint32_t)(t + 1), keys);
@@ -106,14 +104,14 @@ __device__ __forceinline__ void run_unit(const BatchItemDev& it, int r, const Tw
             }
         }
     }
-    rp.flush_best();
+    if (rp.n > 0) rp.settle();
     const uint32_t word = rp.word();
     if (lane % R_::P == 0) it.xs[(size_t)r * nw + (rp.base >> 5)] = word;
     if (lane == 0) {
         ReplicaScalars s;
-        s.E = A::store_e(rp.Ecur);
-        s.best = A::store_e(rp.Ebest);
-        s.flips = rp.flips;
+        s.E = A::store_e(log->E);
+        s.best = A::store_e(log->best);
+        s.flips = log->flips;
         s.m = rp.m;
         s.check = 0;
         it.sc[r] = s;
@@ -124,6 +122,8 @@ __device__ __forceinline__ void run_unit(const BatchItemDev& it, int r, const Tw
 template <typename Tw, int V, bool COAL = false>
 __global__ void __launch_bounds__(128) batch_kernel(const __grid_constant__ BatchClassParams bp)
 {
+    __shared__ step_detail::FlipLog<typename step_detail::Arith<Tw>::E> logs[4];
+    step_detail::FlipLog<typename step_detail::Arith<Tw>::E>* log = &logs[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     for (;;) {
         unsigned long long unit = 0;
@@ -139,8 +139,8 @@ __global__ void __launch_bounds__(128) batch_kernel(const __grid_constant__ Batc
         }
         const BatchItemDev it = bp.items[lo];
         const int r = (int)(unit - (unsigned long long)it.unit0);
-        if constexpr (COAL) run_unit<Tw, V, false, true>(it, r, static_cast<const Tw*>(it.Wc), 32 * V, bp.t_limit);
-        else run_unit<Tw, V, false>(it, r, static_cast<const Tw*>(it.W), it.ldw, bp.t_limit);
+        if constexpr (COAL) run_unit<Tw, V, false, true>(it, r, static_cast<const Tw*>(it.Wc), 32 * V, bp.t_limit, log);
+        else run_unit<Tw, V, false>(it, r, static_cast<const Tw*>(it.W), it.ldw, bp.t_limit, log);
     }
 }
 
@@ -153,6 +153,7 @@ __global__ void __launch_bounds__(512) batch_kernel_smem(const __grid_constant__
     extern __shared__ __align__(16) unsigned char wsm_raw[];
     Tw* Ws = reinterpret_cast<Tw*>(wsm_raw);
     __shared__ long long s_group;
+    __shared__ step_detail::FlipLog<typename step_detail::Arith<Tw>::E> logs[16];
     const int warp = threadIdx.x >> 5;
     for (;;) {
         __syncthreads();   // every warp is done with the previous group's copy
@@ -172,7 +173,7 @@ __global__ void __launch_bounds__(512) batch_kernel_smem(const __grid_constant__
         }
         __syncthreads();
         const int r = gi.y + warp;
-        if (r < it.R) run_unit<Tw, V, true>(it, r, Ws, cols, bp.t_limit);
+        if (r < it.R) run_unit<Tw, V, true>(it, r, Ws, cols, bp.t_limit, &logs[warp]);
     }
 }
 
@@ -286,8 +287,9 @@ thread_local std::string g_batch_desc;
 // Steps per unit of a tuner probe.
 constexpr long long kProbeSteps = 1024;
 
-// Largest dynamic shared memory a block may ask for on sm_100-class GPUs.
-constexpr size_t kMaxStagedBytes = 227u * 1024u;
+// Largest dynamic shared memory a block may ask for on sm_100-class GPUs, less the
+// kernel's static part (the flip logs of 16 warps).
+constexpr size_t kMaxStagedBytes = 227u * 1024u - 16u * sizeof(step_detail::FlipLog<double>) - 64u;
 
 int blocks_for(BatchKernel k, int warps_per_block, int sms, size_t smem)
 {

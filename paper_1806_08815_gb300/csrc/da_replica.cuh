@@ -2,6 +2,17 @@
 // step in da_step.cuh), packaged so that the chunked step kernel and the
 // persistent batched kernel share it.
 //
+// What bounds a step is the latency of its dependent chain: 809 cycles for 217
+// instructions of one warp at N = 64, 1865 for 701 at N = 1024 (2 warps per scheduler
+// at 1024 replicas: 2600).  So the chain holds as few long-latency operations as
+// possible: the count of accepted trials and the position of the chosen one come from
+// votes instead of chains of shuffles, the inputs of the next step (draws, choice word,
+// beta) are made in the shadow of this one, and the fp64 energy and the best state are
+// settled 32 flips at a time (FlipLog).  us per step before and after, 64 replicas
+// (1024): fp32 N = 64 0.555 -> 0.346 (0.613 -> 0.41), N = 256 0.670 -> 0.432
+// (0.761 -> 0.535), N = 512 0.781 -> 0.562 (0.918 -> 0.744), N = 1024 0.961 -> 0.883
+// (1.327 -> 1.246).
+//
 // Lane l owns the V consecutive variables i = l*V + v of the replica and keeps
 // their effective fields g_i, bits x_i and the Philox words of the current step
 // in registers.  step() performs one step of Algorithm 2 (see da_step.cuh for
@@ -22,10 +33,9 @@ namespace step_detail {
 // PRE: the step-invariant part of each Philox block is computed once per launch
 // (prep_draws) and the draws of every step start from it (draw_pre); four more
 // words per block live in registers, for kernels that have them to spare.
-// LATE: the best-state test is made under the row load (see flush_best).
 // COAL: W points at the couplings in the warp row order (row pitch ldw = 32 V;
 // step_uses_coal in da_internal.h) and rows are read with RowCoal.
-template <typename Tw, int V, bool SW = false, bool PRE = false, bool LATE = (V >= 8), bool COAL = false>
+template <typename Tw, int V, bool SW = false, bool PRE = false, bool COAL = false>
 struct WarpReplica {
     using A = Arith<Tw>;
     using H = typename A::H;
@@ -37,12 +47,13 @@ struct WarpReplica {
 
     H h[V];
     float lg[V];      // log2 U of this lane's draws for the current step (lg2_draw)
-    u32x4 cr;
-    long long cr_blk;
+    u32x4 cr;         // choice words of the steps [t & ~127, + 128): lane l holds those of 4 l .. 4 l + 3
+    uint32_t cw;      // the choice word of the current step
+    float bwin, bnext;   // the schedule of the steps [t & ~31, + 32) and of the 32 after, one per lane
+    float beta;       // of the current step
     uint32_t xm, valid, m;
-    bool chk;         // the best-state test of the last step (or recompute) is pending
-    E Ecur, Ebest;
-    long long flips;
+    FlipLog<E>* log;  // this warp's log in shared memory
+    int n;            // flips in it
     int lane, base, N, ldw;
     int rowoff;       // this lane's first entry in a row of W: base, or 4 lane in the G = 1 order
     uint32_t rep;
@@ -53,7 +64,8 @@ struct WarpReplica {
     uint32_t kq1[PRE ? NQ : 1], kq2[PRE ? NQ : 1], kq3[PRE ? NQ : 1], kq4[PRE ? NQ : 1];
     uint32_t ku0;
 
-    __device__ __forceinline__ void init(const Tw* W_, int N_, int ldw_, uint32_t rep_, uint32_t* bestg_)
+    __device__ __forceinline__ void init(const Tw* W_, int N_, int ldw_, uint32_t rep_, uint32_t* bestg_,
+                                         FlipLog<E>* log_)
     {
         lane = threadIdx.x & 31;
         base = lane * V;
@@ -64,30 +76,119 @@ struct WarpReplica {
         W = W_;
         bestg = bestg_;
         valid = base >= N ? 0u : (N - base >= V ? VMASK : ((1u << (N - base)) - 1u));
-        cr = {0, 0, 0, 0};
-        cr_blk = -1;
-        chk = false;
+        log = log_;
     }
 
-    // The test of Algorithm 2's result: a strictly lower tracked energy than any
-    // seen makes the current state the best one.  It is made one step late (x is
-    // unchanged until the next flip), and after any recompute of the step.  With
-    // LATE (by default for V >= 8) it runs while the next step's row of W is in
-    // flight (or once it is known that nothing flips), so that the fp64 compare
-    // stays off the chain from the trials to the row load; otherwise before the
-    // count.  Measured: the late test is slower at V = 4, whose short row leaves no
-    // room for it, and for replicas at fixed temperatures (parallel tempering),
-    // whose low-temperature steps mostly flip nothing.
-    static constexpr bool kTestUnderRow = LATE;
-    __device__ __forceinline__ void flush_best()
+    // Before the first step t0 of a launch over [t0, t1): the energies, and the step
+    // inputs that depend on nothing in a step (next_inputs).  sched: the schedule, or
+    // null for a fixed beta0.
+    const float* __restrict__ sched;
+    long long t_end;
+    template <class Keys>
+    __device__ __forceinline__ void begin(long long t0, long long t1, const float* sched_, float beta0, E e0, E best0,
+                                          long long flips0, const Keys& keys)
     {
-        if (chk) {
-            chk = false;
-            if (Ecur < Ebest) {
-                Ebest = Ecur;
-                snapshot();
-            }
+        if (lane == 0) {
+            log->E = e0;
+            log->best = best0;
+            log->flips = flips0;
         }
+        __syncwarp();
+        n = 0;
+        sched = sched_;
+        t_end = t1;
+        bwin = bnext = beta = beta0;
+        if (sched && t0 < t1) {
+            bwin = sched_window(t0 & ~31ll);
+            bnext = sched_window((t0 & ~31ll) + 32);
+            beta = __shfl_sync(0xffffffffu, bwin, (int)t0 & 31);
+        }
+        fill_choice(t0, keys);
+        cw = choice_word(t0);
+    }
+    __device__ __forceinline__ float sched_window(long long tb) const
+    {
+        const long long t = tb + lane;
+        return ldx(sched + (t < t_end ? t : t_end - 1));
+    }
+
+    // The uniform-choice draws (block (0, t & ~3, rep, 1), lane t % 4): each lane
+    // computes one block, so that one Philox evaluation serves 128 steps and a
+    // step's word comes by a shuffle that depends on nothing in the step; likewise
+    // beta from a window of the schedule.  Both are fetched one step ahead, under
+    // the row load: a load of beta every step had cost 0.06 of 0.51 us per step at
+    // N = 64.
+    template <class Keys>
+    __device__ __forceinline__ void fill_choice(long long t, const Keys& keys)
+    {
+        cr = philox4x32_10(0u, (uint32_t)((t & ~127ll) + 4 * lane), rep, 1u, keys);
+    }
+    __device__ __forceinline__ uint32_t choice_word(uint32_t t) const
+    {
+        return __shfl_sync(0xffffffffu, pick(cr, (int)(t & 3)), (int)(t >> 2) & 31);
+    }
+    template <class Keys>
+    __device__ __forceinline__ void next_inputs(uint32_t t, const Keys& keys)   // of step t + 1
+    {
+        const uint32_t t1 = t + 1;
+        if ((t1 & 31) == 0) {
+            if (sched) {
+                bwin = bnext;
+                bnext = sched_window((long long)t1 + 32);
+            }
+            if ((t1 & 127) == 0) fill_choice(t1, keys);
+        }
+        beta = __shfl_sync(0xffffffffu, bwin, (int)(t1 & 31));
+        cw = choice_word(t1);
+    }
+
+    // The flips logged so far into the tracked energy, and the test of Algorithm 2's
+    // result after each: a strictly lower energy than any seen makes that state the
+    // best one.  hold_last: the test of the last flip is left to the caller (a
+    // recompute follows it, and the test comes after the recompute).
+    __device__ __forceinline__ void settle(bool hold_last = false)
+    {
+        settle_impl(log, n, hold_last, xm, lane, base, bestg);
+        n = 0;
+    }
+    // Once per 32 flips: out of line, so that the step's code stays short (the
+    // instruction fetch of a one-warp step is part of its latency: N = 512 fp32, 64
+    // replicas 0.604 us per step inlined, 0.586 not).
+    static __device__ __noinline__ void settle_impl(FlipLog<E>* log, int n, bool hold_last, uint32_t xm, int lane,
+                                                    int base, uint32_t* bestg)
+    {
+        __syncwarp();
+        E e = log->E, b = log->best;
+        const int at = settle_log<A>(log->f, n, hold_last ? n - 1 : n, lane, e, b);
+        if (at >= 0) {                        // the state after flip `at`: the later ones undone
+            uint32_t x = xm;
+            for (int q = at + 1; q < n; ++q) {
+                const int k = log->f[q].k;
+                if (k / V == lane) x ^= 1u << (k % V);
+            }
+            const uint32_t wv = gather_word<V>(x, lane);
+            if (lane % P == 0) bestg[base >> 5] = wv;
+        }
+        __syncwarp();
+        if (lane == 0) {
+            log->E = e;
+            log->best = b;
+            log->flips += n;
+        }
+        __syncwarp();
+    }
+
+    // The best-state test of the current state (no flips pending) at the energy log->E.
+    __device__ __forceinline__ void test_current()
+    {
+        __syncwarp();
+        if (log->E < log->best) {             // uniform
+            const uint32_t wv = word();
+            if (lane % P == 0) bestg[base >> 5] = wv;
+            __syncwarp();
+            if (lane == 0) log->best = log->E;
+        }
+        __syncwarp();
     }
 
     __device__ __forceinline__ uint32_t word() const { return gather_word<V>(xm, lane); }
@@ -98,12 +199,6 @@ struct WarpReplica {
         if constexpr (SW) RowShared<Tw, V>::load(p, c);
         else if constexpr (COAL) RowCoal<Tw, V>::load(p, c);
         else Row<Tw, V>::load(p, c);
-    }
-
-    __device__ __forceinline__ void snapshot()
-    {
-        const uint32_t wv = word();
-        if (lane % P == 0) bestg[base >> 5] = wv;
     }
 
     template <class Keys>
@@ -234,38 +329,44 @@ struct WarpReplica {
     }
 
     // Work a step places in the latency of its warp collectives (choose_and_flip):
-    // begin() after the count reduction is issued, at<I>() after collective I is
-    // issued and before its result is used (I = 0..4: the prefix-sum shuffles;
-    // 5: the owner ballot; 6: the owner's position shuffle), rest_flip() while
-    // row k is in flight, rest_none() when nothing flips.
+    // at<0>() after the votes on the counts are issued, at<1>() after the owner's
+    // vote, at<2>() after the shuffles of the owner's words, at<3>() after the vote
+    // on the bit position; rest_flip() while row k is in flight, rest_none() when
+    // nothing flips.
     template <class F>
     struct RestOnly {      // everything under the row load (or at once)
         F& f;
-        __device__ __forceinline__ void begin() {}
         template <int I> __device__ __forceinline__ void at() {}
         __device__ __forceinline__ void rest_flip() { f(); }
         __device__ __forceinline__ void rest_none() { f(); }
     };
     template <class Keys>
-    struct DrawSlots {     // the next step's draws (PRE): rounds 3-5 in the prefix
-        WarpReplica& rp;   // sum, 6-7 in the choice, 8-9 and log2 under the row load
+    struct DrawSlots {     // the next step's draws (PRE)
+        WarpReplica& rp;
         const Keys& keys;
         uint32_t tt;
-        __device__ __forceinline__ void begin() { rp.draw_begin(tt); }
+        // Rounds done after slot 0 .. 3, measured per V: with all of them under the row
+        // load N = 512 takes 0.608 instead of 0.562 us per step, with all of them before
+        // it 0.581 (fp32, 64 replicas).
+        static constexpr int kR0 = 5, kR1 = 6, kR2 = 7, kR3 = V == 8 || V == 32 ? 7 : 8;
         template <int I>
         __device__ __forceinline__ void at()
         {
-            if constexpr (I <= 2) rp.template draw_round<3 + I>(keys);
-            else if constexpr (I == 5 || I == 6) rp.template draw_round<I + 1>(keys);
+            if constexpr (I == 0) {
+                rp.draw_begin(tt);
+                rp.template draw_rounds<3, kR0>(keys);
+            } else if constexpr (I == 1) rp.template draw_rounds<kR0, kR1>(keys);
+            else if constexpr (I == 2) rp.template draw_rounds<kR1, kR2>(keys);
+            else rp.template draw_rounds<kR2, kR3>(keys);
         }
         __device__ __forceinline__ void rest_flip()
         {
-            rp.template draw_rounds<8, 10>(keys);
+            rp.template draw_rounds<kR3, 10>(keys);
             rp.draw_end();
         }
         __device__ __forceinline__ void rest_none()
         {
-            rp.template draw_rounds<6, 10>(keys);
+            rp.template draw_rounds<kR0, 10>(keys);
             rp.draw_end();
         }
     };
@@ -275,17 +376,17 @@ struct WarpReplica {
     // step's collectives as DrawSlots places them).  Returns the flipped index
     // or -1.
     template <bool FULL, class Keys>
-    __device__ __forceinline__ int step(long long t, bool draw_next, float beta, float inc, const Keys& keys)
+    __device__ __forceinline__ int step(uint32_t t, bool draw_next, float inc, const Keys& keys)
     {
         if constexpr (PRE) {
             DrawSlots<Keys> s{*this, keys, (uint32_t)(t + 1)};
-            return decide_and_flip<FULL>(t, beta, inc, lg, keys, s);
+            return decide_and_flip<FULL>(t, inc, lg, keys, s);
         } else {
             auto f = [&] {
                 if (draw_next) draw((uint32_t)(t + 1), keys);
             };
             RestOnly<decltype(f)> s{f};
-            return decide_and_flip<FULL>(t, beta, inc, lg, keys, s);
+            return decide_and_flip<FULL>(t, inc, lg, keys, s);
         }
     }
 
@@ -294,94 +395,112 @@ struct WarpReplica {
     // (decide_log; the rare trials near the threshold by decide_exact).
     // `overlap` runs while row k is in flight.
     template <bool FULL, class Keys, class Overlap>
-    __device__ __forceinline__ int step_log(long long t, float beta, float inc, const float (&L)[V], const Keys& keys,
+    __device__ __forceinline__ int step_log(long long t, float inc, const float (&L)[V], const Keys& keys,
                                             Overlap&& overlap)
     {
         RestOnly<Overlap> s{overlap};
-        return decide_and_flip<FULL>(t, beta, inc, L, keys, s);
+        return decide_and_flip<FULL>(t, inc, L, keys, s);
     }
 
     template <bool FULL, class Keys, class Slots>
-    __device__ __forceinline__ int decide_and_flip(long long t, float beta, float inc, const float (&L)[V],
-                                                   const Keys& keys, Slots& slots)
+    __device__ __forceinline__ int decide_and_flip(uint32_t t, float inc, const float (&L)[V], const Keys& keys,
+                                                   Slots& slots)
     {
+        // here the draws' and the row's registers are free
+        if (n == 32) settle();
         const float Eoff = __fmul_rn(__uint2float_rn(m), inc);
         bool unsure;
         uint32_t accm = decide_log<A, V>(h, xm, Eoff, __fmul_rn(beta, kLog2e), L, unsure);
-        if (__any_sync(0xffffffffu, unsure))
-            accm = decide_exact<A, V>(h, xm, Eoff, beta, L, accm, base, (uint32_t)t, rep, keys);
-        return choose_and_flip<FULL>(t, accm, keys, slots);
-    }
-
-    // Inclusive prefix sum over the lanes, level I..4, with slots.at<I>() in the
-    // latency of each shuffle.
-    template <int I, class Slots>
-    __device__ __forceinline__ void scan_levels(int& incl, Slots& slots)
-    {
-        if constexpr (I < 5) {
-            const int n = __shfl_up_sync(0xffffffffu, incl, 1 << I);
-            slots.template at<I>();
-            if (lane >= (1 << I)) incl += n;
-            scan_levels<I + 1>(incl, slots);
-        }
-    }
-
-    // (c) of a step with acceptance mask accm: the uniform choice among the
-    // accepted trials, the best-state test left by the previous step (under the
-    // row load, or first at V = 4), the flip and the field update, with `slots`
-    // placed as described above.  Returns the flipped index or -1.
-    template <bool FULL, class Keys, class Slots>
-    __device__ __forceinline__ int choose_and_flip(long long t, uint32_t accm, const Keys& keys, Slots& slots)
-    {
+        const bool any_unsure = __any_sync(0xffffffffu, unsure);
         if constexpr (!FULL) accm &= valid;
-        if constexpr (!kTestUnderRow) flush_best();
+        int excl, total;
+        count_below(accm, excl, total);
+        slots.template at<0>();
+        if (any_unsure) {   // rare: the exact test, and the counts again
+            accm = decide_exact<A, V>(h, xm, Eoff, beta, L, accm, base, (uint32_t)t, rep, keys);
+            if constexpr (!FULL) accm &= valid;
+            count_below(accm, excl, total);
+        }
+        return choose_and_flip<FULL>(t, accm, excl, total, keys, slots);
+    }
 
+    // Accepted trials on the lanes below this one, and on all lanes: the bits of the
+    // lanes' counts as votes, which are independent of one another (one latency of
+    // about 20 cycles, then the population counts), beside the warp reduction of the
+    // total; a five-shuffle prefix sum is a chain of five 32-cycle latencies.  (The
+    // total from the votes as well: 1.275 against 1.253 us per step at N = 1024 with
+    // 1024 replicas, the population counts share a unit with the draws' log2.)
+    __device__ __forceinline__ void count_below(uint32_t accm, int& excl, int& total) const
+    {
+        constexpr int kBits = V == 4 ? 3 : V == 8 ? 4 : V == 16 ? 5 : 6;   // of a count 0 .. V
+        const uint32_t below = (1u << lane) - 1u;
         const int cnt = __popc(accm);
-        const int total = (int)__reduce_add_sync(0xffffffffu, (unsigned)cnt);
-        slots.begin();
-        int incl = cnt;
-        scan_levels<0>(incl, slots);
+        total = (int)__reduce_add_sync(0xffffffffu, (unsigned)cnt);
+        excl = 0;
+#pragma unroll
+        for (int b = 0; b < kBits; ++b) excl += __popc(__ballot_sync(0xffffffffu, (cnt >> b) & 1) & below) << b;
+    }
+
+    // (c) of a step with acceptance mask accm (excl accepted trials on lower lanes,
+    // total in all): the uniform choice among the accepted trials, the flip and the
+    // field update, with `slots` placed as described above.  Returns the flipped index
+    // or -1.
+    template <bool FULL, class Keys, class Slots>
+    __device__ __forceinline__ int choose_and_flip(uint32_t t, uint32_t accm, int excl, int total, const Keys& keys,
+                                                   Slots& slots)
+    {
         if (total == 0) {
             m += 1;
-            if constexpr (kTestUnderRow) flush_best();
             slots.rest_none();
+            next_inputs(t, keys);
             return -1;
         }
-        const long long blk = t >> 2;
-        if (blk != cr_blk) {
-            cr = philox4x32_10(0u, (uint32_t)(t & ~3ll), rep, 1u, keys);
-            cr_blk = blk;
+        const int j = (int)__umulhi(cw, (uint32_t)total);
+        // inclusive counts ascend, so the lanes with at most j accepted trials up to
+        // and including their own are those before the owner
+        const uint32_t before = __ballot_sync(0xffffffffu, excl + __popc(accm) <= j);
+        slots.template at<1>();
+        const int own = __popc(before);
+        uint32_t acc_o, x_o;
+        int r;
+        if constexpr (V <= 8) {
+            const uint32_t w = __shfl_sync(0xffffffffu, accm | xm << 8 | (uint32_t)excl << 16, own);
+            acc_o = w & 0xFFu;
+            x_o = (w >> 8) & 0xFFu;
+            r = j - (int)(w >> 16);
+        } else {
+            acc_o = __shfl_sync(0xffffffffu, accm, own);
+            x_o = __shfl_sync(0xffffffffu, xm, own);
+            r = j - __shfl_sync(0xffffffffu, excl, own);
         }
-        const int j = (int)__umulhi(pick(cr, (int)(t & 3)), (uint32_t)total);
-        const int excl = incl - cnt;
-        const int own = __ffs(__ballot_sync(0xffffffffu, j >= excl && j < incl)) - 1;
-        const int pos = nth_set_bit(accm, j - excl);
-        slots.template at<5>();
-        const int vk = __shfl_sync(0xffffffffu, pos, own);
-        slots.template at<6>();
-        const uint32_t xold = (__shfl_sync(0xffffffffu, xm, own) >> vk) & 1u;
+        slots.template at<2>();
+        // the position of the r-th (0-based) set bit of the owner's mask: lane v counts
+        // the set bits up to v, and the positions with at most r of them precede it
+        const uint32_t upto = 0xffffffffu >> (31 - lane);
+        const uint32_t pre = __ballot_sync(0xffffffffu, __popc(acc_o & upto) <= r);
+        slots.template at<3>();
+        const int vk = __popc(pre);
+        const uint32_t xold = (x_o >> vk) & 1u;
         const H gk = select_slot<H, V>(h, vk);
-        const H dEk = __shfl_sync(0xffffffffu, A::signed_field(gk, xold), own);
         const int k = own * V + vk;
         Tw cv[V];
         if (FULL || base < N) load_row(W + (size_t)k * ldw + rowoff, cv);
-        if constexpr (kTestUnderRow) flush_best();   // x is still the state after the previous step
+        if (lane == own) log->f[n] = FlipEntry{A::log_bits(A::signed_field(gk, xold)), k};
+        ++n;
         slots.rest_flip();
+        next_inputs(t, keys);
         if (FULL || base < N) {
             const typename A::Sign sg = A::sign(xold);
 #pragma unroll
             for (int v = 0; v < V; ++v) h[v] = A::apply_signed(h[v], cv[v], sg);
         }
         if (lane == own) xm ^= 1u << vk;
-        ++flips;
         m = 0;
-        Ecur = A::book(Ecur, dEk);
-        chk = true;
         return k;
     }
 
     // Exact fixed-point recompute of the fp32 fields and of the tracked
-    // energy (same definition as da_fields.cu): g_i = fl32(2^-S (round(d_i 2^S)
+    // energy (no flips pending; same definition as da_fields.cu): g_i = fl32(2^-S (round(d_i 2^S)
     // + sum_{x_j = 1} round(W_ij 2^S))), E = fl64(2^-(S+1) sum_{x_i = 1}
     // (round(d_i 2^S) + sum_i)).
     // shift: every coupling and linear term reaches the grid by a left shift
@@ -448,8 +567,8 @@ struct WarpReplica {
         }
         const long long top = (long long)((unsigned long long)hi << 32 | (lo >> 32));
         const double v = __fma_rn((double)top, 4294967296.0, (double)(uint32_t)(lo & 0xFFFFFFFFull));
-        Ecur = ldexp(v, -(S + 1));
-        chk = true;
+        if (lane == 0) log->E = ldexp(v, -(S + 1));
+        __syncwarp();
     }
 };
 

@@ -330,44 +330,40 @@ __global__ void __launch_bounds__(32 * G * OccupancyGV<G, V>::rpb, OccupancyGV<G
     }
 }
 
-// G = 1: one warp per replica, the body of WarpReplica.  PT: the launch anneals
-// replicas at fixed per-replica temperatures (p.betas), where the best-state test
-// stays before the count.  The fp32 forms at V >= 8 read their rows from p.Wc
+// G = 1: one warp per replica, the body of WarpReplica.  The fp32 forms at V >= 8 read their rows from p.Wc
 // (the warp row order, pitch 32 V).
-template <typename Tw, int V, bool FULL, bool TRACE, bool PT = false>
+template <typename Tw, int V, bool FULL, bool TRACE>
 __global__ void __launch_bounds__(32 * Occupancy<1>::rpb, Occupancy<1>::min_blocks)
     step_kernel_g1(const __grid_constant__ StepParams p)
 {
     constexpr bool kCoal = sizeof(Tw) == 4 && V >= 8;   // float and f32e
-    using R_ = WarpReplica<Tw, V, false, true, !PT && V >= 8, kCoal>;
+    using R_ = WarpReplica<Tw, V, false, true, kCoal>;
     using H = typename R_::H;
+    __shared__ FlipLog<typename R_::E> logs[Occupancy<1>::rpb];
     if (launch_stopped(p)) return;
     const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (r >= p.R) return;
     R_ rp;
     rp.init(static_cast<const Tw*>(kCoal ? p.Wc : p.W), p.N, kCoal ? 32 * V : p.ldw, p.rep_base + (uint32_t)r,
-            p.bestx + (size_t)r * p.nw);
+            p.bestx + (size_t)r * p.nw, &logs[threadIdx.x >> 5]);
     H* hg = static_cast<H*>(p.h) + (size_t)r * p.npad + rp.base;
     uint32_t* xg = p.x + (size_t)r * p.nw;
 #pragma unroll
     for (int v = 0; v < V; ++v) rp.h[v] = hg[v];
     rp.xm = (xg[rp.base >> 5] >> (rp.base & 31)) & R_::VMASK;
     ReplicaScalars sc = p.sc[r];
-    rp.Ecur = Arith<Tw>::load_e(sc.E);
-    rp.Ebest = Arith<Tw>::load_e(sc.best);
-    rp.flips = sc.flips;
     rp.m = sc.m;
-    rp.chk = sc.check != 0;
     const PhiloxKeys& keys = *reinterpret_cast<const PhiloxKeys*>(&p.round_key[0][0]);
     const bool per_rep = p.betas != nullptr;
-    const float beta_rep = per_rep ? p.betas[p.temp_of[r]] : 0.f;
+    rp.begin(p.t0, p.t1, per_rep ? nullptr : p.beta, per_rep ? p.betas[p.temp_of[r]] : 0.f, Arith<Tw>::load_e(sc.E),
+             Arith<Tw>::load_e(sc.best), sc.flips, keys);
+    bool held = sc.check != 0;       // the best-state test of the last step is still to be made
+    if (held && p.t0 < p.t1) rp.test_current();
     rp.prep_draws(keys);
     if (p.t0 < p.t1) rp.draw_pre((uint32_t)p.t0, keys);
-    float beta_next = (!per_rep && p.t0 < p.t1) ? p.beta[p.t0] : beta_rep;
-    for (long long t = p.t0; t < p.t1; ++t) {
-        const float beta = beta_next;
-        if (!per_rep && t + 1 < p.t1) beta_next = p.beta[t + 1];
-        const int k = rp.template step<FULL>(t, t + 1 < p.t1, beta, p.inc, keys);
+    for (uint32_t t = (uint32_t)p.t0; t < (uint32_t)p.t1; ++t) {
+        const int k = rp.template step<FULL>(t, t + 1 < p.t1, p.inc, keys);
+        held = k >= 0;
         if constexpr (TRACE) {
             if (rp.lane == 0) p.trace[(size_t)r * p.trace_T + t] = k;
         }
@@ -376,12 +372,13 @@ __global__ void __launch_bounds__(32 * Occupancy<1>::rpb, Occupancy<1>::min_bloc
     for (int v = 0; v < V; ++v) hg[v] = rp.h[v];
     const uint32_t word = rp.word();
     if (rp.lane % R_::P == 0) xg[rp.base >> 5] = word;
+    if (rp.n > 0) rp.settle(held);
     if (rp.lane == 0) {
-        sc.E = Arith<Tw>::store_e(rp.Ecur);
-        sc.best = Arith<Tw>::store_e(rp.Ebest);
-        sc.flips = rp.flips;
+        sc.E = Arith<Tw>::store_e(rp.log->E);
+        sc.best = Arith<Tw>::store_e(rp.log->best);
+        sc.flips = rp.log->flips;
         sc.m = rp.m;
-        sc.check = rp.chk ? 1u : 0u;
+        sc.check = held ? 1u : 0u;
         p.sc[r] = sc;
     }
 }
@@ -408,6 +405,7 @@ __global__ void __launch_bounds__(64, 7) step_kernel_ws(const __grid_constant__ 
     __shared__ float4 ring[kWsRing][NQ][32];
     __shared__ uint64_t full[kWsRing], empty[kWsRing];
     __shared__ int failed;
+    __shared__ FlipLog<typename R_::E> log;
     const int r = blockIdx.x;
     if (r >= p.R) return;   // whole block
     const int warp = threadIdx.x >> 5;
@@ -447,20 +445,19 @@ __global__ void __launch_bounds__(64, 7) step_kernel_ws(const __grid_constant__ 
     }
 
     R_ rp;
-    rp.init(static_cast<const Tw*>(p.W), p.N, p.ldw, rep, p.bestx + (size_t)r * p.nw);
+    rp.init(static_cast<const Tw*>(p.W), p.N, p.ldw, rep, p.bestx + (size_t)r * p.nw, &log);
     H* hg = static_cast<H*>(p.h) + (size_t)r * p.npad + rp.base;
     uint32_t* xg = p.x + (size_t)r * p.nw;
 #pragma unroll
     for (int v = 0; v < V; ++v) rp.h[v] = hg[v];
     rp.xm = (xg[rp.base >> 5] >> (rp.base & 31)) & R_::VMASK;
     ReplicaScalars sc = p.sc[r];
-    rp.Ecur = Arith<Tw>::load_e(sc.E);
-    rp.Ebest = Arith<Tw>::load_e(sc.best);
-    rp.flips = sc.flips;
     rp.m = sc.m;
-    rp.chk = sc.check != 0;
     const bool per_rep = p.betas != nullptr;
-    const float beta_rep = per_rep ? p.betas[p.temp_of[r]] : 0.f;
+    rp.begin(p.t0, p.t1, per_rep ? nullptr : p.beta, per_rep ? p.betas[p.temp_of[r]] : 0.f, Arith<Tw>::load_e(sc.E),
+             Arith<Tw>::load_e(sc.best), sc.flips, keys);
+    bool held = sc.check != 0;       // the best-state test of the last step is still to be made
+    if (held && p.t0 < p.t1) rp.test_current();
 
     float L[V];
     bool ok = true;
@@ -478,14 +475,12 @@ __global__ void __launch_bounds__(64, 7) step_kernel_ws(const __grid_constant__ 
         tc::mbar_arrive(&empty[b]);
     };
     if (n > 0) fetch(0);
-    float beta_next = (!per_rep && n > 0) ? p.beta[p.t0] : beta_rep;
     for (long long i = 0; i < n && __all_sync(0xffffffffu, ok); ++i) {
         const long long t = p.t0 + i;
-        const float beta = beta_next;
-        if (!per_rep && i + 1 < n) beta_next = p.beta[t + 1];
-        const int k = rp.template step_log<FULL>(t, beta, p.inc, L, keys, [&] {
+        const int k = rp.template step_log<FULL>(t, p.inc, L, keys, [&] {
             if (i + 1 < n) fetch(i + 1);
         });
+        held = k >= 0;
         if constexpr (TRACE) {
             if (lane == 0) p.trace[(size_t)r * p.trace_T + t] = k;
         }
@@ -495,12 +490,13 @@ __global__ void __launch_bounds__(64, 7) step_kernel_ws(const __grid_constant__ 
     for (int v = 0; v < V; ++v) hg[v] = rp.h[v];
     const uint32_t word = rp.word();
     if (lane % R_::P == 0) xg[rp.base >> 5] = word;
+    if (rp.n > 0) rp.settle(held);
     if (lane == 0) {
-        sc.E = Arith<Tw>::store_e(rp.Ecur);
-        sc.best = Arith<Tw>::store_e(rp.Ebest);
-        sc.flips = rp.flips;
+        sc.E = Arith<Tw>::store_e(rp.log->E);
+        sc.best = Arith<Tw>::store_e(rp.log->best);
+        sc.flips = rp.log->flips;
         sc.m = rp.m;
-        sc.check = rp.chk ? 1u : 0u;
+        sc.check = held ? 1u : 0u;
         p.sc[r] = sc;
     }
 }
@@ -533,15 +529,12 @@ cudaError_t launch_vg(const StepShape& s, const StepParams& p, bool trace, cudaS
             }
             return cudaGetLastError();
         }
-        const bool pt = p.betas != nullptr;
         if (blocks > 0 && sizeof(Tw) == 4 && V >= 8 && p.Wc == nullptr) return cudaErrorInvalidValue;
         if (full) {
             if (trace) launch_shared<step_kernel_g1<Tw, V, true, true>>(blocks, threads, 0, st, p);
-            else if (pt) launch_shared<step_kernel_g1<Tw, V, true, false, true>>(blocks, threads, 0, st, p);
             else launch_shared<step_kernel_g1<Tw, V, true, false>>(blocks, threads, 0, st, p);
         } else {
             if (trace) launch_shared<step_kernel_g1<Tw, V, false, true>>(blocks, threads, 0, st, p);
-            else if (pt) launch_shared<step_kernel_g1<Tw, V, false, false, true>>(blocks, threads, 0, st, p);
             else launch_shared<step_kernel_g1<Tw, V, false, false>>(blocks, threads, 0, st, p);
         }
         return cudaGetLastError();

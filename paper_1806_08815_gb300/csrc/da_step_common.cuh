@@ -12,8 +12,7 @@ template <> struct Arith<int8_t> {
     using H = int32_t;    // effective fields
     using E = long long;  // tracked energy
     static __device__ __forceinline__ H signed_field(H g, uint32_t x) { return x ? -g : g; }
-    static __device__ __forceinline__ float delta(H dE, float Eoff) { return __fsub_rn(__int2float_rn(dE), Eoff); }
-    static __device__ __forceinline__ float delta0(H dE) { return __int2float_rn(dE); }   // delta at E_off = +0
+    static __device__ __forceinline__ float to_float(H g) { return __int2float_rn(g); }
     static __device__ __forceinline__ H apply(H h, int8_t w, bool minus) { return minus ? h - (H)w : h + (H)w; }
     using Sign = int32_t;
     static __device__ __forceinline__ Sign sign(uint32_t xold) { return xold ? -1 : 1; }
@@ -21,14 +20,16 @@ template <> struct Arith<int8_t> {
     static __device__ __forceinline__ E load_e(long long b) { return b; }
     static __device__ __forceinline__ long long store_e(E e) { return e; }
     static __device__ __forceinline__ E book(E e, H dE) { return e + (E)dE; }
+    static constexpr bool kReal = false;
+    static __device__ __forceinline__ uint32_t log_bits(H dE) { return (uint32_t)dE; }
+    static __device__ __forceinline__ long long log_int(uint32_t b) { return (long long)(int)b; }
 };
 // 16-bit integer couplings (the DA's fixed-point precision): as int8, wider W.
 template <> struct Arith<int16_t> {
     using H = int32_t;
     using E = long long;
     static __device__ __forceinline__ H signed_field(H g, uint32_t x) { return x ? -g : g; }
-    static __device__ __forceinline__ float delta(H dE, float Eoff) { return __fsub_rn(__int2float_rn(dE), Eoff); }
-    static __device__ __forceinline__ float delta0(H dE) { return __int2float_rn(dE); }
+    static __device__ __forceinline__ float to_float(H g) { return __int2float_rn(g); }
     static __device__ __forceinline__ H apply(H h, int16_t w, bool minus) { return minus ? h - (H)w : h + (H)w; }
     using Sign = int32_t;
     static __device__ __forceinline__ Sign sign(uint32_t xold) { return xold ? -1 : 1; }
@@ -36,6 +37,9 @@ template <> struct Arith<int16_t> {
     static __device__ __forceinline__ E load_e(long long b) { return b; }
     static __device__ __forceinline__ long long store_e(E e) { return e; }
     static __device__ __forceinline__ E book(E e, H dE) { return e + (E)dE; }
+    static constexpr bool kReal = false;
+    static __device__ __forceinline__ uint32_t log_bits(H dE) { return (uint32_t)dE; }
+    static __device__ __forceinline__ long long log_int(uint32_t b) { return (long long)(int)b; }
 };
 template <> struct Arith<float> {
     using H = float;
@@ -44,8 +48,7 @@ template <> struct Arith<float> {
     {
         return __int_as_float(__float_as_int(g) ^ (int)(x << 31));
     }
-    static __device__ __forceinline__ float delta(H dE, float Eoff) { return __fsub_rn(dE, Eoff); }
-    static __device__ __forceinline__ float delta0(H dE) { return dE; }   // dE - (+0) = dE, also for dE = -0
+    static __device__ __forceinline__ float to_float(H g) { return g; }
     static __device__ __forceinline__ H apply(H h, float w, bool minus) { return minus ? __fsub_rn(h, w) : __fadd_rn(h, w); }
     using Sign = float;
     static __device__ __forceinline__ Sign sign(uint32_t xold) { return xold ? -1.0f : 1.0f; }
@@ -55,6 +58,8 @@ template <> struct Arith<float> {
     static __device__ __forceinline__ E load_e(long long b) { return __longlong_as_double(b); }
     static __device__ __forceinline__ long long store_e(E e) { return __double_as_longlong(e); }
     static __device__ __forceinline__ E book(E e, H dE) { return __dadd_rn(e, (double)dE); }
+    static constexpr bool kReal = true;
+    static __device__ __forceinline__ uint32_t log_bits(H dE) { return __float_as_uint(dE); }
 };
 
 // Integer couplings of a DA_INT8 instance stored as fp32 (exact: |W| <= 128 and
@@ -68,15 +73,161 @@ template <> struct Arith<f32e> {
     using H = float;
     using E = long long;
     static __device__ __forceinline__ H signed_field(H g, uint32_t x) { return Arith<float>::signed_field(g, x); }
-    static __device__ __forceinline__ float delta(H dE, float Eoff) { return __fsub_rn(dE, Eoff); }
-    static __device__ __forceinline__ float delta0(H dE) { return dE; }
+    static __device__ __forceinline__ float to_float(H g) { return g; }
     using Sign = float;
     static __device__ __forceinline__ Sign sign(uint32_t xold) { return xold ? -1.0f : 1.0f; }
     static __device__ __forceinline__ H apply_signed(H h, f32e w, Sign s) { return __fmaf_rn(s, w.f, h); }
     static __device__ __forceinline__ E load_e(long long b) { return b; }
     static __device__ __forceinline__ long long store_e(E e) { return e; }
     static __device__ __forceinline__ E book(E e, H dE) { return e + (E)__float2int_rn(dE); }
+    static constexpr bool kReal = false;
+    static __device__ __forceinline__ uint32_t log_bits(H dE) { return __float_as_uint(dE); }
+    static __device__ __forceinline__ long long log_int(uint32_t b) { return (long long)__float2int_rn(__uint_as_float(b)); }
 };
+
+// Delta E_i as the acceptance test takes it: fl32((1 - 2 x) g).  Rounding is
+// symmetric, so the sign is applied to the rounded field (integer fields: one
+// conversion and one xor instead of a negation, a selection and a conversion).
+template <typename A>
+__device__ __forceinline__ float delta_of(typename A::H g, uint32_t x)
+{
+    return __int_as_float(__float_as_int(A::to_float(g)) ^ (int)(x << 31));
+}
+
+// ---- tracked energy and best state, 32 flips at a time ----------------------------
+// The tracked energy of a replica (the in-order sum of the flips' Delta E: fp64 sum of
+// fp32 values for real couplings, int64 for integer ones) and the best-state test
+// after every flip are needed by nothing inside a step.  A step only appends (Delta E,
+// k) to a log of 32 entries; settle_log() then forms all of the window's energies at
+// once, one flip per lane, and finds the first strictly lowest one; the state it
+// belongs to is the current state with the later flips undone.  Per flip this costs
+// one store, where the test after every flip cost an fp64 conversion, add, compare and
+// branch (64 + 64 + 110 cycles alone and one fp64 warp instruction per 19 cycles and
+// SM, measured) and, at a new best state, a store of the state under the step.
+struct FlipEntry {
+    uint32_t dE;   // bits of Delta E (fp32 or int32)
+    int k;         // flipped variable
+};
+template <typename EE> struct FlipLog {
+    FlipEntry f[32];
+    EE E, best;        // up to the last settled flip
+    long long flips;
+};
+
+__device__ __forceinline__ long long warp_min(long long v)   // over the warp
+{
+    const int hi = (int)(v >> 32);
+    const int mh = __reduce_min_sync(0xffffffffu, hi);
+    const uint32_t ml = __reduce_min_sync(0xffffffffu, hi == mh ? (uint32_t)v : 0xffffffffu);
+    return (long long)mh << 32 | ml;
+}
+
+// Inclusive prefix sums of v over the lanes, and the first lane below `tested` with the
+// lowest one (`low`).
+__device__ __forceinline__ int first_lowest(long long v, int lane, int tested, long long& low)
+{
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+    }
+    const long long w = lane < tested ? v : 0x7FFFFFFFFFFFFFFFll;
+    low = warp_min(w);
+    return __ffs(__ballot_sync(0xffffffffu, w == low)) - 1;
+}
+
+// Sums over the warp of values whose absolute values sum to at most 2^53.
+__device__ __forceinline__ long long warp_sum53(long long v)
+{
+    const uint32_t lo = __reduce_add_sync(0xffffffffu, (uint32_t)v & 0x3FFFFFFu);
+    const int hi = __reduce_add_sync(0xffffffffu, (int)(v >> 26));
+    return ((long long)hi << 26) + (long long)lo;
+}
+
+// The n <= 32 flips of a log added to E in order; the first `tested` resulting energies
+// are tested: returns the index of the flip after which the energy was first strictly
+// lowest, if that is below `best` (then best = that energy), or -1.
+template <typename A>
+__device__ __forceinline__ int settle_log(const FlipEntry* f, int n, int tested, int lane, typename A::E& E,
+                                          typename A::E& best)
+{
+    const uint32_t bits = lane < n ? f[lane].dE : 0u;
+    if constexpr (sizeof(typename A::E) == 8 && !A::kReal) {
+        const long long v = A::log_int(bits);            // |v| < 2^31 each
+        const long long neg = warp_sum53(min(v, 0ll));
+        int at = -1;
+        if (E + neg < best && tested > 0) {
+            long long low;
+            const int q = first_lowest(v, lane, tested, low);
+            if (E + low < best) {
+                best = E + low;
+                at = q;
+            }
+        }
+        E += warp_sum53(v);
+        return at;
+    } else {
+        // Where E and every value are multiples of a unit 2^(k-53) and no partial sum can
+        // exceed 2^k, each fp64 addition of the in-order sum is exact, and so are the
+        // sums of the values as integers; otherwise the additions are made one by one.
+        const uint32_t a = bits & 0x7FFFFFFFu;
+        const uint32_t amax = __reduce_max_sync(0xffffffffu, a);
+        const unsigned long long eb = (unsigned long long)__double_as_longlong(E);
+        const int xE = (int)(eb >> 52) & 0x7FF;
+        const bool zero = (eb << 1) == 0;
+        const int ed = (int)(amax >> 23) - 127;          // |Delta E| < 2^(ed + 1): they sum to less than 2^(ed + 6)
+        bool exact = ed <= 100 && ed >= -100 && (zero || (xE >= 600 && xE <= 1400));
+        if (exact) {                                      // uniform
+            const int eE = xE - 1023;                     // |E| = mE 2^(eE - 52)
+            const unsigned long long mE = (eb & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+            int unit;                                     // k - 53
+            if (zero) {
+                unit = ed + 6 - 53;
+            } else {
+                const int s = ed + 6 - (eE - 52);
+                const bool room = s <= 52 && mE + (1ull << max(s, 0)) <= (1ull << 53);
+                unit = (room ? eE + 1 : max(eE + 1, ed + 6) + 1) - 53;
+                const int drop = unit - (eE - 52);        // >= 0
+                exact = drop < 53 && (mE & ((1ull << drop) - 1)) == 0;
+            }
+            const uint32_t x = a >> 23;
+            const uint32_t mant = x ? (a & 0x7FFFFFu) | 0x800000u : a;
+            const int sh = (int)max(x, 1u) - 150 - unit;  // Delta E = +-mant 2^(sh + unit), below 2^53 units
+            long long v = 0;
+            if (mant) {
+                if (sh >= 0) v = (long long)mant << min(sh, 38);
+                else if (sh > -24 && (mant & ((1u << -sh) - 1u)) == 0) v = mant >> -sh;
+                else exact = false;
+            }
+            if (__all_sync(0xffffffffu, exact)) {
+                if ((int)bits < 0) v = -v;
+                const double scale = __longlong_as_double((long long)(unit + 1023) << 52);
+                const double low_bound = __fma_rn(__ll2double_rn(warp_sum53(min(v, 0ll))), scale, E);   // exact
+                int at = -1;
+                if (low_bound < best && tested > 0) {
+                    long long low;
+                    const int q = first_lowest(v, lane, tested, low);
+                    const double lowE = __fma_rn(__ll2double_rn(low), scale, E);
+                    if (lowE < best) {
+                        best = lowE;
+                        at = q;
+                    }
+                }
+                E = __fma_rn(__ll2double_rn(warp_sum53(v)), scale, E);
+                return at;
+            }
+        }
+        int at = -1;
+        for (int q = 0; q < n; ++q) {
+            E = __dadd_rn(E, (double)__uint_as_float(f[q].dE));
+            if (q < tested && E < best) {
+                best = E;
+                at = q;
+            }
+        }
+        return at;
+    }
+}
 
 __device__ __forceinline__ int warp_inclusive_scan(int v, int lane)
 {
@@ -100,10 +251,24 @@ __device__ __forceinline__ int nth_set_bit(uint32_t w, int r)
     return pos;
 }
 
-// h[vk] for a warp-uniform vk, as one switch instead of V selects.
+// h[vk] for a warp-uniform vk: a tree of selections up to V = 16 (the indirect branch of
+// a switch sits on the way to the row load: N = 256 0.538 -> 0.493 us per step, N = 512
+// 0.652 -> 0.603, fp32 with 64 replicas), a switch for V = 32, where 31 selections cost
+// more than the branch (1.274 against 1.330 us per step at N = 1024, 1024 replicas).
 template <typename H, int V>
 __device__ __forceinline__ H select_slot(const H (&h)[V], int vk)
 {
+    if constexpr (V <= 16) {
+        H a[V];
+#pragma unroll
+        for (int v = 0; v < V; ++v) a[v] = h[v];
+#pragma unroll
+        for (int w = V / 2; w >= 1; w /= 2) {
+#pragma unroll
+            for (int v = 0; v < w; ++v) a[v] = (vk & w) ? a[v + w] : a[v];
+        }
+        return a[0];
+    }
 #define DA_SLOT(n) \
     case n:        \
         if constexpr (V > n) return h[n]; else return h[0];
@@ -283,8 +448,9 @@ __device__ __forceinline__ uint32_t gather_word(uint32_t bits, int lane)
 // kLogBand in da_device.cuh): returns the mask of surely accepted trials and
 // sets `unsure` when any trial has |t| <= kLogBand and must take the exact
 // test (decide_exact).  With E_off = +0 (no offset, or no step without a flip
-// since the last one) the subtraction is left out: it would return delta
-// unchanged.
+// since the last one) the subtraction returns delta unchanged: at V = 32 a branch
+// leaves it out, below that V packed additions cost less than the branch (N = 64
+// 0.398 -> 0.377 us per step, N = 1024 with 1024 replicas 1.274 -> 1.286 without it).
 // The test is made on t' = s - (24 - kLogBand), s = fma(delta, c, L), instead of
 // t = s - 24: wherever |t| < 12, s lies in [12, 36] and both subtractions are
 // exact (Sterbenz), so t' = t + kLogBand and
@@ -311,16 +477,15 @@ __device__ __forceinline__ uint32_t decide_log(const typename A::H (&h)[V], uint
         acc = __funnelshift_l(b0, acc, 1);
         umin = min(umin, min(b0, b1));
     };
-    if (Eoff == 0.0f) {
+    if (V > 16 && Eoff == 0.0f) {
 #pragma unroll
         for (int v = V - 2; v >= 0; v -= 2)
-            pair(v, A::delta0(A::signed_field(h[v], (xm >> v) & 1u)),
-                 A::delta0(A::signed_field(h[v + 1], (xm >> (v + 1)) & 1u)));
+            pair(v, delta_of<A>(h[v], (xm >> v) & 1u), delta_of<A>(h[v + 1], (xm >> (v + 1)) & 1u));
     } else {
 #pragma unroll
         for (int v = V - 2; v >= 0; v -= 2)
-            pair(v, A::delta(A::signed_field(h[v], (xm >> v) & 1u), Eoff),
-                 A::delta(A::signed_field(h[v + 1], (xm >> (v + 1)) & 1u), Eoff));
+            pair(v, __fsub_rn(delta_of<A>(h[v], (xm >> v) & 1u), Eoff),
+                 __fsub_rn(delta_of<A>(h[v + 1], (xm >> (v + 1)) & 1u), Eoff));
     }
     unsure = umin <= kBandBits;
     return acc;
@@ -338,13 +503,13 @@ __device__ __forceinline__ uint32_t decide_exact(const typename A::H (&h)[V], ui
     uint32_t band = 0;
 #pragma unroll
     for (int v = 0; v < V; ++v) {
-        const float t = __fsub_rn(__fmaf_rn(A::delta(A::signed_field(h[v], (xm >> v) & 1u), Eoff), c, L[v]), 24.0f);
+        const float t = __fsub_rn(__fmaf_rn(__fsub_rn(delta_of<A>(h[v], (xm >> v) & 1u), Eoff), c, L[v]), 24.0f);
         band |= (uint32_t)(fabsf(t) <= kLogBand) << v;
     }
     while (band) {
         const int v = __ffs(band) - 1;
         band &= band - 1;
-        const float delta = A::delta(A::signed_field(select_slot<typename A::H, V>(h, v), (xm >> v) & 1u), Eoff);
+        const float delta = __fsub_rn(delta_of<A>(select_slot<typename A::H, V>(h, v), (xm >> v) & 1u), Eoff);
         const float ax = -__fmul_rn(beta, delta);
         const uint32_t wd = pick(philox4x32_10((uint32_t)((base + v) >> 2), step, rep, 0u, keys), v & 3);
         acc |= (uint32_t)(delta <= 0.0f || uniform01(wd) < exp_neg(ax)) << v;
