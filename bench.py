@@ -41,8 +41,8 @@ C3 = dict(N=1024, replicas=1024, steps=200_000, recompute_every=1024, beta0=0.1,
 # capture of the headline workload, valid while the kernel source has the recorded hash.
 # Warp instructions per replica-step of the step kernel (smsp__inst_executed.sum / (R x steps))
 # from the same capture: the issue-slot roofline of a kernel bound by instruction issue.
-STEP_INST_PER_REPLICA_STEP = 690.3
-STEP_TRAFFIC = {"source_sha256_16": "c35e749fb617e047", "bytes_per_launch": 8.6190e6}
+STEP_INST_PER_REPLICA_STEP = 690.4
+STEP_TRAFFIC = {"source_sha256_16": "c5796cf18bfb7361", "bytes_per_launch": 8.6198e6}
 
 
 def step_source_sha():

@@ -55,7 +55,7 @@ struct da_ctx {
     int device = 0;
     void* W = nullptr;
     void* Wf = nullptr;  // DA_INT8: the couplings as exact fp32, for the step kernel
-    void* Wc[6][4] = {};  // the step couplings in the warp row order, by (log2 V, log2 G) (step_uses_coal)
+    void* Wc[9] = {};  // the step couplings in the warp row order, by log2(npad / 32) (step_uses_coal)
     void* diag = nullptr;
     da::TcOperand tc;  // digit planes of W for the tensor-core recompute
     void* ws = nullptr;
@@ -81,32 +81,31 @@ bool is_int(const da_ctx* c) { return c->dtype != DA_FP32; }
 int step_wtype(const da_ctx* c) { return c->dtype == DA_INT8 ? da::kWInt8AsF32 : (int)c->dtype; }
 const void* step_W(const da_ctx* c) { return c->dtype == DA_INT8 ? c->Wf : c->W; }
 
-// Default launch shape: one warp per replica up to N = 1024 (V <= 32
-// variables per lane).  Beyond, the fewest warps per replica that cover N
-// with V <= 32 (G = 2, 4 or 8), doubled while the launch has fewer than 1024
-// warps (few replicas: more warps per replica keep the SMs busy); V the
-// smallest supported width for that G.  Register budgets keep every choice in
-// one wave for the replica counts that select it.
+// Default launch shape by N and the replicas R: few replicas are bound by the latency of
+// a step, which more warps per replica shorten (each warp decides fewer trials, at the
+// price of a barrier); many by the work of a step, which more warps only add to.  The
+// lines lie where the two meet, in warps per SM scheduler (152 SMs x 4).  Measured, us
+// per step, fp32 (G = 1 / 2 / 4 / 8 with the narrowest V):
+//   N = 256:  R = 32 .440 / .484, so one warp below 257 variables whatever R;
+//   N = 500:  R = 304 .622 / .609 / .574, R = 512 .625 / .702 / .811;
+//   N = 1024: R = 304 .917 / .738 / .693, R = 512 .926 / .951 / 1.094;
+//   N = 2048: R = 304 - / 1.294 / .978 / 1.195, R = 512 - / 1.633 / 1.666 / 2.283,
+//             R = 1024 - / 3.237 / 2.850 / 3.958;
+//   N = 4096: R = 152 - / - / 1.354 / 1.141, R = 256 - / - / 1.678 / 2.132.
 StepShape auto_shape(int N, int R)
 {
+    constexpr int kSMs = 152;
+    int G;
+    if (N <= 256) G = 1;
+    else if (N <= 1024) G = R <= 2 * kSMs ? 4 : 1;
+    else if (N <= 2048) G = 4;
+    else if (N <= 4096) G = R <= kSMs ? 8 : 4;
+    else G = 8;
     StepShape s;
-    if (N <= 1024) {
-        int V = 4;
-        while (32 * V < N) V *= 2;
-        s.V = V; s.G = 1; s.rpb = 4;
-        return s;
-    }
-    auto width = [N](int G) {
-        int V = G == 8 ? 8 : 4;
-        while (32 * V * G < N) V *= 2;
-        return V;
-    };
-    int G = 2;
-    while (32 * 32 * G < N) G *= 2;
-    while (G < 8 && (long long)R * G < 1024) G *= 2;
     s.G = G;
-    s.V = width(G);
-    s.rpb = G == 2 ? 2 : 1;
+    s.V = G == 8 ? 8 : 4;
+    while (32 * s.V * G < N) s.V *= 2;
+    s.rpb = G == 1 ? 4 : 1;
     return s;
 }
 
@@ -127,7 +126,7 @@ StepShape shape_for(const da_ctx* c, int R)
         auto f = g_shape_cache.find(std::make_tuple(c->device, step_wtype(c), c->N, R));
         if (f != g_shape_cache.end()) return f->second;
     }
-    StepShape s = auto_shape(c->N, R);
+    StepShape s = auto_shape(c->N, c->draw_warp ? 1 << 30 : R);   // the producer-warp form is a one-warp shape
     s.ws = s.G == 1 && c->draw_warp;
     return s;
 }
@@ -209,9 +208,9 @@ struct RunBuffers {
 
 int log2_of(int v) { return 31 - __builtin_clz((unsigned)v); }
 
-// The copy of the step couplings in the warp row order for shape s, built on the
-// context's stream (and waited for) the first time a launch of that shape needs it.
-void*& coal_slot(da_ctx* c, const StepShape& s) { return c->Wc[log2_of(s.V)][log2_of(s.G)]; }
+// The copy of the step couplings in the warp row order for the padded width of shape s,
+// built on the context's stream (and waited for) the first time a launch needs it.
+void*& coal_slot(da_ctx* c, const StepShape& s) { return c->Wc[log2_of(s.V * s.G)]; }
 
 da_status ensure_coal(da_ctx* c, const StepShape& s)
 {
@@ -222,7 +221,7 @@ da_status ensure_coal(da_ctx* c, const StepShape& s)
         cudaGetLastError();
         return fail(DA_ENOMEM, std::string("row-ordered couplings: ") + cudaGetErrorString(e));
     }
-    e = da::launch_coalesce_W(static_cast<const float*>(step_W(c)), c->N, c->ldw, s.V, s.G, static_cast<float*>(p),
+    e = da::launch_coalesce_W(static_cast<const float*>(step_W(c)), c->N, c->ldw, s.npad(), static_cast<float*>(p),
                               c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
@@ -237,7 +236,7 @@ StepParams base_params(const da_ctx* c, const RunBuffers& b)
 {
     StepParams p;
     p.W = step_W(c);
-    p.Wc = da::step_uses_coal(step_wtype(c), b.s) ? c->Wc[log2_of(b.s.V)][log2_of(b.s.G)] : nullptr;
+    p.Wc = da::step_uses_coal(step_wtype(c), b.s) ? c->Wc[log2_of(b.s.V * b.s.G)] : nullptr;
     p.diag = c->diag;
     p.N = c->N;
     p.ldw = c->ldw;
@@ -519,8 +518,8 @@ da_status da_create(const void* Q, int64_t N, da_dtype dtype, da_ctx** out)
         return bail(e == cudaErrorMemoryAllocation ? DA_ENOMEM : DA_ECUDA,
                     std::string("tensor-core operand: ") + cudaGetErrorString(e));
     }
-    // the row-ordered couplings of the default one-warp shape, so that an anneal in that
-    // shape waits for nothing
+    // the row-ordered couplings of the padded width up to N = 1024, so that an anneal
+    // in a default shape (any number of warps per replica) waits for nothing
     if (n <= 1024)
         if (da_status st = ensure_coal(c, auto_shape(n, 1024))) return bail(st, std::string(g_err));
     *out = c;
@@ -559,9 +558,8 @@ void da_destroy(da_ctx* c)
     if (c->stream) cudaStreamSynchronize(c->stream);
     if (c->W) da::dev_free(c->W);
     if (c->Wf) da::dev_free(c->Wf);
-    for (auto& row : c->Wc)
-        for (void* w : row)
-            if (w) da::dev_free(w);
+    for (void* w : c->Wc)
+        if (w) da::dev_free(w);
     if (c->diag) da::dev_free(c->diag);
     da::tc_operand_free(&c->tc);
     if (c->ws) da::dev_free(c->ws);

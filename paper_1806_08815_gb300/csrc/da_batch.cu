@@ -64,7 +64,7 @@ __device__ __forceinline__ void run_unit(const BatchItemDev& it, int r, const Tw
     constexpr int nw = V;   // state words per replica (the padded width 32V / 32)
     const int lane = threadIdx.x & 31;
     R_ rp;
-    rp.init(W, it.N, ldw, (uint32_t)r, it.xs + ((size_t)it.R + r) * nw, log);
+    rp.init(W, it.N, ldw, (uint32_t)r, it.xs + ((size_t)it.R + r) * nw, log->f, &log->head);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
         if constexpr (std::is_same<Tw, step_detail::f32e>::value)   // int32 diagonal, exact in fp32
@@ -109,9 +109,9 @@ __device__ __forceinline__ void run_unit(const BatchItemDev& it, int r, const Tw
     if (lane % R_::P == 0) it.xs[(size_t)r * nw + (rp.base >> 5)] = word;
     if (lane == 0) {
         ReplicaScalars s;
-        s.E = A::store_e(log->E);
-        s.best = A::store_e(log->best);
-        s.flips = log->flips;
+        s.E = A::store_e(log->head.E);
+        s.best = A::store_e(log->head.best);
+        s.flips = log->head.flips;
         s.m = rp.m;
         s.check = 0;
         it.sc[r] = s;

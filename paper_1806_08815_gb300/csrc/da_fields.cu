@@ -271,7 +271,7 @@ cudaError_t launch_zero(void* p, size_t bytes, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// One thread per entry m of the reordered rows (pitch 32 V G): in warp slice
+// One thread per entry m of the reordered rows (pitch P, V = min(32, P / 32)): in slice
 // s = m / 32 V, entry m' = 128 q + 4 l + e holds variable i = s 32 V + l V + 4 q + e
 // (see step_uses_coal in da_internal.h).
 __global__ void __launch_bounds__(256) coalesce_kernel(const float* __restrict__ W, int N, int ldw, int V, int P,
@@ -293,12 +293,12 @@ bool step_uses_coal(int wtype, const StepShape& s)
 
 size_t coal_W_bytes(int N, const StepShape& s) { return (size_t)N * s.npad() * sizeof(float); }
 
-cudaError_t launch_coalesce_W(const float* W, int N, int ldw, int V, int G, float* Wc, cudaStream_t st)
+cudaError_t launch_coalesce_W(const float* W, int N, int ldw, int npad, float* Wc, cudaStream_t st)
 {
-    const int P = 32 * V * G;
+    const int P = npad, V = std::min(32, npad / 32);
     const long long n = (long long)N * P;
     if (n == 0) return cudaSuccess;
-    if (V < 8 || V > 32 || (V & (V - 1)) || G < 1 || G > 8 || (G & (G - 1)) || P < N) return cudaErrorInvalidValue;
+    if (P < 256 || P > 8192 || (P & (P - 1)) || P < N) return cudaErrorInvalidValue;
     prefer_shared<coalesce_kernel>();
     coalesce_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(W, N, ldw, V, P, Wc);
     return cudaGetLastError();

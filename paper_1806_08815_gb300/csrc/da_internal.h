@@ -96,17 +96,19 @@ cudaError_t launch_step(int wtype, const StepShape& s, const StepParams& p, bool
 
 // The step kernel (no producer warp) of the fp32 coupling forms (fp32, and int8
 // held as exact fp32) at V >= 8 variables per lane reads its rows of W from a copy
-// in another order, "the warp row order": in the 32 V entries of warp w's slice of
-// a row, variable i = w 32 V + l V + v (lane l, slot v) sits at entry
-// w 32 V + 128 (v / 4) + 4 l + v % 4, so that float4 number q of lane l (entries
-// w 32 V + 128 q + 4 l .. + 3) holds the lane's slots 4 q .. 4 q + 3 and each
-// 16-byte load instruction of the warp reads 512 contiguous bytes (in the plain
-// order every lane's 16 bytes fall in a different 128-byte line).  Entries of
-// padding variables (i >= N) are 0.  The copy is [N][32 V G] floats (the shape's
-// padded width), 16-byte aligned (da_fields.cu).
+// in another order, "the warp row order": with V0 = min(32, npad / 32), a row is cut
+// into slices of 32 V0 entries, and in slice s variable i = s 32 V0 + l V0 + v
+// (l < 32, v < V0) sits at entry s 32 V0 + 128 (v / 4) + 4 l + v % 4.  A warp whose
+// lanes own V0 variables each reads one slice, float4 number q of lane l being
+// entries 128 q + 4 l .. + 3, so each of its 16-byte load instructions covers 512
+// contiguous bytes (in the plain order every lane's 16 bytes fall in a different
+// 128-byte line).  A warp with V < V0 variables per lane (more warps per replica)
+// reads the same copy: 128-byte pieces of whole lines.  Entries of padding variables
+// (i >= N) are 0.  The copy is [N][npad] floats (the shape's padded width, the same
+// for every shape of that width), 16-byte aligned (da_fields.cu).
 bool step_uses_coal(int wtype, const StepShape& s);
 size_t coal_W_bytes(int N, const StepShape& s);
-cudaError_t launch_coalesce_W(const float* W, int N, int ldw, int V, int G, float* Wc, cudaStream_t st);
+cudaError_t launch_coalesce_W(const float* W, int N, int ldw, int npad, float* Wc, cudaStream_t st);
 bool step_shape_supported(const StepShape& s);
 
 // Field recompute and energies (da_fields.cu).

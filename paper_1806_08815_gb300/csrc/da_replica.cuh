@@ -33,9 +33,9 @@ namespace step_detail {
 // PRE: the step-invariant part of each Philox block is computed once per launch
 // (prep_draws) and the draws of every step start from it (draw_pre); four more
 // words per block live in registers, for kernels that have them to spare.
-// COAL: W points at the couplings in the warp row order (row pitch ldw = 32 V;
-// step_uses_coal in da_internal.h) and rows are read with RowCoal.
-template <typename Tw, int V, bool SW = false, bool PRE = false, bool COAL = false>
+// COAL: W points at the couplings in the warp row order (row pitch ldw, slices of 32 V0
+// entries; step_uses_coal in da_internal.h) and rows are read with RowCoal.
+template <typename Tw, int V, bool SW = false, bool PRE = false, bool COAL = false, int V0 = V>
 struct WarpReplica {
     using A = Arith<Tw>;
     using H = typename A::H;
@@ -52,10 +52,11 @@ struct WarpReplica {
     float bwin, bnext;   // the schedule of the steps [t & ~31, + 32) and of the 32 after, one per lane
     float beta;       // of the current step
     uint32_t xm, valid, m;
-    FlipLog<E>* log;  // this warp's log in shared memory
-    int n;            // flips in it
+    FlipEntry* log;   // the replica's flip log and this warp's energies, in shared memory
+    FlipHead<E>* head;
+    int n;            // flips in the log
     int lane, base, N, ldw;
-    int rowoff;       // this lane's first entry in a row of W: base, or 4 lane in the G = 1 order
+    int rowoff;       // this lane's first entry in a row of W
     uint32_t rep;
     const Tw* __restrict__ W;
     uint32_t* bestg;  // best-state words of this replica
@@ -65,11 +66,11 @@ struct WarpReplica {
     uint32_t ku0;
 
     __device__ __forceinline__ void init(const Tw* W_, int N_, int ldw_, uint32_t rep_, uint32_t* bestg_,
-                                         FlipLog<E>* log_)
+                                         FlipEntry* log_, FlipHead<E>* head_, int slice = 0)
     {
         lane = threadIdx.x & 31;
-        base = lane * V;
-        rowoff = COAL ? 4 * lane : base;
+        base = slice + lane * V;
+        rowoff = COAL ? base / (32 * V0) * (32 * V0) + base % V0 * 32 + base % (32 * V0) / V0 * 4 : base;
         N = N_;
         ldw = ldw_;
         rep = rep_;
@@ -77,6 +78,7 @@ struct WarpReplica {
         bestg = bestg_;
         valid = base >= N ? 0u : (N - base >= V ? VMASK : ((1u << (N - base)) - 1u));
         log = log_;
+        head = head_;
     }
 
     // Before the first step t0 of a launch over [t0, t1): the energies, and the step
@@ -88,11 +90,7 @@ struct WarpReplica {
     __device__ __forceinline__ void begin(long long t0, long long t1, const float* sched_, float beta0, E e0, E best0,
                                           long long flips0, const Keys& keys)
     {
-        if (lane == 0) {
-            log->E = e0;
-            log->best = best0;
-            log->flips = flips0;
-        }
+        if (lane == 0) *head = FlipHead<E>{e0, best0, flips0};
         __syncwarp();
         n = 0;
         sched = sched_;
@@ -148,45 +146,41 @@ struct WarpReplica {
     // recompute follows it, and the test comes after the recompute).
     __device__ __forceinline__ void settle(bool hold_last = false)
     {
-        settle_impl(log, n, hold_last, xm, lane, base, bestg);
+        settle_impl(head, log, n, hold_last, xm, lane, base, bestg);
         n = 0;
     }
     // Once per 32 flips: out of line, so that the step's code stays short (the
     // instruction fetch of a one-warp step is part of its latency: N = 512 fp32, 64
     // replicas 0.604 us per step inlined, 0.586 not).
-    static __device__ __noinline__ void settle_impl(FlipLog<E>* log, int n, bool hold_last, uint32_t xm, int lane,
-                                                    int base, uint32_t* bestg)
+    static __device__ __noinline__ void settle_impl(FlipHead<E>* head, const FlipEntry* log, int n, bool hold_last,
+                                                    uint32_t xm, int lane, int base, uint32_t* bestg)
     {
         __syncwarp();
-        E e = log->E, b = log->best;
-        const int at = settle_log<A>(log->f, n, hold_last ? n - 1 : n, lane, e, b);
+        E e = head->E, b = head->best;
+        const int at = settle_log<A>(log, n, hold_last ? n - 1 : n, lane, e, b);
         if (at >= 0) {                        // the state after flip `at`: the later ones undone
             uint32_t x = xm;
             for (int q = at + 1; q < n; ++q) {
-                const int k = log->f[q].k;
-                if (k / V == lane) x ^= 1u << (k % V);
+                const int k = log[q].k - base;
+                if (k >= 0 && k < V) x ^= 1u << k;
             }
             const uint32_t wv = gather_word<V>(x, lane);
             if (lane % P == 0) bestg[base >> 5] = wv;
         }
         __syncwarp();
-        if (lane == 0) {
-            log->E = e;
-            log->best = b;
-            log->flips += n;
-        }
+        if (lane == 0) *head = FlipHead<E>{e, b, head->flips + n};
         __syncwarp();
     }
 
-    // The best-state test of the current state (no flips pending) at the energy log->E.
+    // The best-state test of the current state (no flips pending) at the energy head->E.
     __device__ __forceinline__ void test_current()
     {
         __syncwarp();
-        if (log->E < log->best) {             // uniform
+        if (head->E < head->best) {             // uniform
             const uint32_t wv = word();
             if (lane % P == 0) bestg[base >> 5] = wv;
             __syncwarp();
-            if (lane == 0) log->best = log->E;
+            if (lane == 0) head->best = head->E;
         }
         __syncwarp();
     }
@@ -474,10 +468,7 @@ struct WarpReplica {
             r = j - __shfl_sync(0xffffffffu, excl, own);
         }
         slots.template at<2>();
-        // the position of the r-th (0-based) set bit of the owner's mask: lane v counts
-        // the set bits up to v, and the positions with at most r of them precede it
-        const uint32_t upto = 0xffffffffu >> (31 - lane);
-        const uint32_t pre = __ballot_sync(0xffffffffu, __popc(acc_o & upto) <= r);
+        const uint32_t pre = bits_before(acc_o, r, lane);
         slots.template at<3>();
         const int vk = __popc(pre);
         const uint32_t xold = (x_o >> vk) & 1u;
@@ -485,7 +476,7 @@ struct WarpReplica {
         const int k = own * V + vk;
         Tw cv[V];
         if (FULL || base < N) load_row(W + (size_t)k * ldw + rowoff, cv);
-        if (lane == own) log->f[n] = FlipEntry{A::log_bits(A::signed_field(gk, xold)), k};
+        if (lane == own) log[n] = FlipEntry{A::log_bits(A::signed_field(gk, xold)), k};
         ++n;
         slots.rest_flip();
         next_inputs(t, keys);
@@ -567,7 +558,7 @@ struct WarpReplica {
         }
         const long long top = (long long)((unsigned long long)hi << 32 | (lo >> 32));
         const double v = __fma_rn((double)top, 4294967296.0, (double)(uint32_t)(lo & 0xFFFFFFFFull));
-        if (lane == 0) log->E = ldexp(v, -(S + 1));
+        if (lane == 0) head->E = ldexp(v, -(S + 1));
         __syncwarp();
     }
 };

@@ -260,7 +260,7 @@ bool admit(da_server* s, Req& q, long long& launches)
     void* Wc = q.o_Wc ? q.dmem + q.o_Wc : nullptr;
     if (Wc) {
         if (!cu_ok(da::launch_coalesce_W(static_cast<const float*>(q.dtype == DA_INT8 ? Wf : W), q.N, q.inst.ldw,
-                                         q.shape.V, q.shape.G, static_cast<float*>(Wc), st),
+                                         q.shape.npad(), static_cast<float*>(Wc), st),
                    q, "row-ordered couplings"))
             return false;
         launches += 1;

@@ -103,12 +103,10 @@ extern "C" da_status da_anneal_static(const int8_t* W, const int32_t* diag, int6
         return fail(DA_EINVAL, "need replicas >= 1, 0 <= steps < 2^32 and a schedule");
     if (!(offset_inc >= 0.f) || !std::isfinite(offset_inc)) return fail(DA_EINVAL, "offset_inc must be finite and >= 0");
 
-    da::StepShape s;
-    s.V = (int)(pitch / 32);
-    s.G = 1;
-    s.rpb = 4;
     const int R = replicas;
     const int n = (int)N;
+    const da::StepShape s = da::default_shape(n, R);   // its padded width is the pitch for every R
+    if (s.npad() != pitch) return fail(DA_EINVAL, "internal: launch shape");
     const size_t tiles = ((size_t)s.npad() + 63) / 64;
     const size_t o_h = 0;
     const size_t o_x = o_h + align256((size_t)R * s.npad() * 4);

@@ -54,278 +54,197 @@ __device__ __forceinline__ bool launch_stopped(const StepParams& p)
     return s_stop != 0;
 }
 
+// What a lane publishes for the choice: its acceptance mask, its state bits and the
+// accepted trials on the lanes of its warp below it.
+template <int V> struct Published {   // V = 32
+    using T = uint4;
+    static __device__ __forceinline__ T pack(uint32_t acc, uint32_t x, int excl) { return make_uint4(acc, x, excl, 0); }
+    static __device__ __forceinline__ uint32_t acc(const T& e) { return e.x; }
+    static __device__ __forceinline__ uint32_t x(const T& e) { return e.y; }
+    static __device__ __forceinline__ int excl(const T& e) { return (int)e.z; }
+};
+template <> struct Published<16> {
+    using T = uint2;
+    static __device__ __forceinline__ T pack(uint32_t acc, uint32_t x, int excl) { return make_uint2(acc | x << 16, excl); }
+    static __device__ __forceinline__ uint32_t acc(const T& e) { return e.x & 0xFFFFu; }
+    static __device__ __forceinline__ uint32_t x(const T& e) { return e.x >> 16; }
+    static __device__ __forceinline__ int excl(const T& e) { return (int)e.y; }
+};
+template <> struct Published<8> {
+    using T = uint32_t;
+    static __device__ __forceinline__ T pack(uint32_t acc, uint32_t x, int excl) { return acc | x << 8 | (uint32_t)excl << 16; }
+    static __device__ __forceinline__ uint32_t acc(const T& e) { return e & 0xFFu; }
+    static __device__ __forceinline__ uint32_t x(const T& e) { return (e >> 8) & 0xFFu; }
+    static __device__ __forceinline__ int excl(const T& e) { return (int)(e >> 16); }
+};
+template <> struct Published<4> : Published<8> {};
+
+template <typename E, int V, int G> struct GroupShared {
+    typename Published<V>::T lanes[2][32 * G];   // by step parity
+    alignas(16) int total[2][(G + 3) / 4 * 4];   // accepted trials of each warp, by step parity
+    FlipEntry log[2][32];                        // by window parity
+    FlipHead<E> head[G];
+};
+
+// G > 1 warps per replica: warp w owns the slice [32 V w, 32 V (w + 1)) of the variables.
+// One barrier per step: every lane publishes its mask, state bits and in-warp prefix
+// count, every warp its total; after the barrier each warp finds the owner warp from the
+// G totals and reads only that warp's 32 entries.  Bound by the latency of the step's
+// chain (one to two warps per scheduler).  us per step, fp32 with 32 replicas, against
+// the form in which every warp scanned all 32 G masks and booked the energy in fp64:
+// N = 1024 (G = 4, V = 8) 1.015 -> 0.611, N = 2048 (G = 4, V = 16) 1.168 -> 0.755,
+// N = 4096 (G = 8, V = 16) 1.564 -> 1.109, N = 8192 (G = 8, V = 32) 2.712 -> 1.758
+// (there the rows of W come from HBM).  16 warps per replica are no faster: N = 2048
+// 0.978, N = 4096 1.314, N = 8192 1.955.
 template <typename Tw, int V, int G, bool FULL, bool TRACE>
 __global__ void __launch_bounds__(32 * G * OccupancyGV<G, V>::rpb, OccupancyGV<G, V>::min_blocks)
     step_kernel(const __grid_constant__ StepParams p)
 {
+    constexpr bool kCoal = sizeof(Tw) == 4 && V >= 8;   // fp32 forms: rows from p.Wc (step_uses_coal)
+    constexpr int kRegCap = 65536 / (32 * G * OccupancyGV<G, V>::rpb * OccupancyGV<G, V>::min_blocks);
+    constexpr bool kPre = kRegCap >= (V <= 8 ? 96 : V == 16 ? 128 : 255);
+    using R_ = WarpReplica<Tw, V, false, kPre, kCoal, (V * G < 32 ? V * G : 32)>;
     using A = Arith<Tw>;
-    using H = typename A::H;
-    using E = typename A::E;
-    static_assert(V % 4 == 0 && V <= 32, "V must be 4, 8, 16 or 32");
-    constexpr int NQ = V / 4;                       // Philox blocks per lane per step
-    constexpr uint32_t VMASK = V == 32 ? 0xffffffffu : ((1u << V) - 1u);
-    constexpr int P = 32 / V;                       // lanes per state word
-
-    extern __shared__ uint32_t smem[];
+    using H = typename R_::H;
+    using Pub = Published<V>;
+    __shared__ GroupShared<typename R_::E, V, G> shared[OccupancyGV<G, V>::rpb];
     if (launch_stopped(p)) return;
-    const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
     const int g = wib / G;                          // group (replica) within the block
     const int w = wib - g * G;                      // warp within the group
-    const int rpb = blockDim.x / (32 * G);
-    const int r = blockIdx.x * rpb + g;
+    const int r = blockIdx.x * (blockDim.x / (32 * G)) + g;
     if (r >= p.R) return;
+    auto& gs = shared[g];
 
-    uint32_t* gs = smem + g * (4 * 32 * G + 4);
-    uint32_t* accs = gs;                            // [2][32G] lane acceptance masks
-    uint32_t* xss = gs + 2 * 32 * G;                // [2][32G] lane state masks
-    H* pub = reinterpret_cast<H*>(gs + 4 * 32 * G); // [2] Delta E of the flipped variable
-
-    const Tw* __restrict__ Wm = static_cast<const Tw*>(p.W);
-    constexpr bool kCoal = sizeof(Tw) == 4 && V >= 8;   // fp32 forms: rows from p.Wc (step_uses_coal)
-    const int base = w * 32 * V + lane * V;         // first variable of this lane
-    H* hg = static_cast<H*>(p.h) + (size_t)r * p.npad + base;
+    R_ rp;
+    rp.init(static_cast<const Tw*>(kCoal ? p.Wc : p.W), p.N, kCoal ? p.npad : p.ldw, p.rep_base + (uint32_t)r,
+            p.bestx + (size_t)r * p.nw, gs.log[0], &gs.head[w], w * 32 * V);
+    const int lane = rp.lane;
+    H* hg = static_cast<H*>(p.h) + (size_t)r * p.npad + rp.base;
     uint32_t* xg = p.x + (size_t)r * p.nw;
-    uint32_t* bestg = p.bestx + (size_t)r * p.nw;
-    const int word_of_lane = base >> 5;
-
-    H h[V];
 #pragma unroll
-    for (int v = 0; v < V; ++v) h[v] = hg[v];
-    uint32_t xm = (xg[word_of_lane] >> (base & 31)) & VMASK;
-    uint32_t valid = VMASK;
-    if constexpr (!FULL) valid = base >= p.N ? 0u : (p.N - base >= V ? VMASK : ((1u << (p.N - base)) - 1u));
-
+    for (int v = 0; v < V; ++v) rp.h[v] = hg[v];
+    rp.xm = (xg[rp.base >> 5] >> (rp.base & 31)) & R_::VMASK;
     ReplicaScalars sc = p.sc[r];
-    E Ecur = A::load_e(sc.E), Ebest = A::load_e(sc.best);
-    long long flips = sc.flips;
-    uint32_t m = sc.m;
-    bool chk = sc.check != 0;       // best-state test pending from the previous launch
-    const uint32_t rep = p.rep_base + (uint32_t)r;
+    rp.m = sc.m;
     const PhiloxKeys& keys = *reinterpret_cast<const PhiloxKeys*>(&p.round_key[0][0]);
     const bool per_rep = p.betas != nullptr;
-    const float beta_rep = per_rep ? p.betas[p.temp_of[r]] : 0.f;
-    u32x4 cr = {0, 0, 0, 0};
-    long long cr_blk = -1;
-    bool pending = false;
-
-    auto snapshot = [&]() {
-        const uint32_t word = gather_word<V>(xm, lane);
-        if (lane % P == 0) bestg[word_of_lane] = word;
-    };
-    // Acceptance draws of one step as log2 U (lg2_draw): Philox block q covers
-    // variables base + 4q .. + 3.
-    // The step-invariant Philox words precomputed (as WarpReplica's PRE form) where the
-    // launch bounds leave at least 128 registers a thread and V <= 16; V = 32 and the
-    // 7-blocks-per-SM shapes have no room for them.
-    constexpr int kRegCap = 65536 / (32 * G * OccupancyGV<G, V>::rpb * OccupancyGV<G, V>::min_blocks);
-    constexpr bool kPre = V <= 16 && kRegCap >= 128;
-    constexpr int NP = kPre ? NQ : 1;
-    uint32_t kq1[NP], kq2[NP], kq3[NP], kq4[NP], ku0 = 0;
+    rp.begin(p.t0, p.t1, per_rep ? nullptr : p.beta, per_rep ? p.betas[p.temp_of[r]] : 0.f, A::load_e(sc.E),
+             A::load_e(sc.best), sc.flips, keys);
+    bool held = sc.check != 0;
+    if (held && p.t0 < p.t1) rp.test_current();
     if constexpr (kPre) {
-        const uint64_t pb0 = (uint64_t)kPhiloxMulB * rep;
-        ku0 = (uint32_t)(pb0 >> 32) ^ keys.a[0];
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            const uint64_t pa0 = (uint64_t)kPhiloxMulA * ((uint32_t)(base >> 2) + q);
-            const uint64_t pb1 = (uint64_t)kPhiloxMulB * ((uint32_t)(pa0 >> 32) ^ keys.b[0]);
-            const uint64_t pa2 = (uint64_t)kPhiloxMulA * ((uint32_t)(pb1 >> 32) ^ (uint32_t)pb0 ^ keys.a[1]);
-            kq1[q] = (uint32_t)pa0 ^ keys.b[1];
-            kq2[q] = (uint32_t)pb1 ^ keys.a[2];
-            kq3[q] = (uint32_t)(pa2 >> 32) ^ keys.b[2];
-            kq4[q] = (uint32_t)pa2 ^ keys.b[3];
-        }
+        rp.prep_draws(keys);
+        if (p.t0 < p.t1) rp.draw_pre((uint32_t)p.t0, keys);
+    } else {
+        if (p.t0 < p.t1) rp.draw((uint32_t)p.t0, keys);
     }
-    auto draw_step = [&](float (&lg)[V], uint32_t tt) {
-        if constexpr (kPre) {
-            const uint64_t P = (uint64_t)kPhiloxMulA * (ku0 ^ tt);
-            const uint32_t hP = (uint32_t)(P >> 32), lP = (uint32_t)P;
-            uint32_t c0[NQ], c1[NQ], c2[NQ], c3[NQ];
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) {
-                const uint64_t pb = (uint64_t)kPhiloxMulB * (hP ^ kq1[q]);
-                c0[q] = (uint32_t)(pb >> 32) ^ kq2[q];
-                c1[q] = (uint32_t)pb;
-                c2[q] = kq3[q] ^ lP;
-                c3[q] = kq4[q];
-            }
-#pragma unroll
-            for (int round = 3; round < 10; ++round) {
-#pragma unroll
-                for (int q = 0; q < NQ; ++q) {
-                    const uint64_t pa = (uint64_t)kPhiloxMulA * c0[q];
-                    const uint64_t pb = (uint64_t)kPhiloxMulB * c2[q];
-                    c0[q] = (uint32_t)(pb >> 32) ^ c1[q] ^ keys.a[round];
-                    // kq4 carried kb_3 into c3, so round 3 adds no key to it
-                    c2[q] = (uint32_t)(pa >> 32) ^ c3[q] ^ (round == 3 ? 0u : keys.b[round]);
-                    c1[q] = (uint32_t)pb;
-                    c3[q] = (uint32_t)pa;
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) {
-                lg[4 * q] = lg2_draw(c0[q]);
-                lg[4 * q + 1] = lg2_draw(c1[q]);
-                lg[4 * q + 2] = lg2_draw(c2[q]);
-                lg[4 * q + 3] = lg2_draw(c3[q]);
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) {
-                const u32x4 w4 = philox4x32_10((uint32_t)(base >> 2) + q, tt, rep, 0u, keys);
-                lg[4 * q] = lg2_draw(w4.x);
-                lg[4 * q + 1] = lg2_draw(w4.y);
-                lg[4 * q + 2] = lg2_draw(w4.z);
-                lg[4 * q + 3] = lg2_draw(w4.w);
-            }
-        }
-    };
-    float lg[V];
-    if (p.t0 < p.t1) draw_step(lg, (uint32_t)p.t0);
+    int window = 0;
 
-    float beta_next = (!per_rep && p.t0 < p.t1) ? p.beta[p.t0] : beta_rep;
-    for (long long t = p.t0; t < p.t1; ++t) {
-        const float beta = beta_next;
-        if (!per_rep && t + 1 < p.t1) beta_next = p.beta[t + 1];
-        const float Eoff = __fmul_rn(__uint2float_rn(m), p.inc);
-
-        // (a) + (b): every trial of this lane in the log domain (decide_log),
-        // the rare trials near the threshold by the exact test (decide_exact).
+    auto one_step = [&](uint32_t t, auto& slots) -> int {
+        const float Eoff = __fmul_rn(__uint2float_rn(rp.m), p.inc);
         bool unsure;
-        uint32_t accm = decide_log<A, V>(h, xm, Eoff, __fmul_rn(beta, kLog2e), lg, unsure);
-        if (__any_sync(0xffffffffu, unsure))
-            accm = decide_exact<A, V>(h, xm, Eoff, beta, lg, accm, base, (uint32_t)t, rep, keys);
-        if constexpr (!FULL) accm &= valid;
-
-        // (c) uniform choice among the accepted trials
-        int k = -1, own_lane = 0, own_warp = 0, vk = 0;
-        uint32_t xold = 0;
-        if constexpr (G == 1) {
-            const int cnt = __popc(accm);
-            const int incl = warp_inclusive_scan(cnt, lane);
-            const int total = __shfl_sync(0xffffffffu, incl, 31);
-            if (total == 0) {
-                m += 1;
-            } else {
-                const long long blk = t >> 2;
-                if (blk != cr_blk) {
-                    cr = philox4x32_10(0u, (uint32_t)(t & ~3ll), rep, 1u, keys);
-                    cr_blk = blk;
-                }
-                const int j = (int)__umulhi(pick(cr, (int)(t & 3)), (uint32_t)total);
-                const int excl = incl - cnt;
-                own_lane = __ffs(__ballot_sync(0xffffffffu, j >= excl && j < incl)) - 1;
-                const int pos = nth_set_bit(accm, j - excl);
-                vk = __shfl_sync(0xffffffffu, pos, own_lane);
-                xold = (__shfl_sync(0xffffffffu, xm, own_lane) >> vk) & 1u;
-                k = own_lane * V + vk;
-                m = 0;
+        uint32_t accm = decide_log<A, V>(rp.h, rp.xm, Eoff, __fmul_rn(rp.beta, kLog2e), rp.lg, unsure);
+        const bool any_unsure = __any_sync(0xffffffffu, unsure);
+        if constexpr (!FULL) accm &= rp.valid;
+        int excl, mine;
+        rp.count_below(accm, excl, mine);
+        slots.template at<0>();
+        if (any_unsure) {
+            accm = decide_exact<A, V>(rp.h, rp.xm, Eoff, rp.beta, rp.lg, accm, rp.base, t, rp.rep, keys);
+            if constexpr (!FULL) accm &= rp.valid;
+            rp.count_below(accm, excl, mine);
+        }
+        gs.lanes[t & 1][w * 32 + lane] = Pub::pack(accm, rp.xm, excl);
+        if (lane == 0) gs.total[t & 1][w] = mine;
+        group_barrier(1 + g, 32 * G);
+        // the flips up to the step before are in the log of every warp: settled here, by
+        // every warp for its own words
+        if (rp.n == 32) {
+            rp.settle();
+            window ^= 1;
+            rp.log = gs.log[window];
+        }
+        int before[G];                              // accepted trials on the warps below u
+        int total = 0;
+#pragma unroll
+        for (int u = 0; u < G; ++u) {
+            before[u] = total;
+            total += gs.total[t & 1][u];
+        }
+        if (total == 0) {
+            rp.m += 1;
+            slots.rest_none();
+            rp.next_inputs(t, keys);
+            return -1;
+        }
+        int j = (int)__umulhi(rp.cw, (uint32_t)total);
+        int ow = 0, skip = 0;
+#pragma unroll
+        for (int u = 1; u < G; ++u)
+            if (j >= before[u]) {
+                ow = u;
+                skip = before[u];
             }
+        j -= skip;
+        const typename Pub::T e = gs.lanes[t & 1][ow * 32 + lane];
+        const uint32_t lower = __ballot_sync(0xffffffffu, Pub::excl(e) + __popc(Pub::acc(e)) <= j);
+        slots.template at<1>();
+        const int ent = ow * 32 + __popc(lower);
+        const typename Pub::T o = gs.lanes[t & 1][ent];
+        slots.template at<2>();
+        const uint32_t pre = bits_before(Pub::acc(o), j - Pub::excl(o), lane);
+        slots.template at<3>();
+        const int vk = __popc(pre);
+        const uint32_t xold = (Pub::x(o) >> vk) & 1u;
+        const int k = ent * V + vk;
+        Tw cv[V];
+        if (FULL || rp.base < p.N) R_::load_row(rp.W + (size_t)k * rp.ldw + rp.rowoff, cv);
+        const bool own = w * 32 + lane == ent;
+        if (w == ow) {                              // warp-uniform
+            const H gk = select_slot<H, V>(rp.h, vk);
+            if (own) rp.log[rp.n] = FlipEntry{A::log_bits(A::signed_field(gk, xold)), k};
+        }
+        ++rp.n;
+        slots.rest_flip();
+        rp.next_inputs(t, keys);
+        if (FULL || rp.base < p.N) {
+            const typename A::Sign sg = A::sign(xold);
+#pragma unroll
+            for (int v = 0; v < V; ++v) rp.h[v] = A::apply_signed(rp.h[v], cv[v], sg);
+        }
+        if (own) rp.xm ^= 1u << vk;
+        rp.m = 0;
+        return k;
+    };
+    for (uint32_t t = (uint32_t)p.t0; t < (uint32_t)p.t1; ++t) {
+        int k;
+        if constexpr (kPre) {
+            typename R_::template DrawSlots<PhiloxKeys> s{rp, keys, t + 1};
+            k = one_step(t, s);
         } else {
-            uint32_t* ap = accs + (t & 1) * 32 * G;
-            uint32_t* xp = xss + (t & 1) * 32 * G;
-            ap[w * 32 + lane] = accm;
-            xp[w * 32 + lane] = xm;
-            group_barrier(1 + g, 32 * G);
-            if (pending) {          // book the flip of step t - 1
-                Ecur = A::book(Ecur, pub[(t - 1) & 1]);
-                chk = true;
-            }
-            if (chk) {              // and test it: x is still the state after step t - 1
-                chk = false;
-                if (Ecur < Ebest) { Ebest = Ecur; snapshot(); }
-            }
-            uint32_t e[G];
-            int cnt = 0;
-#pragma unroll
-            for (int u = 0; u < G; ++u) { e[u] = ap[lane * G + u]; cnt += __popc(e[u]); }
-            const int total = (int)__reduce_add_sync(0xffffffffu, (unsigned)cnt);
-            const int incl = warp_inclusive_scan(cnt, lane);
-            if (total == 0) {
-                m += 1;
-            } else {
-                const long long blk = t >> 2;
-                if (blk != cr_blk) {
-                    cr = philox4x32_10(0u, (uint32_t)(t & ~3ll), rep, 1u, keys);
-                    cr_blk = blk;
-                }
-                const int j = (int)__umulhi(pick(cr, (int)(t & 3)), (uint32_t)total);
-                const int excl = incl - cnt;
-                const int L = __ffs(__ballot_sync(0xffffffffu, j >= excl && j < incl)) - 1;
-                int ent = 0, pos = 0, rk = j - excl;
-#pragma unroll
-                for (int u = 0; u < G; ++u) {
-                    const int cu = __popc(e[u]);
-                    if (rk >= 0 && rk < cu) { ent = lane * G + u; pos = nth_set_bit(e[u], rk); }
-                    rk -= cu;
-                }
-                ent = __shfl_sync(0xffffffffu, ent, L);
-                vk = __shfl_sync(0xffffffffu, pos, L);
-                own_warp = ent >> 5;
-                own_lane = ent & 31;
-                xold = (xp[ent] >> vk) & 1u;
-                k = ent * V + vk;
-                m = 0;
-            }
+            auto f = [&] { rp.draw(t + 1, keys); };
+            typename R_::template RestOnly<decltype(f)> s{f};
+            k = one_step(t, s);
         }
-
-        if (k >= 0) {
-            // Delta E_k from the owner's registers
-            const H gk = select_slot<H, V>(h, vk);
-            H dEk = 0;
-            if constexpr (G == 1) {
-                dEk = __shfl_sync(0xffffffffu, A::signed_field(gk, xold), own_lane);
-            } else {
-                if (w == own_warp && lane == own_lane) pub[t & 1] = A::signed_field(gk, xold);
-            }
-            Tw cv[V];
-            if (FULL || base < p.N) {
-                if constexpr (kCoal)   // this warp's slice of the row in the warp row order (pitch npad)
-                    RowCoal<Tw, V>::load(static_cast<const Tw*>(p.Wc) + (size_t)k * p.npad + w * 32 * V + 4 * lane,
-                                         cv);
-                else
-                    Row<Tw, V>::load(Wm + (size_t)k * p.ldw + base, cv);
-            }
-            // the next step's draws do not depend on row k: compute them while
-            // its loads are in flight
-            if (t + 1 < p.t1) draw_step(lg, (uint32_t)(t + 1));
-            if (FULL || base < p.N) {
-                const typename A::Sign sg = A::sign(xold);
-#pragma unroll
-                for (int v = 0; v < V; ++v) h[v] = A::apply_signed(h[v], cv[v], sg);
-            }
-            if (w == own_warp && lane == own_lane) xm ^= 1u << vk;
-            ++flips;
-            if constexpr (G == 1) {
-                Ecur = A::book(Ecur, dEk);
-                if (Ecur < Ebest) { Ebest = Ecur; snapshot(); }
-            }
-        } else if (t + 1 < p.t1) {
-            draw_step(lg, (uint32_t)(t + 1));
-        }
-        if constexpr (G > 1) pending = k >= 0;
+        held = k >= 0;
         if constexpr (TRACE) {
             if (w == 0 && lane == 0) p.trace[(size_t)r * p.trace_T + t] = k;
         }
     }
-    if constexpr (G > 1) {
-        group_barrier(1 + g, 32 * G);
-        if (pending) {              // book the last flip; its test waits for any recompute
-            Ecur = A::book(Ecur, pub[(p.t1 - 1) & 1]);
-            chk = true;
-        }
-    }
+    group_barrier(1 + g, 32 * G);                   // the last flip is in the log
+    if (rp.n > 0) rp.settle(held);
 
 #pragma unroll
-    for (int v = 0; v < V; ++v) hg[v] = h[v];
-    const uint32_t word = gather_word<V>(xm, lane);
-    if (lane % P == 0) xg[word_of_lane] = word;
+    for (int v = 0; v < V; ++v) hg[v] = rp.h[v];
+    const uint32_t word = rp.word();
+    if (lane % R_::P == 0) xg[rp.base >> 5] = word;
     if (w == 0 && lane == 0) {
-        sc.E = A::store_e(Ecur);
-        sc.best = A::store_e(Ebest);
-        sc.flips = flips;
-        sc.m = m;
-        sc.check = chk ? 1u : 0u;
+        sc.E = A::store_e(rp.head->E);
+        sc.best = A::store_e(rp.head->best);
+        sc.flips = rp.head->flips;
+        sc.m = rp.m;
+        sc.check = held ? 1u : 0u;
         p.sc[r] = sc;
     }
 }
@@ -333,19 +252,20 @@ __global__ void __launch_bounds__(32 * G * OccupancyGV<G, V>::rpb, OccupancyGV<G
 // G = 1: one warp per replica, the body of WarpReplica.  The fp32 forms at V >= 8 read their rows from p.Wc
 // (the warp row order, pitch 32 V).
 template <typename Tw, int V, bool FULL, bool TRACE>
-__global__ void __launch_bounds__(32 * Occupancy<1>::rpb, Occupancy<1>::min_blocks)
+__global__ void __launch_bounds__(32 * OccupancyGV<1, V>::rpb, OccupancyGV<1, V>::min_blocks)
     step_kernel_g1(const __grid_constant__ StepParams p)
 {
     constexpr bool kCoal = sizeof(Tw) == 4 && V >= 8;   // float and f32e
     using R_ = WarpReplica<Tw, V, false, true, kCoal>;
     using H = typename R_::H;
-    __shared__ FlipLog<typename R_::E> logs[Occupancy<1>::rpb];
+    __shared__ FlipLog<typename R_::E> logs[OccupancyGV<1, V>::rpb];
     if (launch_stopped(p)) return;
     const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (r >= p.R) return;
     R_ rp;
     rp.init(static_cast<const Tw*>(kCoal ? p.Wc : p.W), p.N, kCoal ? 32 * V : p.ldw, p.rep_base + (uint32_t)r,
-            p.bestx + (size_t)r * p.nw, &logs[threadIdx.x >> 5]);
+            p.bestx + (size_t)r * p.nw, logs[threadIdx.x >> 5].f,
+            &logs[threadIdx.x >> 5].head);
     H* hg = static_cast<H*>(p.h) + (size_t)r * p.npad + rp.base;
     uint32_t* xg = p.x + (size_t)r * p.nw;
 #pragma unroll
@@ -374,9 +294,9 @@ __global__ void __launch_bounds__(32 * Occupancy<1>::rpb, Occupancy<1>::min_bloc
     if (rp.lane % R_::P == 0) xg[rp.base >> 5] = word;
     if (rp.n > 0) rp.settle(held);
     if (rp.lane == 0) {
-        sc.E = Arith<Tw>::store_e(rp.log->E);
-        sc.best = Arith<Tw>::store_e(rp.log->best);
-        sc.flips = rp.log->flips;
+        sc.E = Arith<Tw>::store_e(rp.head->E);
+        sc.best = Arith<Tw>::store_e(rp.head->best);
+        sc.flips = rp.head->flips;
         sc.m = rp.m;
         sc.check = held ? 1u : 0u;
         p.sc[r] = sc;
@@ -445,7 +365,7 @@ __global__ void __launch_bounds__(64, 7) step_kernel_ws(const __grid_constant__ 
     }
 
     R_ rp;
-    rp.init(static_cast<const Tw*>(p.W), p.N, p.ldw, rep, p.bestx + (size_t)r * p.nw, &log);
+    rp.init(static_cast<const Tw*>(p.W), p.N, p.ldw, rep, p.bestx + (size_t)r * p.nw, log.f, &log.head);
     H* hg = static_cast<H*>(p.h) + (size_t)r * p.npad + rp.base;
     uint32_t* xg = p.x + (size_t)r * p.nw;
 #pragma unroll
@@ -492,9 +412,9 @@ __global__ void __launch_bounds__(64, 7) step_kernel_ws(const __grid_constant__ 
     if (lane % R_::P == 0) xg[rp.base >> 5] = word;
     if (rp.n > 0) rp.settle(held);
     if (lane == 0) {
-        sc.E = Arith<Tw>::store_e(rp.log->E);
-        sc.best = Arith<Tw>::store_e(rp.log->best);
-        sc.flips = rp.log->flips;
+        sc.E = Arith<Tw>::store_e(rp.head->E);
+        sc.best = Arith<Tw>::store_e(rp.head->best);
+        sc.flips = rp.head->flips;
         sc.m = rp.m;
         sc.check = held ? 1u : 0u;
         p.sc[r] = sc;
@@ -515,7 +435,6 @@ cudaError_t launch_vg(const StepShape& s, const StepParams& p, bool trace, cudaS
 {
     const int threads = 32 * G * s.rpb;
     const int blocks = (p.R + s.rpb - 1) / s.rpb;
-    const size_t shm = G > 1 ? (size_t)s.rpb * (4 * 32 * G + 4) * sizeof(uint32_t) : 0;
     const bool full = p.N == 32 * V * G;
     if constexpr (G == 1) {
         if (s.ws) {
@@ -538,16 +457,17 @@ cudaError_t launch_vg(const StepShape& s, const StepParams& p, bool trace, cudaS
             else launch_shared<step_kernel_g1<Tw, V, false, false>>(blocks, threads, 0, st, p);
         }
         return cudaGetLastError();
-    }
-    if (blocks > 0 && sizeof(Tw) == 4 && V >= 8 && p.Wc == nullptr) return cudaErrorInvalidValue;
-    if (full) {
-        if (trace) launch_shared<step_kernel<Tw, V, G, true, true>>(blocks, threads, shm, st, p);
-        else launch_shared<step_kernel<Tw, V, G, true, false>>(blocks, threads, shm, st, p);
     } else {
-        if (trace) launch_shared<step_kernel<Tw, V, G, false, true>>(blocks, threads, shm, st, p);
-        else launch_shared<step_kernel<Tw, V, G, false, false>>(blocks, threads, shm, st, p);
+        if (blocks > 0 && sizeof(Tw) == 4 && V >= 8 && p.Wc == nullptr) return cudaErrorInvalidValue;
+        if (full) {
+            if (trace) launch_shared<step_kernel<Tw, V, G, true, true>>(blocks, threads, 0, st, p);
+            else launch_shared<step_kernel<Tw, V, G, true, false>>(blocks, threads, 0, st, p);
+        } else {
+            if (trace) launch_shared<step_kernel<Tw, V, G, false, true>>(blocks, threads, 0, st, p);
+            else launch_shared<step_kernel<Tw, V, G, false, false>>(blocks, threads, 0, st, p);
+        }
+        return cudaGetLastError();
     }
-    return cudaGetLastError();
 }
 
 template <typename Tw>

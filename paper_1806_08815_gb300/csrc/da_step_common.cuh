@@ -108,10 +108,13 @@ struct FlipEntry {
     uint32_t dE;   // bits of Delta E (fp32 or int32)
     int k;         // flipped variable
 };
-template <typename EE> struct FlipLog {
-    FlipEntry f[32];
+template <typename EE> struct FlipHead {   // one per warp
     EE E, best;        // up to the last settled flip
     long long flips;
+};
+template <typename EE> struct FlipLog {
+    FlipEntry f[32];
+    FlipHead<EE> head;
 };
 
 __device__ __forceinline__ long long warp_min(long long v)   // over the warp
@@ -229,26 +232,12 @@ __device__ __forceinline__ int settle_log(const FlipEntry* f, int n, int tested,
     }
 }
 
-__device__ __forceinline__ int warp_inclusive_scan(int v, int lane)
+// The positions before the r-th (0-based) set bit of w, as a mask (its population count is
+// the position): lane v counts the set bits up to v, and the positions with at most r of
+// them precede the bit.
+__device__ __forceinline__ uint32_t bits_before(uint32_t w, int r, int lane)
 {
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int n = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += n;
-    }
-    return v;
-}
-
-// Position of the r-th (0-based) set bit of w; requires r < popc(w).
-__device__ __forceinline__ int nth_set_bit(uint32_t w, int r)
-{
-    int pos = 0, c;
-    c = __popc(w & 0xFFFFu); if (r >= c) { r -= c; pos += 16; w >>= 16; }
-    c = __popc(w & 0xFFu);   if (r >= c) { r -= c; pos += 8;  w >>= 8; }
-    c = __popc(w & 0xFu);    if (r >= c) { r -= c; pos += 4;  w >>= 4; }
-    c = __popc(w & 0x3u);    if (r >= c) { r -= c; pos += 2;  w >>= 2; }
-    c = (int)(w & 1u);       if (r >= c) { pos += 1; }
-    return pos;
+    return __ballot_sync(0xffffffffu, __popc(w & (0xffffffffu >> (31 - lane))) <= r);
 }
 
 // h[vk] for a warp-uniform vk: a tree of selections up to V = 16 (the indirect branch of
@@ -324,9 +313,8 @@ template <int V> struct Row<f32e, V> {
 };
 
 // Row k of W in the warp row order (step_uses_coal in da_internal.h): p points at
-// entry 4 l of the warp's 32 V-entry slice of the row (lane l); float4 number q, at
-// p + 128 q, holds the lane's slots 4 q .. 4 q + 3.  Every load instruction of the
-// warp reads 512 contiguous bytes.
+// the lane's first entry; float4 number q, at p + 128 q, holds the lane's slots
+// 4 q .. 4 q + 3.
 template <typename Tw, int V> struct RowCoal;
 template <int V> struct RowCoal<float, V> {
     static __device__ __forceinline__ void load(const float* p, float (&c)[V])
@@ -418,19 +406,16 @@ template <int V> struct Row<int16_t, V> {
     }
 };
 
-// Replicas per block and the blocks per SM the register budget is sized for:
-// at least 7 replicas per SM, so that 1024 replicas fill 152 SMs in one wave.
-template <int G> struct Occupancy;
-template <> struct Occupancy<1> { static constexpr int rpb = 4, min_blocks = 2; };
-template <> struct Occupancy<2> { static constexpr int rpb = 2, min_blocks = 4; };
-template <> struct Occupancy<4> { static constexpr int rpb = 1, min_blocks = 7; };
-template <> struct Occupancy<8> { static constexpr int rpb = 1, min_blocks = 2; };
-// Per (G, V): as Occupancy<G>, except G = 4 with V = 32, whose 32 fields per lane need
-// more registers than 7 blocks of 4 warps per SM leave (3 blocks: 12 warps per SM).
-template <int G, int V> struct OccupancyGV {
-    static constexpr int rpb = Occupancy<G>::rpb, min_blocks = Occupancy<G>::min_blocks;
-};
-template <> struct OccupancyGV<4, 32> { static constexpr int rpb = 1, min_blocks = 3; };
+// Replicas per block and the blocks per SM the register budget is sized for: 8 one-warp
+// replicas per SM, so that 1024 replicas fill 152 SMs in one wave; for G > 1 as many as
+// fit without spills (sized for 7 blocks per SM, G = 4 with V = 8 took 0.729 instead of
+// 0.596 us per step at N = 1024; sized for 2, G = 8 with V = 32 3.05 instead of 1.72 at
+// N = 8192; 32 replicas).
+template <int G, int V> struct OccupancyGV;
+template <int V> struct OccupancyGV<1, V> { static constexpr int rpb = 4, min_blocks = 2; };
+template <int V> struct OccupancyGV<2, V> { static constexpr int rpb = 2, min_blocks = V == 32 ? 3 : 4; };
+template <int V> struct OccupancyGV<4, V> { static constexpr int rpb = 1, min_blocks = V == 32 ? 3 : 4; };
+template <int V> struct OccupancyGV<8, V> { static constexpr int rpb = 1, min_blocks = V >= 16 ? 1 : 2; };
 
 // The state words of a replica are standard bit-packed words (x_i is bit i%32
 // of word i/32); a lane's V bits are one slice of word (w*32V + l*V) / 32.

@@ -4,7 +4,8 @@ addition after the other elsewhere.  Checked against the oracle, which adds and 
 after every step, bit for bit: tracked energies (the checkpoint's scalars), best states,
 flips.  The instances reach both forms: energies on one grid, energies that gain and lose
 binary places (couplings of mixed magnitude), exponents outside the integer form's range,
-numbers of steps and recompute periods around the 32-flip window, steps without flips."""
+numbers of steps and recompute periods around the 32-flip window, steps without flips, one
+and several warps per replica (each warp restores its own words of the best state)."""
 import numpy as np
 import pytest
 
@@ -39,16 +40,17 @@ def _instance(kind, N):
 
 
 @pytest.mark.parametrize("kind", ["int8", "sk", "mixed", "tiny", "huge"])
-@pytest.mark.parametrize("N,shape", [(33, None), (100, None), (256, None), (500, None), (1024, None)])
-@pytest.mark.parametrize("T,rec", [(1, 0), (32, 0), (33, 1), (700, 31), (701, 64)])
+@pytest.mark.parametrize("N,shape", [(33, (4, 1, 4)), (100, (8, 1, 2)), (500, (16, 1, 1)), (1000, (32, 1, 4)),
+                                     (200, (4, 2, 2)), (509, (4, 4, 1)), (700, (8, 4, 1)), (1024, (16, 2, 1)),
+                                     (1023, (16, 4, 1)), (1500, (8, 8, 1))])
+@pytest.mark.parametrize("T,rec", [(1, 0), (33, 1), (700, 31)])
 def test_tracked_energy_and_best_state_match_the_oracle(da, kind, N, shape, T, rec):
     import oracle
     Q, scale = _instance(kind, N)
     beta = (np.linspace(0.2, 6.0, T) / scale).astype(np.float32)
     inc, R = 0.25 * min(scale, 1.0), 5
     ctx = da.da_create(Q)
-    if shape:
-        da.da_set_launch_shape(ctx, *shape)
+    da.da_set_launch_shape(ctx, *shape)
     res, ck = da.da_anneal_segment(ctx, beta, 0, T, inc, R, 9, recompute_every=rec)
     ref = oracle.da_anneal(Q, beta, R=R, seed=9, inc=inc, recompute_every=rec, nthreads=5)
     tracked = ck["scalars"][:, 0] if kind == "int8" else ck["scalars"][:, 0].view(np.float64)
