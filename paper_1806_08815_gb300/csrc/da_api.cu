@@ -51,7 +51,6 @@ struct da_ctx {
     da_dtype dtype = DA_INT8;
     int ldw = 0;
     int S = 0;  // fixed-point scale of the fp32 recompute
-    bool exact_shift = false;  // fp32: every entry reaches the grid by a left shift
     int device = 0;
     void* W = nullptr;
     void* Wf = nullptr;  // DA_INT8: the couplings as exact fp32, for the step kernel
@@ -401,20 +400,6 @@ bool build_instance(const void* Q, int n, int dtype, HostInstance& out, std::str
                 amax = std::max(amax, std::fabs(v));
             }
         out.S = fix_scale(amax, n);
-        // every nonzero entry a normal number whose grid value round(v 2^S) needs no
-        // rounding (a left shift of its significand): the warp-level recompute then
-        // converts with a shift alone
-        out.exact_shift = true;
-        for (int i = 0; i < n && out.exact_shift; ++i)
-            for (int j = i; j < n; ++j) {
-                uint32_t b;
-                std::memcpy(&b, q + (size_t)i * n + j, 4);
-                const int E = (int)((b >> 23) & 0xFFu);
-                if ((b & 0x7FFFFFFFu) != 0 && (E == 0 || E - 150 + out.S < 0)) {
-                    out.exact_shift = false;
-                    break;
-                }
-            }
     }
     return true;
 }
@@ -431,7 +416,6 @@ StepShape default_shape(int N, int R) { return auto_shape(N, R); }
 
 void set_last_error(const std::string& msg) { g_err = msg; }
 const TcOperand& ctx_tc_operand(const da_ctx* c) { return c->tc; }
-bool ctx_exact_shift(const da_ctx* c) { return c->exact_shift; }
 
 const void* ctx_coal_W(da_ctx* c, int V)
 {
@@ -483,7 +467,6 @@ da_status da_create(const void* Q, int64_t N, da_dtype dtype, da_ctx** out)
     c->ldw = ldw;
     c->device = dev;
     c->S = hin.S;
-    c->exact_shift = hin.exact_shift;
     auto bail = [&](da_status s, const std::string& m) {
         da_destroy(c);
         return fail(s, m);

@@ -48,23 +48,34 @@ namespace {
 
 using step_detail::WarpReplica;
 
-// One work unit: replica r of item it, all of its steps, by the calling warp;
+// What a warp of a batched kernel keeps in shared memory: its unit's item (read outside
+// the steps, so that its fields take no registers of the step) and its flip log.
+template <typename Tw> struct UnitShared {
+    BatchItemDev it;
+    step_detail::FlipLog<typename step_detail::Arith<Tw>::E> log;
+};
+
+// One work unit: replica r of item u.it, all of its steps, by the calling warp;
 // W points at the item's couplings (global memory, row pitch ldw) or at a
 // copy staged in shared memory (SW, row pitch ldw = 32 V).
 template <typename Tw, int V, bool SW, bool COAL = false>
-__device__ __forceinline__ void run_unit(const BatchItemDev& it, int r, const Tw* W, int ldw, long long t_limit,
-                                         step_detail::FlipLog<typename step_detail::Arith<Tw>::E>* log)
+__device__ __forceinline__ void run_unit(UnitShared<Tw>& u, int r, const Tw* W, int ldw, long long t_limit)
 {
-    // the precomputed draws (PRE) for V <= 16; the V = 32 kernel has no registers left for
-    // them (measured slower)
-    constexpr bool kPre = V <= 16;
+    // The precomputed Philox words and the table of round keys where there are registers for
+    // them: not beside the recompute at V = 32 (1.39 instead of 1.51 ms per 1024 steps of 512
+    // replicas without the words), and the table only in the staged kernels, whose bounds
+    // leave it room (0.645 against 0.727 ms); the keys come from the unit's item, not from a
+    // launch parameter in constant memory.
+    constexpr bool kPre = V <= 16 || !std::is_same<Tw, float>::value;
     using R_ = WarpReplica<Tw, V, SW, kPre, COAL>;
     using A = step_detail::Arith<Tw>;
     using H = typename R_::H;
+    constexpr bool kReal = std::is_same<Tw, float>::value;
     constexpr int nw = V;   // state words per replica (the padded width 32V / 32)
+    const BatchItemDev& it = u.it;
     const int lane = threadIdx.x & 31;
     R_ rp;
-    rp.init(W, it.N, ldw, (uint32_t)r, it.xs + ((size_t)it.R + r) * nw, log->f, &log->head);
+    rp.init(W, it.N, ldw, (uint32_t)r, it.xs + ((size_t)it.R + r) * nw, u.log.f, &u.log.head);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
         if constexpr (std::is_same<Tw, step_detail::f32e>::value)   // int32 diagonal, exact in fp32
@@ -74,33 +85,36 @@ __device__ __forceinline__ void run_unit(const BatchItemDev& it, int r, const Tw
     }
     rp.xm = 0;
     rp.m = 0;
-    const PhiloxKeys keys(it.seed);
-    const long long T = t_limit > 0 ? std::min(t_limit, it.T) : it.T;
+    const std::conditional_t<SW, PhiloxKeys, PhiloxSeed> keys(it.seed);
+    const float inc = it.inc;
+    const uint32_t T = (uint32_t)(t_limit > 0 ? std::min(t_limit, it.T) : it.T);   // < 2^32
     rp.begin(0, T, it.beta, 0.f, 0, 0, 0, keys);
-    if constexpr (kPre) {
-        rp.prep_draws(keys);
-        if (T > 0) rp.draw_pre(0u, keys);
-    } else {
-        if (T > 0) rp.draw(0u, keys);
-    }
-    // the next step count (t + 1) at which the fp32 fields are recomputed: a running
-    // target instead of a 64-bit remainder every step
-    long long next_rec = std::is_same<Tw, float>::value && it.recompute_every > 0 ? it.recompute_every : -1;
-    for (long long t = 0; t < T; ++t) {
-        const int k = rp.template step<false>(t, t + 1 < T, it.inc, keys);
-        if (it.trace && lane == 0) it.trace[(size_t)r * it.T + t] = k;
-        if (it.stop && (t & 1023) == 1023 && *reinterpret_cast<const volatile int*>(it.stop)) break;
-        if constexpr (std::is_same<Tw, float>::value) {
-            if (t + 1 == next_rec) {
-                next_rec += it.recompute_every;
+    // the steps up to the next point where something else is due: a recompute of the
+    // fp32 fields, a look at the stop flag, the trace of every step, the end
+    uint32_t t = 0;
+    while (t < T) {
+        // the draws (and their step-invariant words) are made anew after a recompute: dead
+        // across it, they free their registers for it
+        if constexpr (kPre) {
+            rp.prep_draws(keys);
+            rp.draw_pre(t, keys);
+        } else {
+            rp.draw(t, keys);
+        }
+        long long due = T;
+        if (kReal && it.recompute_every > 0)
+            due = std::min(due, (t / it.recompute_every + 1) * it.recompute_every);
+        if (it.stop) due = std::min(due, ((long long)t / 1024 + 1) * 1024);
+        if (it.trace) due = t + 1;
+        int k = -1;
+        for (const uint32_t t1 = (uint32_t)due; t < t1; ++t) k = rp.template step<false>(t, true, inc, keys);
+        if (it.trace && lane == 0) it.trace[(size_t)r * it.T + t - 1] = k;
+        if (it.stop && t % 1024 == 0 && *reinterpret_cast<const volatile int*>(it.stop)) break;
+        if constexpr (kReal) {
+            if (it.recompute_every > 0 && t % it.recompute_every == 0) {
                 if (rp.n > 0) rp.settle(k >= 0);
-                rp.recompute(static_cast<const float*>(it.diag), it.S, it.exact_shift != 0);
+                rp.recompute(static_cast<const float*>(it.diag), it.S);
                 rp.test_current();
-                // the draws of t + 1 again: lg is dead across the recompute, which frees its registers
-                if (t + 1 < T) {
-                    if constexpr (kPre) rp.draw_pre((uint32_t)(t + 1), keys);
-                    else rp.draw((uint32_t)(t + 1), keys);
-                }
             }
         }
     }
@@ -109,21 +123,26 @@ __device__ __forceinline__ void run_unit(const BatchItemDev& it, int r, const Tw
     if (lane % R_::P == 0) it.xs[(size_t)r * nw + (rp.base >> 5)] = word;
     if (lane == 0) {
         ReplicaScalars s;
-        s.E = A::store_e(log->head.E);
-        s.best = A::store_e(log->head.best);
-        s.flips = log->head.flips;
+        s.E = A::store_e(u.log.head.E);
+        s.best = A::store_e(u.log.head.best);
+        s.flips = u.log.head.flips;
         s.m = rp.m;
         s.check = 0;
         it.sc[r] = s;
     }
+    __syncwarp();           // every lane is done with the item before the next one takes its place
 }
 
 // COAL: rows of W from the items' copies in the one-warp row order (it.Wc).
+// Blocks per SM in the launch bounds: registers enough for the step without spills (the
+// compiler's own choice leaves V = 16 with fewer: 0.77 instead of 0.69 ms per 1024 steps
+// of 512 fp32 replicas).
 template <typename Tw, int V, bool COAL = false>
-__global__ void __launch_bounds__(128) batch_kernel(const __grid_constant__ BatchClassParams bp)
+__global__ void __launch_bounds__(128, V == 4 ? 4 : V == 8 ? 3 : 2)
+    batch_kernel(const __grid_constant__ BatchClassParams bp)
 {
-    __shared__ step_detail::FlipLog<typename step_detail::Arith<Tw>::E> logs[4];
-    step_detail::FlipLog<typename step_detail::Arith<Tw>::E>* log = &logs[threadIdx.x >> 5];
+    __shared__ UnitShared<Tw> shared[4];
+    UnitShared<Tw>& u = shared[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     for (;;) {
         unsigned long long unit = 0;
@@ -137,10 +156,11 @@ __global__ void __launch_bounds__(128) batch_kernel(const __grid_constant__ Batc
             if ((unsigned long long)bp.items[mid].unit0 <= unit) lo = mid;
             else hi = mid - 1;
         }
-        const BatchItemDev it = bp.items[lo];
-        const int r = (int)(unit - (unsigned long long)it.unit0);
-        if constexpr (COAL) run_unit<Tw, V, false, true>(it, r, static_cast<const Tw*>(it.Wc), 32 * V, bp.t_limit, log);
-        else run_unit<Tw, V, false>(it, r, static_cast<const Tw*>(it.W), it.ldw, bp.t_limit, log);
+        if (lane == 0) u.it = bp.items[lo];
+        __syncwarp();
+        const int r = (int)(unit - (unsigned long long)u.it.unit0);
+        if constexpr (COAL) run_unit<Tw, V, false, true>(u, r, static_cast<const Tw*>(u.it.Wc), 32 * V, bp.t_limit);
+        else run_unit<Tw, V, false>(u, r, static_cast<const Tw*>(u.it.W), u.it.ldw, bp.t_limit);
     }
 }
 
@@ -153,7 +173,7 @@ __global__ void __launch_bounds__(512) batch_kernel_smem(const __grid_constant__
     extern __shared__ __align__(16) unsigned char wsm_raw[];
     Tw* Ws = reinterpret_cast<Tw*>(wsm_raw);
     __shared__ long long s_group;
-    __shared__ step_detail::FlipLog<typename step_detail::Arith<Tw>::E> logs[16];
+    __shared__ UnitShared<Tw> shared[16];
     const int warp = threadIdx.x >> 5;
     for (;;) {
         __syncthreads();   // every warp is done with the previous group's copy
@@ -173,7 +193,9 @@ __global__ void __launch_bounds__(512) batch_kernel_smem(const __grid_constant__
         }
         __syncthreads();
         const int r = gi.y + warp;
-        if (r < it.R) run_unit<Tw, V, true>(it, r, Ws, cols, bp.t_limit, &logs[warp]);
+        if ((threadIdx.x & 31) == 0) shared[warp].it = it;
+        __syncwarp();
+        if (r < it.R) run_unit<Tw, V, true>(shared[warp], r, Ws, cols, bp.t_limit);
     }
 }
 
@@ -288,8 +310,8 @@ thread_local std::string g_batch_desc;
 constexpr long long kProbeSteps = 1024;
 
 // Largest dynamic shared memory a block may ask for on sm_100-class GPUs, less the
-// kernel's static part (the flip logs of 16 warps).
-constexpr size_t kMaxStagedBytes = 227u * 1024u - 16u * sizeof(step_detail::FlipLog<double>) - 64u;
+// kernel's static part.
+constexpr size_t kMaxStagedBytes = 227u * 1024u - 16u * sizeof(UnitShared<float>) - 64u;
 
 int blocks_for(BatchKernel k, int warps_per_block, int sms, size_t smem)
 {
@@ -625,7 +647,6 @@ extern "C" da_status da_batch_anneal(const da_batch_item* items, int32_t n, doub
                 d.S = hi[i].S;
                 d.R = it.replicas;
                 d.inc = it.offset_inc;
-                d.exact_shift = da::ctx_exact_shift(it.ctx) ? 1 : 0;
                 desc[di++] = d;
                 units += it.replicas;
             }

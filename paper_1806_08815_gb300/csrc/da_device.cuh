@@ -39,8 +39,28 @@ struct PhiloxKeys {
     }
 };
 
-__device__ __forceinline__ u32x4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
-                                               const PhiloxKeys& k)
+// The same keys formed where they are used: two registers instead of twenty, one add per
+// round and use.  For kernels whose seed is not a launch parameter (whose keys are not in
+// constant memory) and that have no registers for the table.
+struct PhiloxSeed {
+    struct Words {
+        uint32_t k, weyl;
+        __device__ __forceinline__ uint32_t operator[](int r) const
+        {
+            uint32_t w;   // volatile: not moved out of the step loop, where it would take registers
+            asm volatile("add.u32 %0, %1, %2;" : "=r"(w) : "r"(k), "r"((uint32_t)r * weyl));
+            return w;
+        }
+    };
+    Words a, b;
+    __device__ __forceinline__ explicit PhiloxSeed(uint64_t seed)
+        : a{(uint32_t)seed, kPhiloxWeylA}, b{(uint32_t)(seed >> 32), kPhiloxWeylB}
+    {
+    }
+};
+
+template <class Keys>
+__device__ __forceinline__ u32x4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, const Keys& k)
 {
 #pragma unroll
     for (int round = 0; round < 10; ++round) {
