@@ -151,6 +151,7 @@ da_status ensure_ws(da_ctx* c, size_t bytes)
 // Workspace carve-up for one anneal-like call.
 struct Layout {
     size_t h, xs, sc, sums, eex, beta, res, trace, pt, total;
+    size_t arrived;   // after sc: the counters of the periodic recompute (launch_recompute_tc)
 };
 
 Layout plan(const da_ctx* c, const StepShape& s, int R, long long T, bool with_beta, bool with_trace, size_t pt_bytes)
@@ -160,7 +161,9 @@ Layout plan(const da_ctx* c, const StepShape& s, int R, long long T, bool with_b
     auto take = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes, 256); return at; };
     L.h = take((size_t)R * s.npad() * 4);
     L.xs = take((size_t)2 * R * s.nwords() * 4);
-    L.sc = take((size_t)R * sizeof(ReplicaScalars));
+    L.sc = o;
+    L.arrived = L.sc + (size_t)R * sizeof(ReplicaScalars);
+    take((size_t)R * sizeof(ReplicaScalars) + (size_t)((R + da::kTcStates - 1) / da::kTcStates) * sizeof(unsigned));
     L.sums = take(da::tc_partial_bytes(std::max(s.npad(), c->N), 2 * R));
     L.eex = take((size_t)2 * R * 8);
     L.beta = take(with_beta ? (size_t)T * 4 : 0);
@@ -201,6 +204,8 @@ struct RunBuffers {
     uint32_t* x() const { return reinterpret_cast<uint32_t*>(base + L.xs); }
     uint32_t* bestx() const { return x() + (size_t)R * s.nwords(); }
     ReplicaScalars* sc() const { return reinterpret_cast<ReplicaScalars*>(base + L.sc); }
+    size_t zeroed_bytes() const { return L.sums - L.sc; }   // sc and the counters
+    unsigned* arrived() const { return reinterpret_cast<unsigned*>(base + L.arrived); }
     long long* sums() const { return reinterpret_cast<long long*>(base + L.sums); }
     long long* eex() const { return reinterpret_cast<long long*>(base + L.eex); }
 };
@@ -256,7 +261,7 @@ da_status reset_state(const da_ctx* c, const RunBuffers& b, cudaStream_t st)
 {
     DA_CU(da::launch_init_state(is_int(c), c->diag, c->N, b.R, b.h(), b.s.npad(), st, c->dtype == DA_INT8));
     DA_CU(cudaMemsetAsync(b.x(), 0, (size_t)2 * b.R * b.s.nwords() * 4, st));
-    DA_CU(cudaMemsetAsync(b.sc(), 0, (size_t)b.R * sizeof(ReplicaScalars), st));
+    DA_CU(cudaMemsetAsync(b.sc(), 0, b.zeroed_bytes(), st));
     return DA_OK;
 }
 
@@ -326,7 +331,7 @@ da_status run_anneal(da_ctx* c, const RunBuffers& b, const float* beta_dev, long
         if (rec && p.t1 % recompute_every == 0) {
             DA_CU(da::launch_recompute_tc(false, c->tc, c->diag, c->N, c->S, b.x(), b.s.nwords(), b.R, b.h(),
                                           b.s.npad(), reinterpret_cast<long long*>(b.sc()),
-                                          (int)(sizeof(ReplicaScalars) / 8), st, b.sums()));
+                                          (int)(sizeof(ReplicaScalars) / 8), st, b.sums(), b.arrived()));
         }
     }
     DA_CU(da::launch_best_fixup(b.R, b.sc(), is_int(c), b.x(), b.bestx(), b.s.nwords(), st));
@@ -1063,6 +1068,7 @@ da_status restore_state(const da_ctx* c, const RunBuffers& b, const da_checkpoin
         sc[r].m = (uint32_t)in->scalars[4 * r + 3];
         sc[r].check = 0;
     }
+    DA_CU(cudaMemsetAsync(b.sc(), 0, b.zeroed_bytes(), st));   // the counters
     DA_CU(cudaMemcpyAsync(b.sc(), sc, (size_t)R * sizeof(ReplicaScalars), cudaMemcpyHostToDevice, st));
     return DA_OK;
 }

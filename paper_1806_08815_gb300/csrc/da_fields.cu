@@ -161,15 +161,7 @@ __global__ void energy_kernel(const I128* __restrict__ part, int tiles, int R, i
     if (r >= R) return;
     I128 s = {0ull, 0ll};
     for (int b = 0; b < tiles; ++b) s = i128_add(s, part[(size_t)b * R + r]);
-    if constexpr (INT8) {
-        E[(size_t)r * Estride] = (long long)s.lo / 2;   // |2E| < 2^63
-    } else {
-        // value = hi 2^64 + lo; top = value >> 32 (exact in fp64, |value| < 2^76)
-        const long long top = (long long)((unsigned long long)s.hi << 32 | (s.lo >> 32));
-        const double bottom = (double)(uint32_t)(s.lo & 0xFFFFFFFFull);
-        const double v = __fma_rn((double)top, 4294967296.0, bottom);
-        E[(size_t)r * Estride] = __double_as_longlong(ldexp(v, -(S + 1)));
-    }
+    E[(size_t)r * Estride] = energy_of_sum<INT8>(s.lo, s.hi, S);
 }
 
 // g[r][i] = diag[i] for i < N, 0 on the padding (MODE 0: int32 diag and

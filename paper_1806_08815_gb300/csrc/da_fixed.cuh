@@ -37,31 +37,38 @@ __device__ __forceinline__ long long fixed_of_f32(float w, int S)
 }
 
 // fl32(v) 2^-S: v rounded to fp32 (to nearest, ties to even), then scaled;
-// equal to ldexpf(__ll2float_rn(v), -S).  Results outside the normal range
-// are left to ldexpf.
+// equal to ldexpf(__ll2float_rn(v), -S).  |v| is shifted so that its leading bit is
+// bit 31 of a 32-bit word whose lowest bit also stands for all bits below it: the
+// word's conversion then rounds as the 64-bit value would, and the scale is a
+// multiplication by a power of two.  Scales outside the normal range are left to
+// ldexpf.
 __device__ __forceinline__ float scaled_f32_of(long long v, int S)
 {
-    if (v == 0) return 0.f;
-    const uint32_t sign = v < 0 ? 0x80000000u : 0u;
     const unsigned long long u = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
-    int e = 63 - __clzll((long long)u);          // u in [2^e, 2^(e+1))
-    uint32_t mant;
-    if (e <= 23) {
-        mant = (uint32_t)(u << (23 - e));
+    const int z = __clzll((long long)u);         // 64 for v = 0
+    const unsigned long long n = u << (z & 63);
+    const uint32_t top = (uint32_t)(n >> 32) | ((uint32_t)n != 0u ? 1u : 0u);
+    const float f = __uint_as_float(__float_as_uint(__uint2float_rn(top)) | (v < 0 ? 0x80000000u : 0u));
+    const int x = 32 - z - S;                     // |v| 2^-S = top 2^x
+    // the product stays normal: top is 0 or at least 2^31, at most 2^32
+    if (x >= -126 && x <= 95) return v == 0 ? 0.f : __fmul_rn(f, __uint_as_float((uint32_t)(x + 127) << 23));
+    return v == 0 ? 0.f : ldexpf(f, x);
+}
+
+// The energy (hi 2^64 + lo) / 2^(S + 1) of a 128-bit sum: integer couplings (S = 0) as
+// int64 (exact), fp32 ones rounded once to fp64, as its bits.
+template <bool INT8>
+__device__ __forceinline__ long long energy_of_sum(unsigned long long lo, long long hi, int S)
+{
+    if constexpr (INT8) {
+        return (long long)lo / 2;   // |2E| < 2^63
     } else {
-        const int rs = e - 23;
-        const unsigned long long q = u >> rs;
-        const unsigned long long rem = u & ((1ull << rs) - 1ull);
-        const unsigned long long half = 1ull << (rs - 1);
-        mant = (uint32_t)q + ((rem > half || (rem == half && (q & 1ull))) ? 1u : 0u);
-        if (mant == (1u << 24)) {
-            mant >>= 1;
-            ++e;
-        }
+        // value = hi 2^64 + lo; top = value >> 32 (exact in fp64, |value| < 2^76)
+        const long long top = (long long)((unsigned long long)hi << 32 | (lo >> 32));
+        const double bottom = (double)(uint32_t)(lo & 0xFFFFFFFFull);
+        const double v = __fma_rn((double)top, 4294967296.0, bottom);
+        return __double_as_longlong(ldexp(v, -(S + 1)));
     }
-    const int be = e - S + 127;
-    if (be >= 1 && be <= 254) return __uint_as_float(sign | ((uint32_t)be << 23) | (mant & 0x7FFFFFu));
-    return ldexpf(__uint_as_float(sign | ((uint32_t)(e + 127) << 23) | (mant & 0x7FFFFFu)), -S);
 }
 
 // The integer value of an fp32 that holds an integer of magnitude < 2^22

@@ -161,10 +161,13 @@ cudaError_t tc_operand_build_in(int wtype, const void* W, const void* diag, int 
 // 64-column tile.
 size_t tc_partial_bytes(int rows, int R);
 // Arguments as launch_recompute (is_int8: integer couplings of either width,
-// int32 fields); with E, scratch must hold tc_partial_bytes(rows, R) bytes.
+// int32 fields); with E, scratch must hold tc_partial_bytes(rows, R) bytes.  arrived
+// (optional): ceil(R / kTcStates) counters, 0 before the call and left 0 by it, not shared
+// with another call in flight: the kernel then sums the partial energies itself.
 cudaError_t launch_recompute_tc(bool is_int8, const TcOperand& op, const void* diag, int N, int S,
                                 const uint32_t* xs, int nw, int R, void* hout, int npad, long long* E, int Estride,
-                                cudaStream_t st, long long* scratch);
+                                cudaStream_t st, long long* scratch, unsigned* arrived = nullptr);
+constexpr int kTcStates = 128;   // states per tile of the kernel
 
 // PT exchange (da_pt.cu).
 cudaError_t launch_pt_exchange(bool is_int8, const float* betas, int K, int L,

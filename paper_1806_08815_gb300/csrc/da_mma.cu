@@ -22,16 +22,23 @@
 // staged in HBM at all: two warps of the block expand the tile's state bits
 // (2 words per state and stage) to f16 {0, 1} directly into the stage.
 //
-// Block: 16 warps, 128 states x 64 variables.  Warp 0 allocates tensor memory
-// and one of its threads issues the digit planes' bulk copies into a 3-stage
-// ring; warps 2-3 write the stage's state tile (the words of the next chunk
-// loaded while the current one is written); one thread of warp 1 issues the
-// MMAs (4 K-steps of 16 per stage, one per digit plane each) and commits the
-// stage back to both producers; then all 16 warps read their TMEM lanes (warp
-// w: states 32 (w % 4).., 16 variables from 16 (w / 4)) and write fields and
-// 128-bit partial energies.  (32-variable tiles, two blocks an SM, measured
-// slower: every block expands its states again, and at 6 digit planes only one
-// block fits.)
+// Block: 16 warps, 128 states x 64 variables.  Warp 0 allocates tensor memory and
+// issues the digit planes' bulk copies (4 KB a lane) into a 3-stage ring; warps 2-9
+// write the stage's state tile (half a state each, the word of the next chunk loaded
+// while the current one is written); one thread of warp 1 issues the MMAs (4 K-steps of
+// 16 per stage, the digit planes side by side as up to 192 columns of one or two MMAs:
+// one MMA of 64 columns per plane took 1.17 us a stage at 5 planes, this form 0.85) and
+// commits the stage back to both producers; then all 16 warps read their TMEM lanes
+// (warp w: states 32 (w % 4).., 16 variables from 16 (w / 4)) and write fields and
+// 128-bit partial energies, and the last block of a state tile sums those.
+//
+// What bounds it at the sizes of an anneal (N = 1024) is the chain of a short launch:
+// 16 stages of 0.5 us of MMAs each, and half the time outside them.  With the step
+// launch that follows, a recompute at N = 1024 costs 30 us with 128 states (38.5 with
+// the energies in a launch of their own and the form before) and 34 us with 1024 (49.4);
+// at N = 8192 it streams the digit planes from HBM.  (32-variable tiles, two blocks an
+// SM, measured slower: every block expands its states again, and at 6 digit planes only
+// one block fits.)
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -46,13 +53,14 @@
 namespace da {
 namespace {
 
-constexpr int kBM = 128;   // states per tile (TMEM lanes)
+constexpr int kBM = kTcStates;   // states per tile (TMEM lanes)
 constexpr int kBN = 64;    // variables per tile (TMEM columns per digit plane)
 constexpr int kBK = 64;    // couplings per pipeline stage
 constexpr int kStages = 3;
+constexpr uint32_t kPiece = 4096;            // bytes of one bulk copy (kBTile is a multiple)
 constexpr int kThreads = 128 * (kBN / 16);   // warp w reads TMEM lanes 32 (w % 4).., columns 16 (w / 4)..
 constexpr int kMinBlocks = 512 / kThreads;   // blocks per SM the launch bounds plan for
-constexpr int kExpanders = 64;  // threads of warps 2-3: the state tile of each stage, 2 states each
+constexpr int kExpanders = 2 * kBM;  // threads of warps 2-9: the state tile of each stage, half a state each
 constexpr uint32_t kATile = kBM * kBK * 2;   // bytes of one state tile (16 KB)
 constexpr uint32_t kBTile = kBN * kBK * 2;   // bytes of one digit-plane tile (8 KB)
 constexpr uint32_t kWaitLimit = 1u << 26;    // polls of one mbarrier before giving up ...
@@ -119,7 +127,7 @@ __global__ void build_digits_kernel(const void* __restrict__ W, int N, int ldw, 
             v[e] = (v[e] - d) >> bits;
             h[e] = __int2half_rn((int)d);
         }
-        __half* dst = B + ((size_t)tile * limbs + l) * (kBN * kBK) + core_offset(kBN, row, g * 8);
+        __half* dst = B + (size_t)tile * limbs * (kBN * kBK) + core_offset(kBN * limbs, l * kBN + row, g * 8);
         *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(h);
     }
 }
@@ -146,12 +154,30 @@ __device__ __forceinline__ void i128_add(I128& a, long long v)
     a.lo = lo;
 }
 
+__device__ __forceinline__ void i128_add2(I128& a, const I128& b)
+{
+    const unsigned long long lo = a.lo + b.lo;
+    a.hi += b.hi + (lo < a.lo ? 1ll : 0ll);
+    a.lo = lo;
+}
+
+// A partial sum that another block wrote (16-byte aligned), from L2.
+__device__ __forceinline__ I128 load_partial(const I128* p)
+{
+    const ulonglong2 v = __ldcg(reinterpret_cast<const ulonglong2*>(p));
+    return I128{v.x, (long long)v.y};
+}
+
 struct TcParams {
     const __half* B;        // [ceil(N/64)][kchunks][limbs] digit-plane tiles
     const long long* dfix;  // [kchunks * 64] fixed-point diagonal, zero-padded
     const uint32_t* xs;     // [R][nw] state bits (x_i = bit i % 32 of word i / 32)
     void* hout;             // [R][npad] or null
     I128* part;             // [gridDim.x][R] or null
+    unsigned* arrived;      // [gridDim.y], 0 before the launch and after it, or null: the block
+                            // of a state tile that comes last sums the partial energies itself
+    long long* E;           // with arrived: E[r Estride] as launch_energy_sum writes it
+    int Estride;
     int* err;
     int N, S, bits, limbs, kchunks, nw, R, npad;
     uint32_t ncols;         // tensor-memory columns allocated
@@ -213,25 +239,33 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) recompute_tc_kernel(cons
     const int nk = p.kchunks;
 
     if (warp == 0) {
-        if (lane == 0) {   // bulk-copy issuer: the digit planes of each stage
-            const __half* b_src = p.B + (size_t)blockIdx.x * nk * p.limbs * (kBN * kBK);
-            const uint32_t b_bytes = (uint32_t)p.limbs * kBTile;
-            for (int c = 0; c < nk; ++c) {
-                const int s = c % kStages;
-                const uint32_t u = (uint32_t)(c / kStages);
-                if (u > 0 && !tc::mbar_wait(&empty[s], (u - 1) & 1u, kWaitLimit, kWaitNs)) {
-                    s_fail = 1;
-                    break;
-                }
-                uint8_t* st = sm + s * stage_bytes;
-                tc::mbar_arrive_expect_tx(&full[s], b_bytes);
-                tc::bulk_g2s(st + kATile, b_src + (size_t)c * p.limbs * (kBN * kBK), b_bytes, &full[s]);
+        // bulk-copy issuers: the digit planes of each stage, a piece of kPiece bytes per lane
+        const __half* b_src = p.B + (size_t)blockIdx.x * nk * p.limbs * (kBN * kBK);
+        const uint32_t b_bytes = (uint32_t)p.limbs * kBTile;
+        for (int c = 0; c < nk; ++c) {
+            const int s = c % kStages;
+            const uint32_t u = (uint32_t)(c / kStages);
+            bool ok = true;
+            if (lane == 0) {
+                ok = u == 0 || tc::mbar_wait(&empty[s], (u - 1) & 1u, kWaitLimit, kWaitNs);
+                if (ok) tc::mbar_arrive_expect_tx(&full[s], b_bytes);
+                else s_fail = 1;
             }
+            if (!__all_sync(0xffffffffu, ok)) break;
+            const uint8_t* src = reinterpret_cast<const uint8_t*>(b_src + (size_t)c * p.limbs * (kBN * kBK));
+            uint8_t* st = sm + s * stage_bytes + kATile;
+            for (uint32_t o = lane * kPiece; o < b_bytes; o += 32 * kPiece)
+                tc::bulk_g2s(st + o, src + o, kPiece, &full[s]);
         }
         __syncwarp();
     } else if (warp == 1) {
         if (lane == 0) {   // MMA issuer
-            constexpr uint32_t idesc = tc::idesc_f16_f32(kBM, kBN);
+            // the digit planes side by side as the N side of one MMA (two halves above 256
+            // columns): the accumulator of plane l starts at column 64 l
+            const int parts = p.limbs > 4 ? 2 : 1;
+            const int cols = kBN * p.limbs / parts;      // 64 .. 256, a multiple of 16
+            const uint32_t kstride = (uint32_t)(kBN * p.limbs / 8) * 128;   // between core-matrix columns
+            const uint32_t idesc = tc::idesc_f16_f32(kBM, cols);
             for (int c = 0; c < nk; ++c) {
                 const int s = c % kStages;
                 const uint32_t u = (uint32_t)(c / kStages);
@@ -246,10 +280,9 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) recompute_tc_kernel(cons
                 for (int q = 0; q < kBK / 16; ++q) {
                     // K-step q covers core-matrix columns 2q, 2q + 1 of the stage
                     const uint64_t ad = tc::smem_desc(a0 + q * 2 * (kBM / 8) * 128, (kBM / 8) * 128, 128);
-                    for (int l = 0; l < p.limbs; ++l) {
-                        const uint64_t bd =
-                            tc::smem_desc(b0 + l * kBTile + q * 2 * (kBN / 8) * 128, (kBN / 8) * 128, 128);
-                        tc::mma_f16(tbase + (uint32_t)(l * kBN), ad, bd, idesc, (c > 0 || q > 0) ? 1u : 0u);
+                    for (int h = 0; h < parts; ++h) {
+                        const uint64_t bd = tc::smem_desc(b0 + q * 2 * kstride + (uint32_t)(h * cols / 8) * 128, kstride, 128);
+                        tc::mma_f16(tbase + (uint32_t)(h * cols), ad, bd, idesc, (c > 0 || q > 0) ? 1u : 0u);
                     }
                 }
                 tc::mma_commit(&empty[s]);
@@ -257,50 +290,40 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) recompute_tc_kernel(cons
             tc::mma_commit(done);
         }
         __syncwarp();
-    } else if (warp == 2 || warp == 3) {
-        // the stage's state tile: thread e writes states e and e + 64 of the tile, 64
-        // couplings each (2 state words) as eight 16-byte rows of f16 {0, 1} in the
-        // canonical K-major layout; bits beyond N and states beyond R are 0
+    } else if (warp < 2 + kExpanders / 32) {
+        // the stage's state tile: thread e writes half hh = e / 128 of state e % 128, 32
+        // couplings (one state word) as four 16-byte rows of f16 {0, 1} in the canonical
+        // K-major layout; bits beyond N and states beyond R are 0
         const int e = (int)threadIdx.x - 64;
-        // the two states' words of chunk c: loaded one chunk ahead, so that their latency
-        // overlaps the wait for the stage and the writes of the chunk before
-        auto load = [&](int c, uint32_t (&wv)[4]) {
-            const int w0 = (c * kBK) >> 5;               // < nw: c < kchunks = ceil(N / 64)
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                const int r = blockIdx.y * kBM + e + 64 * hh;
-                const uint32_t* xr = p.xs + (size_t)r * p.nw;
-                wv[2 * hh] = r < p.R ? xr[w0] : 0u;
-                wv[2 * hh + 1] = r < p.R && w0 + 1 < p.nw ? xr[w0 + 1] : 0u;
-            }
+        const int row = e & (kBM - 1), hh = e / kBM;
+        const int rs = blockIdx.y * kBM + row;
+        const uint32_t* xr = p.xs + (size_t)rs * p.nw;
+        // the word of chunk c: loaded one chunk ahead, so that its latency overlaps the
+        // wait for the stage and the writes of the chunk before
+        auto load = [&](int c) {
+            const int w = 2 * c + hh;
+            return rs < p.R && w < p.nw ? xr[w] : 0u;
         };
-        uint32_t cur[4], nxt[4] = {0u, 0u, 0u, 0u};
-        load(0, cur);
+        uint32_t cur = load(0), nxt = 0u;
         for (int c = 0; c < nk; ++c) {
             const int s = c % kStages;
             const uint32_t u = (uint32_t)(c / kStages);
-            if (c + 1 < nk) load(c + 1, nxt);
+            if (c + 1 < nk) nxt = load(c + 1);
             if (u > 0 && !tc::mbar_wait(&empty[s], (u - 1) & 1u, kWaitLimit, kWaitNs)) {
                 s_fail = 1;
                 break;
             }
             uint8_t* st = sm + s * stage_bytes;
-            const int nvalid = min(kBK, p.N - c * kBK);
-            const uint64_t vmask = nvalid >= 64 ? ~0ull : ((1ull << nvalid) - 1ull);
+            const int nvalid = p.N - c * kBK - 32 * hh;
+            const uint32_t bits = nvalid >= 32 ? cur : nvalid <= 0 ? 0u : cur & ((1u << nvalid) - 1u);
 #pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                const int row = e + 64 * hh;
-                const uint64_t bits = (((uint64_t)cur[2 * hh + 1] << 32) | cur[2 * hh]) & vmask;
-#pragma unroll
-                for (int kc = 0; kc < 8; ++kc) {
-                    const uint32_t b = (uint32_t)(bits >> (8 * kc)) & 0xFFu;
-                    const uint4 v = make_uint4(half_pair(b & 3u), half_pair((b >> 2) & 3u), half_pair((b >> 4) & 3u),
-                                               half_pair(b >> 6));
-                    *reinterpret_cast<uint4*>(st + 2 * core_offset(kBM, row, kc * 8)) = v;
-                }
+            for (int kc = 0; kc < 4; ++kc) {
+                const uint32_t b = (bits >> (8 * kc)) & 0xFFu;
+                const uint4 v = make_uint4(half_pair(b & 3u), half_pair((b >> 2) & 3u), half_pair((b >> 4) & 3u),
+                                           half_pair(b >> 6));
+                *reinterpret_cast<uint4*>(st + 2 * core_offset(kBM, row, 32 * hh + 8 * kc)) = v;
             }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) cur[q] = nxt[q];
+            cur = nxt;
             fence_proxy_async_smem();
             tc::mbar_arrive(&full[s]);
         }
@@ -372,14 +395,38 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) recompute_tc_kernel(cons
         I128 t = s_part[0][threadIdx.x];
 #pragma unroll
         for (int g = 1; g < kThreads / kBM; ++g) {
-            const I128 u = s_part[g][threadIdx.x];
-            const unsigned long long lo = t.lo + u.lo;
-            t.hi += u.hi + (lo < t.lo ? 1ll : 0ll);
-            t.lo = lo;
+            i128_add2(t, s_part[g][threadIdx.x]);
         }
         p.part[(size_t)blockIdx.x * p.R + blockIdx.y * kBM + threadIdx.x] = t;
     }
     if (threadIdx.x == 0 && s_fail) atomicExch(p.err, 1);
+
+    // The energies of the tile's states, by the last of its blocks: a launch of their own
+    // takes 5 us beside the 16 us of this one (N = 1024, 128 states).
+    if (p.arrived) {
+        __shared__ int s_last;
+        __threadfence();                                   // the partial sums, before the arrival
+        __syncthreads();
+        const int tiles = (p.N + kBN - 1) / kBN;           // the blocks that come here
+        if (threadIdx.x == 0) s_last = atomicAdd(&p.arrived[blockIdx.y], 1u) == (unsigned)tiles - 1u;
+        __syncthreads();
+        if (!s_last) return;
+        __threadfence();
+        if (threadIdx.x == 0) p.arrived[blockIdx.y] = 0u;
+        I128 t{0ull, 0ll};
+        if (live)
+            for (int b = cg; b < tiles; b += kThreads / kBM) {
+                const I128 u = load_partial(&p.part[(size_t)b * p.R + r]);
+                i128_add2(t, u);
+            }
+        s_part[cg][m] = t;
+        __syncthreads();
+        if (cg == 0 && live) {
+#pragma unroll
+            for (int g = 1; g < kThreads / kBM; ++g) i128_add2(t, s_part[g][m]);
+            p.E[(size_t)r * p.Estride] = energy_of_sum<INT8>(t.lo, t.hi, p.S);
+        }
+    }
 }
 
 size_t smem_bytes(int limbs) { return 1024 + (size_t)kStages * (kATile + (size_t)limbs * kBTile) + 8 * (2 * kStages + 1) + 16; }
@@ -523,7 +570,7 @@ cudaError_t prepare_tc_kernels()
 
 cudaError_t launch_recompute_tc(bool is_int8, const TcOperand& op, const void* diag, int N, int S,
                                 const uint32_t* xs, int nw, int R, void* hout, int npad, long long* E, int Estride,
-                                cudaStream_t st, long long* scratch)
+                                cudaStream_t st, long long* scratch, unsigned* arrived)
 {
     if (R <= 0) return cudaSuccess;
     // the dynamic shared-memory limit of each kernel form, set once per device
@@ -556,6 +603,9 @@ cudaError_t launch_recompute_tc(bool is_int8, const TcOperand& op, const void* d
     p.xs = xs;
     p.hout = hout;
     p.part = E ? reinterpret_cast<I128*>(scratch) : nullptr;
+    p.arrived = E ? arrived : nullptr;
+    p.E = E;
+    p.Estride = Estride;
     p.err = op.err;
     p.N = N;
     p.S = S;
@@ -574,7 +624,7 @@ cudaError_t launch_recompute_tc(bool is_int8, const TcOperand& op, const void* d
     else
         recompute_tc_kernel<false><<<grid, kThreads, smem, st>>>(p);
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || !E) return e;
+    if (e != cudaSuccess || !E || arrived) return e;
     return launch_energy_sum(is_int8, scratch, itiles, R, S, E, Estride, st);
 }
 

@@ -20,6 +20,8 @@
 // energy by their exact fixed-point values (the same definition as the tiled
 // recompute in da_fields.cu, evaluated by the warp itself).
 #pragma once
+#include <type_traits>
+
 #include "da_device.cuh"
 #include "da_fixed.cuh"
 #include "da_internal.h"
@@ -186,6 +188,34 @@ struct WarpReplica {
     }
 
     __device__ __forceinline__ uint32_t word() const { return gather_word<V>(xm, lane); }
+
+    // The lane's V fields between launches (16-byte aligned): a lane's slice is 4 V bytes
+    // from the next one's, so 4-byte accesses took 32 lines each (5 us of a launch of 1024
+    // replicas at N = 1024).
+    __device__ __forceinline__ void load_fields(const H* p)
+    {
+        static_assert(sizeof(H) == 4, "fields are 4 bytes");
+#pragma unroll
+        for (int v = 0; v < V; v += 4) {
+            const uint4 f = *reinterpret_cast<const uint4*>(p + v);
+            const uint32_t w[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if constexpr (std::is_same<H, float>::value) h[v + e] = __uint_as_float(w[e]);
+                else h[v + e] = (H)w[e];
+            }
+        }
+    }
+    __device__ __forceinline__ void store_fields(H* p) const
+    {
+        auto bits = [](H f) {
+            if constexpr (std::is_same<H, float>::value) return __float_as_uint(f);
+            else return (uint32_t)f;
+        };
+#pragma unroll
+        for (int v = 0; v < V; v += 4)
+            *reinterpret_cast<uint4*>(p + v) = make_uint4(bits(h[v]), bits(h[v + 1]), bits(h[v + 2]), bits(h[v + 3]));
+    }
 
     static __device__ __forceinline__ void load_row(const Tw* p, Tw (&c)[V])
     {
@@ -539,9 +569,7 @@ struct WarpReplica {
             hi = hi + ohi + (nlo < lo ? 1ll : 0ll);
             lo = nlo;
         }
-        const long long top = (long long)((unsigned long long)hi << 32 | (lo >> 32));
-        const double v = __fma_rn((double)top, 4294967296.0, (double)(uint32_t)(lo & 0xFFFFFFFFull));
-        if (lane == 0) head->E = ldexp(v, -(S + 1));
+        if (lane == 0) head->E = __longlong_as_double(energy_of_sum<false>(lo, hi, S));
         __syncwarp();
     }
 

@@ -122,8 +122,7 @@ __global__ void __launch_bounds__(32 * G * OccupancyGV<G, V>::rpb, OccupancyGV<G
     const int lane = rp.lane;
     H* hg = static_cast<H*>(p.h) + (size_t)r * p.npad + rp.base;
     uint32_t* xg = p.x + (size_t)r * p.nw;
-#pragma unroll
-    for (int v = 0; v < V; ++v) rp.h[v] = hg[v];
+    rp.load_fields(hg);
     rp.xm = (xg[rp.base >> 5] >> (rp.base & 31)) & R_::VMASK;
     ReplicaScalars sc = p.sc[r];
     rp.m = sc.m;
@@ -235,8 +234,7 @@ __global__ void __launch_bounds__(32 * G * OccupancyGV<G, V>::rpb, OccupancyGV<G
     group_barrier(1 + g, 32 * G);                   // the last flip is in the log
     if (rp.n > 0) rp.settle(held);
 
-#pragma unroll
-    for (int v = 0; v < V; ++v) hg[v] = rp.h[v];
+    rp.store_fields(hg);
     const uint32_t word = rp.word();
     if (lane % R_::P == 0) xg[rp.base >> 5] = word;
     if (w == 0 && lane == 0) {
@@ -268,8 +266,7 @@ __global__ void __launch_bounds__(32 * OccupancyGV<1, V>::rpb, OccupancyGV<1, V>
             &logs[threadIdx.x >> 5].head);
     H* hg = static_cast<H*>(p.h) + (size_t)r * p.npad + rp.base;
     uint32_t* xg = p.x + (size_t)r * p.nw;
-#pragma unroll
-    for (int v = 0; v < V; ++v) rp.h[v] = hg[v];
+    rp.load_fields(hg);
     rp.xm = (xg[rp.base >> 5] >> (rp.base & 31)) & R_::VMASK;
     ReplicaScalars sc = p.sc[r];
     rp.m = sc.m;
@@ -288,8 +285,7 @@ __global__ void __launch_bounds__(32 * OccupancyGV<1, V>::rpb, OccupancyGV<1, V>
             if (rp.lane == 0) p.trace[(size_t)r * p.trace_T + t] = k;
         }
     }
-#pragma unroll
-    for (int v = 0; v < V; ++v) hg[v] = rp.h[v];
+    rp.store_fields(hg);
     const uint32_t word = rp.word();
     if (rp.lane % R_::P == 0) xg[rp.base >> 5] = word;
     if (rp.n > 0) rp.settle(held);
@@ -368,8 +364,7 @@ __global__ void __launch_bounds__(64, 7) step_kernel_ws(const __grid_constant__ 
     rp.init(static_cast<const Tw*>(p.W), p.N, p.ldw, rep, p.bestx + (size_t)r * p.nw, log.f, &log.head);
     H* hg = static_cast<H*>(p.h) + (size_t)r * p.npad + rp.base;
     uint32_t* xg = p.x + (size_t)r * p.nw;
-#pragma unroll
-    for (int v = 0; v < V; ++v) rp.h[v] = hg[v];
+    rp.load_fields(hg);
     rp.xm = (xg[rp.base >> 5] >> (rp.base & 31)) & R_::VMASK;
     ReplicaScalars sc = p.sc[r];
     rp.m = sc.m;
@@ -406,8 +401,7 @@ __global__ void __launch_bounds__(64, 7) step_kernel_ws(const __grid_constant__ 
         }
     }
     if (!__all_sync(0xffffffffu, ok) && lane == 0 && p.err) atomicExch(p.err, 2);
-#pragma unroll
-    for (int v = 0; v < V; ++v) hg[v] = rp.h[v];
+    rp.store_fields(hg);
     const uint32_t word = rp.word();
     if (lane % R_::P == 0) xg[rp.base >> 5] = word;
     if (rp.n > 0) rp.settle(held);
