@@ -9,9 +9,11 @@
 // votes instead of chains of shuffles, the inputs of the next step (draws, choice word,
 // beta) are made in the shadow of this one, and the fp64 energy and the best state are
 // settled 32 flips at a time (FlipLog).  us per step before and after, 64 replicas
-// (1024): fp32 N = 64 0.555 -> 0.346 (0.613 -> 0.41), N = 256 0.670 -> 0.432
-// (0.761 -> 0.535), N = 512 0.781 -> 0.562 (0.918 -> 0.744), N = 1024 0.961 -> 0.883
-// (1.327 -> 1.246).
+// (1024): fp32 N = 64 0.555 -> 0.350 (0.613 -> 0.41), N = 256 0.670 -> 0.432
+// (0.761 -> 0.535), N = 512 0.781 -> 0.562 (0.918 -> 0.757), N = 1024 0.961 -> 0.89
+// (1.327 -> 1.232).  With two warps per scheduler (the last) the pipes bind as much as
+// the chain: a 32 x 32 -> 64 bit product holds the integer multiplier for 4 cycles, and
+// 120 of them with the other multiplications are 1400 of the 2550 cycles.
 //
 // Lane l owns the V consecutive variables i = l*V + v of the replica and keeps
 // their effective fields g_i, bits x_i and the Philox words of the current step
@@ -189,32 +191,42 @@ struct WarpReplica {
 
     __device__ __forceinline__ uint32_t word() const { return gather_word<V>(xm, lane); }
 
-    // The lane's V fields between launches (16-byte aligned): a lane's slice is 4 V bytes
-    // from the next one's, so 4-byte accesses took 32 lines each (5 us of a launch of 1024
-    // replicas at N = 1024).
+    // The lane's V fields between launches (16-byte aligned).  From V = 16 on, where the
+    // lanes' slices are 64 bytes or more apart, as 16-byte accesses: 4-byte ones touch up to
+    // 32 lines each (5 us of a launch of 1024 replicas at N = 1024).
     __device__ __forceinline__ void load_fields(const H* p)
     {
         static_assert(sizeof(H) == 4, "fields are 4 bytes");
+        if constexpr (V < 16) {
 #pragma unroll
-        for (int v = 0; v < V; v += 4) {
-            const uint4 f = *reinterpret_cast<const uint4*>(p + v);
-            const uint32_t w[4] = {f.x, f.y, f.z, f.w};
+            for (int v = 0; v < V; ++v) h[v] = p[v];
+        } else {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                if constexpr (std::is_same<H, float>::value) h[v + e] = __uint_as_float(w[e]);
-                else h[v + e] = (H)w[e];
+            for (int v = 0; v < V; v += 4) {
+                const uint4 f = *reinterpret_cast<const uint4*>(p + v);
+                h[v] = of_bits(f.x);
+                h[v + 1] = of_bits(f.y);
+                h[v + 2] = of_bits(f.z);
+                h[v + 3] = of_bits(f.w);
             }
         }
     }
     __device__ __forceinline__ void store_fields(H* p) const
     {
-        auto bits = [](H f) {
-            if constexpr (std::is_same<H, float>::value) return __float_as_uint(f);
-            else return (uint32_t)f;
-        };
+        if constexpr (V < 16) {
 #pragma unroll
-        for (int v = 0; v < V; v += 4)
-            *reinterpret_cast<uint4*>(p + v) = make_uint4(bits(h[v]), bits(h[v + 1]), bits(h[v + 2]), bits(h[v + 3]));
+            for (int v = 0; v < V; ++v) p[v] = h[v];
+        } else {
+#pragma unroll
+            for (int v = 0; v < V; v += 4)
+                *reinterpret_cast<uint4*>(p + v) =
+                    make_uint4(A::log_bits(h[v]), A::log_bits(h[v + 1]), A::log_bits(h[v + 2]), A::log_bits(h[v + 3]));
+        }
+    }
+    static __device__ __forceinline__ H of_bits(uint32_t b)
+    {
+        if constexpr (std::is_same<H, float>::value) return __uint_as_float(b);
+        else return (H)b;
     }
 
     static __device__ __forceinline__ void load_row(const Tw* p, Tw (&c)[V])
@@ -371,8 +383,10 @@ struct WarpReplica {
         uint32_t tt;
         // Rounds done after slot 0 .. 3, measured per V: with all of them under the row
         // load N = 512 takes 0.608 instead of 0.562 us per step, with all of them before
-        // it 0.581 (fp32, 64 replicas).
-        static constexpr int kR0 = 5, kR1 = 6, kR2 = 7, kR3 = V == 8 || V == 32 ? 7 : 8;
+        // it 0.581 (fp32, 64 replicas); at V = 32 most of them belong before the choice
+        // (5, 6, 7, 7: 1.25 instead of 1.23 us at N = 1024 with 1024 replicas).
+        static constexpr int kR0 = V == 32 ? 7 : 5, kR1 = V == 32 ? 8 : 6, kR2 = V == 32 ? 8 : 7,
+                             kR3 = V == 32 ? 9 : 8;
         template <int I>
         __device__ __forceinline__ void at()
         {
@@ -436,11 +450,17 @@ struct WarpReplica {
         bool unsure;
         uint32_t accm = decide_log<A, V>(h, xm, Eoff, __fmul_rn(beta, kLog2e), L, unsure);
         const bool any_unsure = __any_sync(0xffffffffu, unsure);
+        // the rare exact test: at V = 32 before the count, below that after a first count
+        // whose votes overlap the vote on the band (one latency less; at V = 32 the second
+        // count's code costs more)
+        constexpr bool kFirst = V == 32;
+        if (kFirst && any_unsure)
+            accm = decide_exact<A, V>(h, xm, Eoff, beta, L, accm, base, (uint32_t)t, rep, keys);
         if constexpr (!FULL) accm &= valid;
         int excl, total;
         count_below(accm, excl, total);
         slots.template at<0>();
-        if (any_unsure) {   // rare: the exact test, and the counts again
+        if (!kFirst && any_unsure) {
             accm = decide_exact<A, V>(h, xm, Eoff, beta, L, accm, base, (uint32_t)t, rep, keys);
             if constexpr (!FULL) accm &= valid;
             count_below(accm, excl, total);
@@ -451,18 +471,30 @@ struct WarpReplica {
     // Accepted trials on the lanes below this one, and on all lanes: the bits of the
     // lanes' counts as votes, which are independent of one another (one latency of
     // about 20 cycles, then the population counts), beside the warp reduction of the
-    // total; a five-shuffle prefix sum is a chain of five 32-cycle latencies.  (The
-    // total from the votes as well: 1.275 against 1.253 us per step at N = 1024 with
-    // 1024 replicas, the population counts share a unit with the draws' log2.)
+    // total; a five-shuffle prefix sum is a chain of five 32-cycle latencies.  At V = 32
+    // the shuffles are used all the same: a population count takes 8 cycles of the unit
+    // that also makes the 32 log2 of the draws (8 cycles each), and with two warps per
+    // scheduler that counts for more than the chain (1.25 against 1.29 us per step at
+    // N = 1024 with 1024 replicas).
     __device__ __forceinline__ void count_below(uint32_t accm, int& excl, int& total) const
     {
-        constexpr int kBits = V == 4 ? 3 : V == 8 ? 4 : V == 16 ? 5 : 6;   // of a count 0 .. V
-        const uint32_t below = (1u << lane) - 1u;
         const int cnt = __popc(accm);
         total = (int)__reduce_add_sync(0xffffffffu, (unsigned)cnt);
-        excl = 0;
+        if constexpr (V == 32) {
+            int incl = cnt;
 #pragma unroll
-        for (int b = 0; b < kBits; ++b) excl += __popc(__ballot_sync(0xffffffffu, (cnt >> b) & 1) & below) << b;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += u;
+            }
+            excl = incl - cnt;
+        } else {
+            constexpr int kBits = V == 4 ? 3 : V == 8 ? 4 : 5;   // of a count 0 .. V
+            const uint32_t below = (1u << lane) - 1u;
+            excl = 0;
+#pragma unroll
+            for (int b = 0; b < kBits; ++b) excl += __popc(__ballot_sync(0xffffffffu, (cnt >> b) & 1) & below) << b;
+        }
     }
 
     // (c) of a step with acceptance mask accm (excl accepted trials on lower lanes,
@@ -513,7 +545,17 @@ struct WarpReplica {
         if (FULL || base < N) {
             const typename A::Sign sg = A::sign(xold);
 #pragma unroll
-            for (int v = 0; v < V; ++v) h[v] = A::apply_signed(h[v], cv[v], sg);
+            for (int v = 0; v < V; v += 2) {
+                if constexpr (sizeof(Tw) == 4 && V == 32) {   // packed: the same roundings, half the instructions
+                    const float* w = reinterpret_cast<const float*>(&cv[v]);
+                    const float2 u = __ffma2_rn(make_float2(sg, sg), make_float2(w[0], w[1]), make_float2(h[v], h[v + 1]));
+                    h[v] = u.x;
+                    h[v + 1] = u.y;
+                } else {
+                    h[v] = A::apply_signed(h[v], cv[v], sg);
+                    h[v + 1] = A::apply_signed(h[v + 1], cv[v + 1], sg);
+                }
+            }
         }
         if (lane == own) xm ^= 1u << vk;
         m = 0;
