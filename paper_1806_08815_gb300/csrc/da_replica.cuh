@@ -376,7 +376,8 @@ struct WarpReplica {
         __device__ __forceinline__ void rest_flip() { f(); }
         __device__ __forceinline__ void rest_none() { f(); }
     };
-    template <class Keys>
+    template <class Keys, int kR0 = V == 32 ? 7 : 5, int kR1 = V == 32 ? 8 : 6, int kR2 = V == 32 ? 8 : 7,
+              int kR3 = V == 32 ? 9 : 8>
     struct DrawSlots {     // the next step's draws (PRE)
         WarpReplica& rp;
         const Keys& keys;
@@ -385,8 +386,6 @@ struct WarpReplica {
         // load N = 512 takes 0.608 instead of 0.562 us per step, with all of them before
         // it 0.581 (fp32, 64 replicas); at V = 32 most of them belong before the choice
         // (5, 6, 7, 7: 1.25 instead of 1.23 us at N = 1024 with 1024 replicas).
-        static constexpr int kR0 = V == 32 ? 7 : 5, kR1 = V == 32 ? 8 : 6, kR2 = V == 32 ? 8 : 7,
-                             kR3 = V == 32 ? 9 : 8;
         template <int I>
         __device__ __forceinline__ void at()
         {

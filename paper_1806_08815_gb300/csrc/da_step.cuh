@@ -219,7 +219,11 @@ __global__ void __launch_bounds__(32 * G * OccupancyGV<G, V>::rpb, OccupancyGV<G
     for (uint32_t t = (uint32_t)p.t0; t < (uint32_t)p.t1; ++t) {
         int k;
         if constexpr (kPre) {
-            typename R_::template DrawSlots<PhiloxKeys> s{rp, keys, t + 1};
+            // where the draws' rounds go, measured: V <= 8 and V = 32 have the row load (and V = 32
+            // its HBM latency) to fill; N = 1024 (G = 4, V = 8) 0.637 -> 0.620 us per step, N = 4096
+            // (G = 8, V = 16) 1.048 -> 1.000, N = 8192 1.743 -> 1.606 against the one-warp split
+            constexpr int kR0 = V == 16 ? 5 : 3, kR1 = V == 16 ? 6 : 5, kR2 = V == 16 ? 7 : 5, kR3 = V == 16 && G < 8 ? 8 : 7;
+            typename R_::template DrawSlots<PhiloxKeys, kR0, kR1, kR2, kR3> s{rp, keys, t + 1};
             k = one_step(t, s);
         } else {
             auto f = [&] { rp.draw(t + 1, keys); };
