@@ -282,7 +282,7 @@ da_status check_kernel_flag(da_ctx* c)
     DA_CU(cudaMemcpy(&flag, c->tc.err, sizeof(int), cudaMemcpyDeviceToHost));
     if (flag) {
         DA_CU(cudaMemset(c->tc.err, 0, sizeof(int)));
-        return fail(DA_ETIMEOUT, flag == 2 ? "step kernel: a bounded wait on the draw ring gave up"
+        return fail(DA_ETIMEOUT, flag == 2 ? "step kernel: a bounded wait (draw ring, cluster) gave up"
                                            : "tensor-core recompute: a bounded wait on a pipeline barrier gave up");
     }
     return DA_OK;

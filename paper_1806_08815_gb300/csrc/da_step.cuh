@@ -33,6 +33,8 @@
 // Launches cover steps [t0, t1) and keep the state in global memory between
 // launches (the fp32 path recomputes the fields between launches).
 #pragma once
+#include <cstddef>
+
 #include "da_device.cuh"
 #include "da_internal.h"
 #include "da_replica.cuh"
@@ -79,12 +81,74 @@ template <> struct Published<8> {
 };
 template <> struct Published<4> : Published<8> {};
 
-template <typename E, int V, int G> struct GroupShared {
-    typename Published<V>::T lanes[2][32 * G];   // by step parity
-    alignas(16) int total[2][(G + 3) / 4 * 4];   // accepted trials of each warp, by step parity
+// Of the GA warps of a replica, G of them in this block.
+template <typename E, int V, int GA, int G> struct GroupShared {
+    uint64_t arrived[2];                         // clusters: a step's entries are here, by step parity
+    typename Published<V>::T lanes[2][32 * GA];  // by step parity
+    alignas(16) int total[2][(GA + 3) / 4 * 4];  // accepted trials of each warp, by step parity
     FlipEntry log[2][32];                        // by window parity
     FlipHead<E> head[G];
 };
+
+// ---- one replica on the blocks of a cluster ---------------------------------------
+// Every block of the cluster gets every warp's entries by asynchronous stores into its own
+// shared memory, which count their bytes on a barrier there: one way through the cluster
+// and no acknowledgement (stores followed by the cluster's barrier took 0.3 us longer per
+// step, reading the owner's entries from its block 0.35 us more again).
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t cluster_address(uint32_t shared_address, uint32_t rank)
+{
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(shared_address), "r"(rank));
+    return a;
+}
+// bar: the barrier in the block that a lies in
+__device__ __forceinline__ void cluster_send(uint32_t a, uint32_t v, uint32_t bar)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(a), "r"(v),
+                 "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void cluster_send(uint32_t a, uint2 v, uint32_t bar)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(a),
+                 "r"(v.x), "r"(v.y), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// A bounded wait for the phase of the given parity (tc::mbar_wait), acquiring what the
+// cluster's blocks stored.
+__device__ __forceinline__ bool cluster_try(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+constexpr uint32_t kClusterPolls = 1u << 26;
+constexpr uint64_t kClusterNs = 2000000000ull;
+__device__ __forceinline__ bool cluster_await(uint32_t bar, uint32_t parity)
+{
+    if (cluster_try(bar, parity)) return true;
+    const uint64_t t0 = tc::global_ns();
+    for (uint32_t i = 0; i < kClusterPolls; ++i) {
+        if (cluster_try(bar, parity)) return true;
+        if ((i & 255u) == 255u && tc::global_ns() - t0 > kClusterNs) return false;
+    }
+    return false;
+}
 
 // G > 1 warps per replica: warp w owns the slice [32 V w, 32 V (w + 1)) of the variables.
 // One barrier per step: every lane publishes its mask, state bits and in-warp prefix
@@ -93,32 +157,53 @@ template <typename E, int V, int G> struct GroupShared {
 // chain (one to two warps per scheduler).  us per step, fp32 with 32 replicas, against
 // the form in which every warp scanned all 32 G masks and booked the energy in fp64:
 // N = 1024 (G = 4, V = 8) 1.015 -> 0.611, N = 2048 (G = 4, V = 16) 1.168 -> 0.755,
-// N = 4096 (G = 8, V = 16) 1.564 -> 1.109, N = 8192 (G = 8, V = 32) 2.712 -> 1.758
-// (there the rows of W come from HBM).  16 warps per replica are no faster: N = 2048
-// 0.978, N = 4096 1.314, N = 8192 1.955.
-template <typename Tw, int V, int G, bool FULL, bool TRACE>
+// N = 4096 (G = 8, V = 16) 1.564 -> 1.000, N = 8192 (G = 8, V = 32) 2.712 -> 1.606
+// (there the rows of W come from HBM).  16 warps in one block are no faster: N = 2048
+// 0.978, N = 4096 1.314, N = 8192 1.955; on several SMs they are (kClusterReplicas).
+// C > 1: the replica on the C blocks of a cluster, G warps in each (warp w of block c is
+// warp c G + w); published to every block, the cluster's barrier in the place of the
+// block's.
+template <typename Tw, int V, int G, bool FULL, bool TRACE, int C = 1>
 __global__ void __launch_bounds__(32 * G * OccupancyGV<G, V>::rpb, OccupancyGV<G, V>::min_blocks)
     step_kernel(const __grid_constant__ StepParams p)
 {
     constexpr bool kCoal = sizeof(Tw) == 4 && V >= 8;   // fp32 forms: rows from p.Wc (step_uses_coal)
     constexpr int kRegCap = 65536 / (32 * G * OccupancyGV<G, V>::rpb * OccupancyGV<G, V>::min_blocks);
     constexpr bool kPre = kRegCap >= (V <= 8 ? 96 : V == 16 ? 128 : 255);
-    using R_ = WarpReplica<Tw, V, false, kPre, kCoal, (V * G < 32 ? V * G : 32)>;
+    constexpr int GA = G * C;                       // warps of the replica
+    using R_ = WarpReplica<Tw, V, false, kPre, kCoal, (V * GA < 32 ? V * GA : 32)>;
     using A = Arith<Tw>;
     using H = typename R_::H;
     using Pub = Published<V>;
-    __shared__ GroupShared<typename R_::E, V, G> shared[OccupancyGV<G, V>::rpb];
-    if (launch_stopped(p)) return;
+    using Shared = GroupShared<typename R_::E, V, GA, G>;
+    __shared__ Shared shared[C > 1 ? 1 : OccupancyGV<G, V>::rpb];
+    uint32_t rank = 0, peer[C];
+    if constexpr (C > 1) {
+        rank = cluster_rank();
+        if (threadIdx.x == 0) {
+            tc::mbar_init(&shared[0].arrived[0], 1);
+            tc::mbar_init(&shared[0].arrived[1], 1);
+            tc::mbar_init_fence();
+        }
+        __syncwarp();
+        cluster_arrive();                                // every block is there, its barriers initialised
+        cluster_wait();
+#pragma unroll
+        for (int c = 0; c < C; ++c) peer[c] = cluster_address((uint32_t)__cvta_generic_to_shared(&shared[0]), c);
+    } else {
+        if (launch_stopped(p)) return;
+    }
     const int wib = threadIdx.x >> 5;
-    const int g = wib / G;                          // group (replica) within the block
-    const int w = wib - g * G;                      // warp within the group
-    const int r = blockIdx.x * (blockDim.x / (32 * G)) + g;
+    const int g = C > 1 ? 0 : wib / G;              // group (replica) within the block
+    const int wb = wib - g * G;                     // warp of the group within the block
+    const int w = (int)rank * G + wb;               // and within the replica
+    const int r = C > 1 ? blockIdx.x / C : blockIdx.x * (blockDim.x / (32 * G)) + g;
     if (r >= p.R) return;
     auto& gs = shared[g];
 
     R_ rp;
     rp.init(static_cast<const Tw*>(kCoal ? p.Wc : p.W), p.N, kCoal ? p.npad : p.ldw, p.rep_base + (uint32_t)r,
-            p.bestx + (size_t)r * p.nw, gs.log[0], &gs.head[w], w * 32 * V);
+            p.bestx + (size_t)r * p.nw, gs.log[0], &gs.head[wb], w * 32 * V);
     const int lane = rp.lane;
     H* hg = static_cast<H*>(p.h) + (size_t)r * p.npad + rp.base;
     uint32_t* xg = p.x + (size_t)r * p.nw;
@@ -139,6 +224,15 @@ __global__ void __launch_bounds__(32 * G * OccupancyGV<G, V>::rpb, OccupancyGV<G
         if (p.t0 < p.t1) rp.draw((uint32_t)p.t0, keys);
     }
     int window = 0;
+    // clusters: the number of the step in the launch, its bytes beside the entries (the flip
+    // of the step before), whether a wait gave up
+    uint32_t sent = 0, extra = 0;
+    bool lost = false;
+    constexpr uint32_t kStepBytes = 32 * GA * sizeof(typename Pub::T) + GA * sizeof(int);
+    auto await_step = [&](uint32_t bytes) {
+        if (threadIdx.x == 0) tc::mbar_arrive_expect_tx(&gs.arrived[sent & 1], bytes);
+        return cluster_await((uint32_t)__cvta_generic_to_shared(&gs.arrived[sent & 1]), (sent >> 1) & 1);
+    };
 
     auto one_step = [&](uint32_t t, auto& slots) -> int {
         const float Eoff = __fmul_rn(__uint2float_rn(rp.m), p.inc);
@@ -148,15 +242,38 @@ __global__ void __launch_bounds__(32 * G * OccupancyGV<G, V>::rpb, OccupancyGV<G
         if constexpr (!FULL) accm &= rp.valid;
         int excl, mine;
         rp.count_below(accm, excl, mine);
-        slots.template at<0>();
+        if constexpr (C == 1) slots.template at<0>();
         if (any_unsure) {
             accm = decide_exact<A, V>(rp.h, rp.xm, Eoff, rp.beta, rp.lg, accm, rp.base, t, rp.rep, keys);
             if constexpr (!FULL) accm &= rp.valid;
             rp.count_below(accm, excl, mine);
         }
-        gs.lanes[t & 1][w * 32 + lane] = Pub::pack(accm, rp.xm, excl);
-        if (lane == 0) gs.total[t & 1][w] = mine;
-        group_barrier(1 + g, 32 * G);
+        if constexpr (C > 1) {
+            // buffers and barriers by the parity of `sent`; a buffer is free again when the
+            // step after it has arrived, for which every warp has left it
+            const uint32_t at_lane = (uint32_t)(offsetof(Shared, lanes) +
+                                                ((t & 1) * 32 * GA + w * 32 + lane) * sizeof(typename Pub::T));
+            const uint32_t at_total = (uint32_t)(offsetof(Shared, total) +
+                                                 ((t & 1) * ((GA + 3) / 4 * 4) + w) * sizeof(int));
+            const uint32_t at_bar = (uint32_t)(offsetof(Shared, arrived) + (sent & 1) * sizeof(uint64_t));
+            const typename Pub::T e = Pub::pack(accm, rp.xm, excl);
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                cluster_send(peer[c] + at_lane, e, peer[c] + at_bar);
+                if (lane == c) cluster_send(peer[c] + at_total, (uint32_t)mine, peer[c] + at_bar);
+            }
+            slots.template at<0>();
+            const bool ok = await_step(kStepBytes + extra);
+            ++sent;
+            if (!__all_sync(0xffffffffu, ok)) {
+                lost = true;
+                return -1;
+            }
+        } else {
+            gs.lanes[t & 1][w * 32 + lane] = Pub::pack(accm, rp.xm, excl);
+            if (lane == 0) gs.total[t & 1][w] = mine;
+            group_barrier(1 + g, 32 * G);
+        }
         // the flips up to the step before are in the log of every warp: settled here, by
         // every warp for its own words
         if (rp.n == 32) {
@@ -164,10 +281,10 @@ __global__ void __launch_bounds__(32 * G * OccupancyGV<G, V>::rpb, OccupancyGV<G
             window ^= 1;
             rp.log = gs.log[window];
         }
-        int before[G];                              // accepted trials on the warps below u
+        int before[GA];                             // accepted trials on the warps below u
         int total = 0;
 #pragma unroll
-        for (int u = 0; u < G; ++u) {
+        for (int u = 0; u < GA; ++u) {
             before[u] = total;
             total += gs.total[t & 1][u];
         }
@@ -180,7 +297,7 @@ __global__ void __launch_bounds__(32 * G * OccupancyGV<G, V>::rpb, OccupancyGV<G
         int j = (int)__umulhi(rp.cw, (uint32_t)total);
         int ow = 0, skip = 0;
 #pragma unroll
-        for (int u = 1; u < G; ++u)
+        for (int u = 1; u < GA; ++u)
             if (j >= before[u]) {
                 ow = u;
                 skip = before[u];
@@ -202,7 +319,18 @@ __global__ void __launch_bounds__(32 * G * OccupancyGV<G, V>::rpb, OccupancyGV<G
         const bool own = w * 32 + lane == ent;
         if (w == ow) {                              // warp-uniform
             const H gk = select_slot<H, V>(rp.h, vk);
-            if (own) rp.log[rp.n] = FlipEntry{A::log_bits(A::signed_field(gk, xold)), k};
+            const FlipEntry f{A::log_bits(A::signed_field(gk, xold)), k};
+            if constexpr (C > 1) {
+                const uint32_t at = (uint32_t)(offsetof(Shared, log) + (window * 32 + rp.n) * sizeof(FlipEntry));
+                if (own) {                          // counted with the next step
+                    const uint32_t at_bar = (uint32_t)(offsetof(Shared, arrived) + (sent & 1) * sizeof(uint64_t));
+#pragma unroll
+                    for (int c = 0; c < C; ++c)
+                        cluster_send(peer[c] + at, make_uint2(f.dE, (uint32_t)f.k), peer[c] + at_bar);
+                }
+            } else {
+                if (own) rp.log[rp.n] = f;
+            }
         }
         ++rp.n;
         slots.rest_flip();
@@ -221,8 +349,12 @@ __global__ void __launch_bounds__(32 * G * OccupancyGV<G, V>::rpb, OccupancyGV<G
         if constexpr (kPre) {
             // where the draws' rounds go, measured: V <= 8 and V = 32 have the row load (and V = 32
             // its HBM latency) to fill; N = 1024 (G = 4, V = 8) 0.637 -> 0.620 us per step, N = 4096
-            // (G = 8, V = 16) 1.048 -> 1.000, N = 8192 1.743 -> 1.606 against the one-warp split
-            constexpr int kR0 = V == 16 ? 5 : 3, kR1 = V == 16 ? 6 : 5, kR2 = V == 16 ? 7 : 5, kR3 = V == 16 && G < 8 ? 8 : 7;
+            // (G = 8, V = 16) 1.048 -> 1.000, N = 8192 1.743 -> 1.606 against the one-warp split;
+            // on clusters the wait for the other blocks takes the first two, at N = 8192 the rest
+            // belongs under the row load (1.406 -> 1.356)
+            constexpr bool kMid = V == 16 && C == 1;
+            constexpr int kR0 = V == 16 ? 5 : 3, kR1 = kMid ? 6 : 5, kR2 = kMid ? 7 : 5,
+                          kR3 = C > 1 && V == 16 ? 5 : kMid && G < 8 ? 8 : 7;
             typename R_::template DrawSlots<PhiloxKeys, kR0, kR1, kR2, kR3> s{rp, keys, t + 1};
             k = one_step(t, s);
         } else {
@@ -231,11 +363,25 @@ __global__ void __launch_bounds__(32 * G * OccupancyGV<G, V>::rpb, OccupancyGV<G
             k = one_step(t, s);
         }
         held = k >= 0;
+        if constexpr (C > 1) {
+            extra = held ? (uint32_t)sizeof(FlipEntry) : 0u;
+            if (lost) break;
+        }
         if constexpr (TRACE) {
             if (w == 0 && lane == 0) p.trace[(size_t)r * p.trace_T + t] = k;
         }
     }
-    group_barrier(1 + g, 32 * G);                   // the last flip is in the log
+    // the last flip is in the log
+    if constexpr (C > 1) {
+        if (!lost && !__all_sync(0xffffffffu, await_step(extra))) lost = true;
+        if (lost && lane == 0 && p.err) atomicExch(p.err, 2);
+        __syncwarp();
+        cluster_arrive();                           // no block leaves while another may still store to it
+        cluster_wait();
+        if (lost) return;
+    } else {
+        group_barrier(1 + g, 32 * G);
+    }
     if (rp.n > 0) rp.settle(held);
 
     rp.store_fields(hg);
@@ -428,6 +574,44 @@ inline void launch_shared(int blocks, int threads, size_t shm, cudaStream_t st, 
     if (blocks > 0) K<<<blocks, threads, shm, st>>>(p);
 }
 
+// One launch on clusters of C blocks per replica, G warps in each.
+template <auto K>
+inline cudaError_t launch_cluster(int C, int threads, cudaStream_t st, const StepParams& p)
+{
+    prefer_shared<K>();
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)p.R * C);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)C;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, K, p);
+}
+
+template <typename Tw, int V, int G, int C>
+cudaError_t launch_on_clusters(const StepParams& p, bool trace, cudaStream_t st)
+{
+    if (p.N == 32 * V * G * C)
+        return trace ? launch_cluster<step_kernel<Tw, V, G, true, true, C>>(C, 32 * G, st, p)
+                     : launch_cluster<step_kernel<Tw, V, G, true, false, C>>(C, 32 * G, st, p);
+    return trace ? launch_cluster<step_kernel<Tw, V, G, false, true, C>>(C, 32 * G, st, p)
+                 : launch_cluster<step_kernel<Tw, V, G, false, false, C>>(C, 32 * G, st, p);
+}
+
+// The replicas up to which the widest shapes (8 warps of V = 16 or 32, N > 2048) run on
+// clusters of 4 blocks of 4 warps with half the V, which spreads a replica's decisions,
+// draws and row over four SMs: as many as give every block an SM.  us per step at 32
+// replicas: N = 3000 int8 1.04 -> 0.91, N = 4096 fp32 1.00 -> 0.93, N = 8192 fp32 1.60 ->
+// 1.36, int16 1.65 -> 1.26; at 64 replicas, two blocks to an SM, N = 4096 1.00 -> 1.03 and
+// N = 8192 1.60 -> 1.56.  Not for the request loop's launches (those with a stop flag),
+// which run beside others: its burst of mixed requests ran at 2.9e11 trials/s with
+// clusters, 3.4e11 without.
+constexpr int kClusterReplicas = 38;
+
 template <typename Tw, int V, int G>
 cudaError_t launch_vg(const StepShape& s, const StepParams& p, bool trace, cudaStream_t st)
 {
@@ -457,6 +641,10 @@ cudaError_t launch_vg(const StepShape& s, const StepParams& p, bool trace, cudaS
         return cudaGetLastError();
     } else {
         if (blocks > 0 && sizeof(Tw) == 4 && V >= 8 && p.Wc == nullptr) return cudaErrorInvalidValue;
+        if constexpr (G == 8 && V >= 16) {
+            if (p.R > 0 && p.R <= kClusterReplicas && p.stop == nullptr)
+                return launch_on_clusters<Tw, V / 2, 4, 4>(p, trace, st);
+        }
         if (full) {
             if (trace) launch_shared<step_kernel<Tw, V, G, true, true>>(blocks, threads, 0, st, p);
             else launch_shared<step_kernel<Tw, V, G, true, false>>(blocks, threads, 0, st, p);

@@ -60,3 +60,29 @@ def test_tracked_energy_and_best_state_match_the_oracle(da, kind, N, shape, T, r
     assert np.array_equal(res["best_x"], ref["x_best"])
     assert np.array_equal(tracked, ref["E_final"])
     assert np.array_equal(best, ref["E_best"])
+
+
+@pytest.mark.parametrize("kind", ["int8", "sk", "mixed"])
+@pytest.mark.parametrize("N,shape,R", [(2049, (16, 8, 1), 5), (4096, (16, 8, 1), 3), (1100, (32, 8, 1), 4),
+                                       (4200, (32, 8, 1), 2), (2100, (16, 8, 1), 40)])
+def test_replicas_on_clusters_match_the_oracle(da, kind, N, shape, R):
+    """The widest shapes run few replicas on clusters of four blocks (the last case, with more
+    replicas, on one block each): tracked and best energies, states and flips, in two segments
+    whose cut falls inside a flip window."""
+    import oracle
+    T, rec = 151, 50
+    Q, scale = _instance(kind, N)
+    beta = (np.linspace(0.2, 6.0, T) / scale).astype(np.float32)
+    ctx = da.da_create(Q)
+    da.da_set_launch_shape(ctx, *shape)
+    _, ck = da.da_anneal_segment(ctx, beta, 0, 71, 0.25, R, 9, recompute_every=rec)
+    res, ck = da.da_anneal_segment(ctx, beta, 71, T, 0.25, R, 9, recompute_every=rec, checkpoint=ck)
+    n = min(R, 3)
+    ref = oracle.da_anneal(Q, beta, R=n, seed=9, inc=0.25, recompute_every=rec, nthreads=n)
+    assert np.array_equal(res["final_x"][:n], ref["x_final"])
+    assert np.array_equal(res["flips"][:n], ref["flips"])
+    assert np.array_equal(res["best_x"][:n], ref["x_best"])
+    bits = ck["scalars"] if kind == "int8" else ck["scalars"].view(np.float64)
+    assert np.array_equal(bits[:n, 0], ref["E_final"])
+    assert np.array_equal(bits[:n, 1], ref["E_best"])
+
