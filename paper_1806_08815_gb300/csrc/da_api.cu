@@ -53,7 +53,7 @@ struct da_ctx {
     int S = 0;  // fixed-point scale of the fp32 recompute
     int device = 0;
     void* W = nullptr;
-    void* Wf = nullptr;  // DA_INT8: the couplings as exact fp32, for the step kernel
+    void* Wf = nullptr;  // integer couplings as exact fp32, for the step kernel (HostInstance::exact_f32)
     void* Wc[9] = {};  // the step couplings in the warp row order, by log2(npad / 32) (step_uses_coal)
     void* diag = nullptr;
     da::TcOperand tc;  // digit planes of W for the tensor-core recompute
@@ -75,10 +75,11 @@ namespace {
 // Integer couplings (DA_INT8, DA_INT16): exact fields, exact int64 energies.
 bool is_int(const da_ctx* c) { return c->dtype != DA_FP32; }
 
-// The step kernel's coupling form: DA_INT8 contexts anneal on their couplings
+// The step kernel's coupling form: integer contexts whose fields and Delta E are exact in
+// fp32 (every DA_INT8 one, DA_INT16 ones by their row sums) anneal on their couplings
 // held as exact fp32 (the same values, FFMA updates, int64 energies).
-int step_wtype(const da_ctx* c) { return c->dtype == DA_INT8 ? da::kWInt8AsF32 : (int)c->dtype; }
-const void* step_W(const da_ctx* c) { return c->dtype == DA_INT8 ? c->Wf : c->W; }
+int step_wtype(const da_ctx* c) { return c->Wf ? da::kWInt8AsF32 : (int)c->dtype; }
+const void* step_W(const da_ctx* c) { return c->Wf ? c->Wf : c->W; }
 
 // Default launch shape by N and the replicas R: few replicas are bound by the latency of
 // a step, which more warps per replica shorten (each warp decides fewer trials, at the
@@ -259,7 +260,7 @@ StepParams base_params(const da_ctx* c, const RunBuffers& b)
 // linear terms and E = 0 (all runs start from the same state, Sec. II).
 da_status reset_state(const da_ctx* c, const RunBuffers& b, cudaStream_t st)
 {
-    DA_CU(da::launch_init_state(is_int(c), c->diag, c->N, b.R, b.h(), b.s.npad(), st, c->dtype == DA_INT8));
+    DA_CU(da::launch_init_state(is_int(c), c->diag, c->N, b.R, b.h(), b.s.npad(), st, c->Wf != nullptr));
     DA_CU(cudaMemsetAsync(b.x(), 0, (size_t)2 * b.R * b.s.nwords() * 4, st));
     DA_CU(cudaMemsetAsync(b.sc(), 0, b.zeroed_bytes(), st));
     return DA_OK;
@@ -360,7 +361,7 @@ namespace da {
 // Integer couplings: range of every coupling (upper triangle) and
 // |Q_ii| + sum_j |Q_ij| below row_limit; the rows are read in order.
 static bool check_integer(const int32_t* q, int n, int32_t lo, int32_t hi, long long row_limit, const char* name,
-                          std::string& why)
+                          long long& row_max, std::string& why)
 {
     std::vector<long long> rowabs(n, 0);
     for (int i = 0; i < n; ++i) {
@@ -381,6 +382,7 @@ static bool check_integer(const int32_t* q, int n, int32_t lo, int32_t hi, long 
             why = std::string(name) + " row " + std::to_string(i) + ": |Q_ii| + sum |Q_ij| too large for exact fields";
             return false;
         }
+    row_max = *std::max_element(rowabs.begin(), rowabs.end());
     return true;
 }
 
@@ -388,10 +390,17 @@ bool build_instance(const void* Q, int n, int dtype, HostInstance& out, std::str
 {
     out.ldw = (int)align_up((size_t)n, 128);
     out.S = 0;
+    long long row_max = 0;
     if (dtype == DA_INT8) {
-        if (!check_integer(static_cast<const int32_t*>(Q), n, -128, 127, 1ll << 24, "DA_INT8", why)) return false;
+        if (!check_integer(static_cast<const int32_t*>(Q), n, -128, 127, 1ll << 24, "DA_INT8", row_max, why))
+            return false;
+        out.exact_f32 = true;
     } else if (dtype == DA_INT16) {
-        if (!check_integer(static_cast<const int32_t*>(Q), n, -32767, 32767, 1ll << 31, "DA_INT16", why)) return false;
+        if (!check_integer(static_cast<const int32_t*>(Q), n, -32767, 32767, 1ll << 31, "DA_INT16", row_max, why))
+            return false;
+        // fp32 rows of twice the bytes: while they stay in L2 (64 MB at N = 4096) the fp32 form
+        // is the faster one, beyond that the int16 one (N = 8192: 1.26 against 1.36 us per step)
+        out.exact_f32 = row_max < (1ll << 24) && n <= 4096;
     } else {
         const float* q = static_cast<const float*>(Q);
         float amax = 0.f;
@@ -431,6 +440,8 @@ const void* ctx_coal_W(da_ctx* c, int V)
     if (!step_uses_coal(step_wtype(c), s) || ensure_coal(c, s) != DA_OK) return nullptr;
     return coal_slot(c, s);
 }
+
+int ctx_step_wtype(const da_ctx* c) { return step_wtype(c); }
 
 void ctx_device_view(const da_ctx* c, const void** W, const void** diag, int32_t* ldw, int32_t* S, const void** Wstep)
 {
@@ -480,12 +491,12 @@ da_status da_create(const void* Q, int64_t N, da_dtype dtype, da_ctx** out)
     if (e == cudaSuccess) e = cudaEventCreate(&c->ev0);
     if (e == cudaSuccess) e = cudaEventCreate(&c->ev1);
     if (e != cudaSuccess) return bail(DA_ECUDA, std::string("stream/event: ") + cudaGetErrorString(e));
-    // DA_INT8 also keeps its couplings as exact fp32, same pitch and slack
+    // exact integer instances also keep their couplings as fp32, same pitch and slack
     const size_t qbytes = (size_t)n * n * 4;
     void* qd = nullptr;
     e = da::dev_malloc(&c->W, da::instance_W_bytes(n, (int)dtype));
     if (e == cudaSuccess) e = da::dev_malloc(&c->diag, (size_t)n * 4);
-    if (e == cudaSuccess && dtype == DA_INT8) e = da::dev_malloc(&c->Wf, da::instance_W_bytes(n, DA_FP32));
+    if (e == cudaSuccess && hin.exact_f32) e = da::dev_malloc(&c->Wf, da::instance_W_bytes(n, DA_FP32));
     if (e == cudaSuccess) e = da::dev_malloc(&qd, qbytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -1047,7 +1058,7 @@ da_status restore_state(const da_ctx* c, const RunBuffers& b, const da_checkpoin
     DA_CU(cudaMemsetAsync(b.h(), 0, (size_t)R * npad * 4, st));
     DA_CU(cudaMemsetAsync(b.x(), 0, (size_t)2 * R * nw * 4, st));
     const void* fsrc = in->fields;
-    if (c->dtype == DA_INT8) {   // int32 fields, held as exact fp32 by the step kernel
+    if (c->Wf) {   // int32 fields, held as exact fp32 by the step kernel
         keep.emplace_back((size_t)R * N * 4);
         float* f = reinterpret_cast<float*>(keep.back().data());
         const int32_t* g = static_cast<const int32_t*>(in->fields);
@@ -1099,7 +1110,7 @@ da_status save_state(const da_ctx* c, const RunBuffers& b, da_checkpoint* out, c
 
 void finish_saved(const da_ctx* c, int R, da_checkpoint* out, const std::vector<char>* sc_bytes)
 {
-    if (out->fields && c->dtype == DA_INT8) {   // exact fp32 integers back to int32, in place
+    if (out->fields && c->Wf) {   // exact fp32 integers back to int32, in place
         char* p = static_cast<char*>(out->fields);
         for (size_t k = 0; k < (size_t)R * c->N; ++k) {
             float f;

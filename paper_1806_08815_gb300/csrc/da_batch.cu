@@ -508,7 +508,7 @@ extern "C" da_status da_batch_anneal(const da_batch_item* items, int32_t n, doub
         const void* W;       // couplings for the exact evaluation
         const void* Wstep;   // couplings in the step kernel's form (int8 instances: exact fp32)
         const void* Wc;      // the step couplings in the one-warp row order (fp32 forms, V >= 8), or null
-        int dtype;           // da_dtype of the instance
+        int wk;              // step coupling form (da_internal.h)
         const void* diag;
         int N, ldw, S;
         bool int8;
@@ -535,12 +535,12 @@ extern "C" da_status da_batch_anneal(const da_batch_item* items, int32_t n, doub
         h.ldw = ldw;
         h.S = S;
         h.int8 = dt != DA_FP32;   // integer couplings: exact fields and energies
-        h.dtype = (int)dt;
         int V = 4;
         while (32 * V < h.N) V *= 2;
         h.V = V;
         h.Wc = nullptr;
-        if ((dt == DA_FP32 || dt == DA_INT8) && V >= 8) {
+        h.wk = da::ctx_step_wtype(it.ctx);
+        if (h.wk != da::kWInt16 && V >= 8) {
             h.Wc = da::ctx_coal_W(it.ctx, V);
             if (!h.Wc) return bfail(DA_ENOMEM, "item " + std::to_string(i) + ": " + da_last_error());
         }
@@ -561,7 +561,7 @@ extern "C" da_status da_batch_anneal(const da_batch_item* items, int32_t n, doub
     }
     std::map<std::pair<int, int>, BatchClass> classes;
     for (int i = 0; i < n; ++i) {
-        const int wk = hi[i].dtype == DA_INT8 ? da::kWInt8AsF32 : hi[i].dtype;
+        const int wk = hi[i].wk;
         auto& c = classes[{wk, hi[i].V}];
         c.wk = wk;
         c.V = hi[i].V;
@@ -683,7 +683,7 @@ extern "C" da_status da_batch_anneal(const da_batch_item* items, int32_t n, doub
     for (auto& kv : classes) {
         BatchClass& c = kv.second;
         c.cfg = da::tune_class(c, reps[kv.first], dev, sms, st);
-        desc_text += std::string(desc_text.empty() ? "" : "; ") + (c.wk == da::kWFp32 ? "fp32" : c.wk == da::kWInt16 ? "int16" : "int8") + " V=" +
+        desc_text += std::string(desc_text.empty() ? "" : "; ") + (c.wk == da::kWFp32 ? "fp32" : c.wk == da::kWInt16 ? "int16" : "integer as fp32") + " V=" +
                      std::to_string(c.V) + " (N <= " + std::to_string(c.max_N) + ", " + std::to_string(c.n_items) +
                      " instances, " + std::to_string(c.units) + " replicas): " +
                      (c.cfg.smem ? "W staged in shared memory"

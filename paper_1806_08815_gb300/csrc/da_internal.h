@@ -11,8 +11,9 @@ struct da_ctx;
 namespace da {
 
 // Coupling types, with the values of da_dtype in include/da.h; kWInt8AsF32:
-// int8 couplings held as exact fp32 for the step kernel (int32-exact fields in
-// fp32, int64 energies), the form DA_INT8 contexts anneal with.
+// integer couplings held as exact fp32 for the step kernel (int32-exact fields in
+// fp32, int64 energies), the form DA_INT8 contexts anneal with, and DA_INT16 ones
+// whose |Q_ii| + sum_j |Q_ij| stay below 2^24.
 constexpr int kWInt8 = 0, kWFp32 = 1, kWInt16 = 2, kWInt8AsF32 = 3;
 
 // Per-replica scalars kept in global memory between kernel launches.
@@ -200,6 +201,7 @@ size_t plain_workspace_bytes(int N, int R);
 // otherwise).
 struct HostInstance {
     int ldw = 0, S = 0;
+    bool exact_f32 = false;   // integer couplings: the step may run on them as exact fp32 (kWInt8AsF32)
 };
 size_t instance_W_bytes(int n, int dtype);
 // Zeroes `bytes` bytes at p (device, 16-byte aligned) with a kernel of this
@@ -298,6 +300,8 @@ void set_last_error(const std::string& msg);
 // fp32, kWInt8AsF32; otherwise W).
 void ctx_device_view(const da_ctx* c, const void** W, const void** diag, int32_t* ldw, int32_t* S,
                      const void** Wstep = nullptr);
+// The step kernel's coupling form of the context (kWInt8AsF32, kWFp32, kWInt16).
+int ctx_step_wtype(const da_ctx* c);
 // The context's couplings in the one-warp row order for V variables per lane
 // (built on first use), or null when they cannot be made (da_last_error says why).
 const void* ctx_coal_W(da_ctx* c, int V);
