@@ -161,24 +161,29 @@ Layout plan(const da_ctx* c, const StepShape& s, int R, long long T, bool with_b
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes, 256); return at; };
     L.h = take((size_t)R * s.npad() * 4);
-    L.xs = take((size_t)2 * R * s.nwords() * 4);
-    L.sc = o;
+    // results, flag and states side by side, for one copy to the host; states, scalars and
+    // counters side by side, for one zeroing
+    L.res = take((size_t)4 * R * 8 + 8);
+    L.xs = o;
+    const size_t xs_end = o + align_up((size_t)2 * R * s.nwords() * 4, 32);
+    L.sc = xs_end;
     L.arrived = L.sc + (size_t)R * sizeof(ReplicaScalars);
-    take((size_t)R * sizeof(ReplicaScalars) + (size_t)((R + da::kTcStates - 1) / da::kTcStates) * sizeof(unsigned));
+    take(L.arrived - L.xs + (size_t)((2 * R + da::kTcStates - 1) / da::kTcStates) * sizeof(unsigned));
     L.sums = take(da::tc_partial_bytes(std::max(s.npad(), c->N), 2 * R));
     L.eex = take((size_t)2 * R * 8);
     L.beta = take(with_beta ? (size_t)T * 4 : 0);
-    L.res = take((size_t)4 * R * 8);
     L.trace = take(with_trace ? (size_t)R * T * 4 : 0);
     L.pt = take(pt_bytes);
     L.total = o;
     return L;
 }
 
+// flag_out (optional) receives the error flag err, so that one copy brings it along.
 __global__ void finalize_kernel(bool int8, int R, const ReplicaScalars* sc, const long long* eex, double* final_E,
-                                double* best_E, double* drift, int64_t* flips)
+                                double* best_E, double* drift, int64_t* flips, const int* err, int* flag_out)
 {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r == 0 && flag_out) *flag_out = *err;
     if (r >= R) return;
     double ef, eb, tracked;
     if (int8) {
@@ -205,7 +210,7 @@ struct RunBuffers {
     uint32_t* x() const { return reinterpret_cast<uint32_t*>(base + L.xs); }
     uint32_t* bestx() const { return x() + (size_t)R * s.nwords(); }
     ReplicaScalars* sc() const { return reinterpret_cast<ReplicaScalars*>(base + L.sc); }
-    size_t zeroed_bytes() const { return L.sums - L.sc; }   // sc and the counters
+    size_t zeroed_bytes() const { return L.sums - L.xs; }   // x, sc and the counters
     unsigned* arrived() const { return reinterpret_cast<unsigned*>(base + L.arrived); }
     long long* sums() const { return reinterpret_cast<long long*>(base + L.sums); }
     long long* eex() const { return reinterpret_cast<long long*>(base + L.eex); }
@@ -261,8 +266,7 @@ StepParams base_params(const da_ctx* c, const RunBuffers& b)
 da_status reset_state(const da_ctx* c, const RunBuffers& b, cudaStream_t st)
 {
     DA_CU(da::launch_init_state(is_int(c), c->diag, c->N, b.R, b.h(), b.s.npad(), st, c->Wf != nullptr));
-    DA_CU(cudaMemsetAsync(b.x(), 0, (size_t)2 * b.R * b.s.nwords() * 4, st));
-    DA_CU(cudaMemsetAsync(b.sc(), 0, b.zeroed_bytes(), st));
+    DA_CU(cudaMemsetAsync(b.x(), 0, b.zeroed_bytes(), st));
     return DA_OK;
 }
 
@@ -270,23 +274,62 @@ da_status reset_state(const da_ctx* c, const RunBuffers& b, cudaStream_t st)
 da_status evaluate(const da_ctx* c, const RunBuffers& b, cudaStream_t st)
 {
     DA_CU(da::launch_recompute_tc(is_int(c), c->tc, c->diag, c->N, c->S, b.x(), b.s.nwords(), 2 * b.R, nullptr,
-                                  b.s.npad(), b.eex(), 1, st, b.sums()));
+                                  b.s.npad(), b.eex(), 1, st, b.sums(), b.arrived()));
     return DA_OK;
 }
 
 // After a call's stream work has completed: a bounded wait inside a kernel
 // (the tensor-core recompute's pipeline, the step's producer/annealer
 // handshake) that gave up invalidates the call's results.
+da_status report_flag(da_ctx* c, int flag)
+{
+    if (!flag) return DA_OK;
+    DA_CU(cudaMemset(c->tc.err, 0, sizeof(int)));
+    return fail(DA_ETIMEOUT, flag == 2 ? "step kernel: a bounded wait (draw ring, cluster) gave up"
+                                       : "tensor-core recompute: a bounded wait on a pipeline barrier gave up");
+}
+
 da_status check_kernel_flag(da_ctx* c)
 {
     int flag = 0;
     DA_CU(cudaMemcpy(&flag, c->tc.err, sizeof(int), cudaMemcpyDeviceToHost));
-    if (flag) {
-        DA_CU(cudaMemset(c->tc.err, 0, sizeof(int)));
-        return fail(DA_ETIMEOUT, flag == 2 ? "step kernel: a bounded wait (draw ring, cluster) gave up"
-                                           : "tensor-core recompute: a bounded wait on a pipeline barrier gave up");
-    }
+    return report_flag(c, flag);
+}
+
+// The final results of an anneal: energies, drift, flips and the error flag into the block
+// in front of the states ...
+da_status finalize(const da_ctx* c, const RunBuffers& b, cudaStream_t st)
+{
+    double* res = reinterpret_cast<double*>(b.base + b.L.res);
+    const int R = b.R;
+    finalize_kernel<<<(R + 127) / 128, 128, 0, st>>>(is_int(c), R, b.sc(), b.eex(), res, res + R, res + 2 * R,
+                                                     reinterpret_cast<int64_t*>(res + 3 * R), c->tc.err,
+                                                     reinterpret_cast<int*>(res + 4 * R));
+    DA_CU(cudaGetLastError());
     return DA_OK;
+}
+
+// ... and, after `host` = that block and the states have arrived, out of it into `out`.  One
+// copy of all of it: every copy to pageable memory is a round trip of about 10 us, and the
+// three arrays, the flag and the scalars were five of them.
+size_t result_bytes(const RunBuffers& b) { return b.L.sc - b.L.res; }
+
+void unpack_results(const da_ctx* c, const RunBuffers& b, const char* host, da_result* out)
+{
+    const int R = b.R;
+    const size_t words = (size_t)da_words(c->N), nw = (size_t)b.s.nwords();
+    const size_t r8 = (size_t)R * 8;
+    if (out->final_E) std::memcpy(out->final_E, host, r8);
+    if (out->best_E) std::memcpy(out->best_E, host + r8, r8);
+    if (out->max_drift) std::memcpy(out->max_drift, host + 2 * r8, r8);
+    if (out->flips) std::memcpy(out->flips, host + 3 * r8, r8);
+    const char* xs = host + (b.L.xs - b.L.res);
+    for (int k = 0; k < 2; ++k) {
+        uint32_t* dst = k ? out->best_x : out->final_x;
+        if (!dst) continue;
+        for (int r = 0; r < R; ++r)
+            std::memcpy(dst + (size_t)r * words, xs + ((size_t)k * R + r) * nw * 4, words * 4);
+    }
 }
 
 // Next free pair of profiling events (created on first use).
@@ -358,31 +401,53 @@ struct CtxLock {
 }  // namespace
 
 namespace da {
+// The checks read the upper triangle once, in pieces that stay in the L1 cache, with loops
+// the compiler turns into vector code (no exit from inside a piece; a bad entry is looked
+// for again afterwards).  Entry by entry they took 8.7 of the 9.6 ms of creating an
+// N = 3000 integer instance, 1.8 as written.
+constexpr int kPiece = 2048;
+
 // Integer couplings: range of every coupling (upper triangle) and
 // |Q_ii| + sum_j |Q_ij| below row_limit; the rows are read in order.
 static bool check_integer(const int32_t* q, int n, int32_t lo, int32_t hi, long long row_limit, const char* name,
                           long long& row_max, std::string& why)
 {
-    std::vector<long long> rowabs(n, 0);
+    std::vector<int32_t> sums(n, 0);   // of |Q_ij| over the couplings: below 2^28 once in range
     for (int i = 0; i < n; ++i) {
-        rowabs[i] += std::llabs((long long)q[(size_t)i * n + i]);
-        for (int j = i + 1; j < n; ++j) {
-            const int32_t v = q[(size_t)i * n + j];
-            if (v < lo || v > hi) {
+        const int32_t* row = q + (size_t)i * n;
+        int32_t mine = 0;
+        for (int j0 = i + 1; j0 < n; j0 += kPiece) {
+            const int j1 = std::min(n, j0 + kPiece);
+            int32_t least = 0, most = 0;
+            for (int j = j0; j < j1; ++j) {
+                least = std::min(least, row[j]);
+                most = std::max(most, row[j]);
+            }
+            if (least < lo || most > hi) {
+                int j = j0;
+                while (row[j] >= lo && row[j] <= hi) ++j;
                 why = std::string(name) + " coupling Q[" + std::to_string(i) + "][" + std::to_string(j) + "] = " +
-                      std::to_string(v) + " outside [" + std::to_string(lo) + ", " + std::to_string(hi) + "]";
+                      std::to_string(row[j]) + " outside [" + std::to_string(lo) + ", " + std::to_string(hi) + "]";
                 return false;
             }
-            rowabs[i] += std::abs(v);
-            rowabs[j] += std::abs(v);
+            int32_t* __restrict__ s = sums.data();
+            for (int j = j0; j < j1; ++j) {
+                const int32_t a = row[j] < 0 ? -row[j] : row[j];
+                mine += a;
+                s[j] += a;
+            }
         }
+        sums[i] += mine;
     }
-    for (int i = 0; i < n; ++i)
-        if (rowabs[i] >= row_limit) {
+    row_max = 0;
+    for (int i = 0; i < n; ++i) {
+        const long long sum = std::llabs((long long)q[(size_t)i * n + i]) + sums[i];
+        if (sum >= row_limit) {
             why = std::string(name) + " row " + std::to_string(i) + ": |Q_ii| + sum |Q_ij| too large for exact fields";
             return false;
         }
-    row_max = *std::max_element(rowabs.begin(), rowabs.end());
+        row_max = std::max(row_max, sum);
+    }
     return true;
 }
 
@@ -402,17 +467,25 @@ bool build_instance(const void* Q, int n, int dtype, HostInstance& out, std::str
         // is the faster one, beyond that the int16 one (N = 8192: 1.26 against 1.36 us per step)
         out.exact_f32 = row_max < (1ll << 24) && n <= 4096;
     } else {
-        const float* q = static_cast<const float*>(Q);
-        float amax = 0.f;
-        for (int i = 0; i < n; ++i)
+        // the bits of |v| order as |v| does, infinities and NaN above every finite value
+        const char* q = static_cast<const char*>(Q);
+        uint32_t most = 0;
+        for (int i = 0; i < n; ++i) {
+            const char* row = q + (size_t)i * n * 4;
+            uint32_t m = 0;
             for (int j = i; j < n; ++j) {
-                const float v = q[(size_t)i * n + j];
-                if (!std::isfinite(v)) {
-                    why = "non-finite Q entry";
-                    return false;
-                }
-                amax = std::max(amax, std::fabs(v));
+                uint32_t b;
+                std::memcpy(&b, row + (size_t)j * 4, 4);
+                m = std::max(m, b & 0x7FFFFFFFu);
             }
+            if (m >= 0x7F800000u) {
+                why = "non-finite Q entry";
+                return false;
+            }
+            most = std::max(most, m);
+        }
+        float amax;
+        std::memcpy(&amax, &most, 4);
         out.S = fix_scale(amax, n);
     }
     return true;
@@ -642,37 +715,24 @@ da_status da_anneal(da_ctx* c, const float* beta, int64_t steps, float inc, int3
     DA_CU(cudaEventRecord(c->ev0, st));
     RunBuffers b{};
     if (da_status e = anneal_common(c, beta, true, steps, inc, R, seed, recompute_every, want_trace, st, &b)) return e;
-    double* res = reinterpret_cast<double*>(b.base + b.L.res);
-    finalize_kernel<<<(R + 127) / 128, 128, 0, st>>>(is_int(c), R, b.sc(), b.eex(), res, res + R, res + 2 * R,
-                                                     reinterpret_cast<int64_t*>(res + 3 * R));
-    DA_CU(cudaGetLastError());
+    if (da_status e = finalize(c, b, st)) return e;
     DA_CU(cudaEventRecord(c->ev1, st));
     if (!out) {
         DA_CU(cudaStreamSynchronize(st));
         return check_kernel_flag(c);
     }
-    const size_t words = (size_t)da_words(c->N);
-    std::vector<double> hres((size_t)4 * R);
-    DA_CU(cudaMemcpyAsync(hres.data(), res, hres.size() * 8, cudaMemcpyDeviceToHost, st));
-    if (out->final_x)
-        DA_CU(cudaMemcpy2DAsync(out->final_x, words * 4, b.x(), (size_t)b.s.nwords() * 4, words * 4, R,
-                                cudaMemcpyDeviceToHost, st));
-    if (out->best_x)
-        DA_CU(cudaMemcpy2DAsync(out->best_x, words * 4, b.bestx(), (size_t)b.s.nwords() * 4, words * 4, R,
-                                cudaMemcpyDeviceToHost, st));
+    std::vector<char> host(result_bytes(b));
+    DA_CU(cudaMemcpyAsync(host.data(), b.base + b.L.res, host.size(), cudaMemcpyDeviceToHost, st));
     if (want_trace && steps > 0)
         DA_CU(cudaMemcpyAsync(out->trace, b.base + b.L.trace, (size_t)R * steps * 4, cudaMemcpyDeviceToHost, st));
     DA_CU(cudaStreamSynchronize(st));
-    if (da_status e = check_kernel_flag(c)) return e;
+    int flag;
+    std::memcpy(&flag, host.data() + (size_t)4 * R * 8, sizeof(int));
+    if (da_status e = report_flag(c, flag)) return e;
     float ms = 0.f;
     DA_CU(cudaEventElapsedTime(&ms, c->ev0, c->ev1));
     out->elapsed_s = ms * 1e-3;
-    for (int r = 0; r < R; ++r) {
-        if (out->final_E) out->final_E[r] = hres[r];
-        if (out->best_E) out->best_E[r] = hres[R + r];
-        if (out->max_drift) out->max_drift[r] = hres[2 * R + r];
-        if (out->flips) out->flips[r] = reinterpret_cast<const int64_t*>(hres.data() + 3 * R)[r];
-    }
+    unpack_results(c, b, host.data(), out);
     return DA_OK;
 }
 
@@ -689,7 +749,7 @@ da_status da_anneal_async(da_ctx* c, const float* beta_dev, int64_t steps, float
         return e;
     if (!out) return DA_OK;
     finalize_kernel<<<(R + 127) / 128, 128, 0, st>>>(is_int(c), R, b.sc(), b.eex(), out->final_E, out->best_E,
-                                                     out->max_drift, out->flips);
+                                                     out->max_drift, out->flips, nullptr, nullptr);
     DA_CU(cudaGetLastError());
     const size_t words = (size_t)da_words(c->N);
     if (out->final_x)
@@ -1056,7 +1116,7 @@ da_status restore_state(const da_ctx* c, const RunBuffers& b, const da_checkpoin
     const int R = b.R, N = c->N, npad = b.s.npad(), nw = b.s.nwords();
     const size_t words = (size_t)da_words(N);
     DA_CU(cudaMemsetAsync(b.h(), 0, (size_t)R * npad * 4, st));
-    DA_CU(cudaMemsetAsync(b.x(), 0, (size_t)2 * R * nw * 4, st));
+    DA_CU(cudaMemsetAsync(b.x(), 0, b.zeroed_bytes(), st));
     const void* fsrc = in->fields;
     if (c->Wf) {   // int32 fields, held as exact fp32 by the step kernel
         keep.emplace_back((size_t)R * N * 4);
@@ -1079,7 +1139,6 @@ da_status restore_state(const da_ctx* c, const RunBuffers& b, const da_checkpoin
         sc[r].m = (uint32_t)in->scalars[4 * r + 3];
         sc[r].check = 0;
     }
-    DA_CU(cudaMemsetAsync(b.sc(), 0, b.zeroed_bytes(), st));   // the counters
     DA_CU(cudaMemcpyAsync(b.sc(), sc, (size_t)R * sizeof(ReplicaScalars), cudaMemcpyHostToDevice, st));
     return DA_OK;
 }
@@ -1166,36 +1225,23 @@ extern "C" da_status da_anneal_segment(da_ctx* c, const float* beta, int64_t tot
     }
     if (da_status e = run_anneal(c, b, beta_dev, t0, t1, inc, seed, recompute_every, nullptr, st)) return e;
     if (da_status e = evaluate(c, b, st)) return e;
-    double* resd = reinterpret_cast<double*>(b.base + L.res);
-    finalize_kernel<<<(R + 127) / 128, 128, 0, st>>>(is_int(c), R, b.sc(), b.eex(), resd, resd + R, resd + 2 * R,
-                                                     reinterpret_cast<int64_t*>(resd + 3 * R));
-    DA_CU(cudaGetLastError());
+    if (da_status e = finalize(c, b, st)) return e;
     DA_CU(cudaEventRecord(c->ev1, st));
-    std::vector<double> hres((size_t)4 * R);
-    DA_CU(cudaMemcpyAsync(hres.data(), resd, hres.size() * 8, cudaMemcpyDeviceToHost, st));
-    const size_t words = (size_t)da_words(c->N);
-    if (res && res->final_x)
-        DA_CU(cudaMemcpy2DAsync(res->final_x, words * 4, b.x(), (size_t)s.nwords() * 4, words * 4, R,
-                                cudaMemcpyDeviceToHost, st));
-    if (res && res->best_x)
-        DA_CU(cudaMemcpy2DAsync(res->best_x, words * 4, b.bestx(), (size_t)s.nwords() * 4, words * 4, R,
-                                cudaMemcpyDeviceToHost, st));
+    std::vector<char> host(result_bytes(b));
+    DA_CU(cudaMemcpyAsync(host.data(), b.base + b.L.res, host.size(), cudaMemcpyDeviceToHost, st));
     const size_t sc_idx = keep.size();
     if (out)
         if (da_status e = save_state(c, b, out, st, keep)) return e;
     DA_CU(cudaStreamSynchronize(st));
-    if (da_status e = check_kernel_flag(c)) return e;
+    int flag;
+    std::memcpy(&flag, host.data() + (size_t)4 * R * 8, sizeof(int));
+    if (da_status e = report_flag(c, flag)) return e;
     if (out) finish_saved(c, R, out, out->scalars ? &keep[sc_idx] : nullptr);
     if (res) {
         float ms = 0.f;
         DA_CU(cudaEventElapsedTime(&ms, c->ev0, c->ev1));
         res->elapsed_s = ms * 1e-3;
-        for (int r = 0; r < R; ++r) {
-            if (res->final_E) res->final_E[r] = hres[r];
-            if (res->best_E) res->best_E[r] = hres[R + r];
-            if (res->max_drift) res->max_drift[r] = hres[2 * R + r];
-            if (res->flips) res->flips[r] = reinterpret_cast<const int64_t*>(hres.data() + 3 * R)[r];
-        }
+        unpack_results(c, b, host.data(), res);
     }
     return DA_OK;
 }
