@@ -41,8 +41,8 @@ C3 = dict(N=1024, replicas=1024, steps=200_000, recompute_every=1024, beta0=0.1,
 # capture of the headline workload, valid while the kernel source has the recorded hash.
 # Warp instructions per replica-step of the step kernel (smsp__inst_executed.sum / (R x steps))
 # from the same capture: the issue-slot roofline of a kernel bound by instruction issue.
-STEP_INST_PER_REPLICA_STEP = 650.2
-STEP_TRAFFIC = {"source_sha256_16": "09fc783acf24a84b", "bytes_per_launch": 8.6162e6}
+STEP_INST_PER_REPLICA_STEP = 636.8
+STEP_TRAFFIC = {"source_sha256_16": "3b34819b0d1a21a9", "bytes_per_launch": 8.6244e6}
 
 
 def step_source_sha():

@@ -123,7 +123,14 @@ struct WarpReplica {
     template <class Keys>
     __device__ __forceinline__ void fill_choice(long long t, const Keys& keys)
     {
-        cr = philox4x32_10(0u, (uint32_t)((t & ~127ll) + 4 * lane), rep, 1u, keys);
+        const uint32_t c = (uint32_t)((t & ~127ll) + 4 * lane);
+        if constexpr (kRareOutOfLine<V>) cr = choice_block(c, rep, keys);
+        else cr = philox4x32_10(0u, c, rep, 1u, keys);
+    }
+    template <class Keys>
+    static __device__ __noinline__ u32x4 choice_block(uint32_t c, uint32_t rep, const Keys& keys)
+    {
+        return philox4x32_10(0u, c, rep, 1u, keys);
     }
     __device__ __forceinline__ uint32_t choice_word(uint32_t t) const
     {
@@ -454,13 +461,13 @@ struct WarpReplica {
         // count's code costs more)
         constexpr bool kFirst = V == 32;
         if (kFirst && any_unsure)
-            accm = decide_exact<A, V>(h, xm, Eoff, beta, L, accm, base, (uint32_t)t, rep, keys);
+            accm = decide_exact_out<A, V>(h, xm, Eoff, beta, L, accm, base, (uint32_t)t, rep, keys);
         if constexpr (!FULL) accm &= valid;
         int excl, total;
         count_below(accm, excl, total);
         slots.template at<0>();
         if (!kFirst && any_unsure) {
-            accm = decide_exact<A, V>(h, xm, Eoff, beta, L, accm, base, (uint32_t)t, rep, keys);
+            accm = decide_exact_out<A, V>(h, xm, Eoff, beta, L, accm, base, (uint32_t)t, rep, keys);
             if constexpr (!FULL) accm &= valid;
             count_below(accm, excl, total);
         }

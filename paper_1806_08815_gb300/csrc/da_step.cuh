@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(32 * G * OccupancyGV<G, V>::rpb, OccupancyGV<G
         rp.count_below(accm, excl, mine);
         if constexpr (C == 1) slots.template at<0>();
         if (any_unsure) {
-            accm = decide_exact<A, V>(rp.h, rp.xm, Eoff, rp.beta, rp.lg, accm, rp.base, t, rp.rep, keys);
+            accm = decide_exact_out<A, V>(rp.h, rp.xm, Eoff, rp.beta, rp.lg, accm, rp.base, t, rp.rep, keys);
             if constexpr (!FULL) accm &= rp.valid;
             rp.count_below(accm, excl, mine);
         }
