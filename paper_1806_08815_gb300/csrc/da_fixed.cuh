@@ -71,7 +71,7 @@ __device__ __forceinline__ long long energy_of_sum(unsigned long long lo, long l
     }
 }
 
-// The integer value of an fp32 that holds an integer of magnitude < 2^22
+// The integer value of an fp32 that holds an integer in [-2^22, 2^22)
 // (the tensor cores' digit sums): adding 1.5 2^23 puts it in the mantissa.
 __device__ __forceinline__ int small_int_of(float f)
 {

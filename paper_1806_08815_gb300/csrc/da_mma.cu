@@ -9,7 +9,7 @@
 // the same integers: v is split into balanced digits of b bits,
 //   v = sum_l d_l 2^(b l),   d_l in [-2^(b-1), 2^(b-1)),
 // every digit is exact in fp16 (|d| <= 2048), and b is chosen so that no
-// partial sum of digits over the K side exceeds 2^21 in magnitude, far inside
+// partial sum of digits over the K side exceeds 2^22 in magnitude, inside
 // the 24-bit integer range of the fp32 accumulator.  Each digit plane is one
 // accumulator in tensor memory; the epilogue combines the planes in 64-bit
 // integers, adds the fixed-point diagonal and rounds once, exactly like the
@@ -447,8 +447,10 @@ void tc_digits(int wtype, int N, int* bits, int* limbs)
         *limbs = 1;
         return;
     }
-    // |partial sum| <= 2^(b-1) * N <= 2^21
-    const int b = std::min(12, 22 - ceil_log2(std::max(N, 2)));
+    // -2^22 <= partial sum < 2^22 (digits -2^(b-1) .. 2^(b-1) - 1), the range of small_int_of.
+    // At half of it N = 4096 and 8192 need a sixth plane: 805 instead of 671 MB to stream at
+    // N = 8192.
+    const int b = std::min(12, 23 - ceil_log2(std::max(N, 2)));
     *bits = b;
     if (wtype == kWInt16) {  // |v| <= 2^15 - 1 needs b * limbs >= 17
         *limbs = (17 + b - 1) / b;
