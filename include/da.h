@@ -154,9 +154,9 @@ da_status da_ctx_info(const da_ctx* ctx, int64_t* N, da_dtype* dtype);
 
 /* Fix the launch shape of the step kernel for this context instead of the
  * automatic choice: a group of G warps per replica, V variables per lane
- * (32 * V * G >= N), rpb replicas per thread block.  Supported: G = 1 or 2
- * with V in {4, 8, 16, 32}; G = 4 with V in {4, 8, 16}; G = 8 with V in
- * {8, 16, 32}; rpb <= 4 (G = 1), <= 2 (G = 2), = 1 (G = 4, 8).  V = 0
+ * (32 * V * G >= N), rpb replicas per thread block.  Supported: G = 1, 2 or 4
+ * with V in {4, 8, 16, 32}; G = 8 with V in {8, 16, 32}; rpb <= 4 (G = 1),
+ * <= 2 (G = 2), = 1 (G = 4, 8).  V = 0
  * restores the automatic choice.  Results do
  * not depend on the shape (the random numbers are keyed by variable index,
  * step and replica).  Errors: DA_EINVAL. */
@@ -175,7 +175,7 @@ da_status da_set_launch_shape(da_ctx* ctx, int32_t V, int32_t G, int32_t rpb);
 da_status da_tune_shape(da_ctx* ctx, int32_t replicas, int64_t probe_steps, int32_t* V, int32_t* G, int32_t* rpb,
                         int32_t* draw_warp);
 
-/* For shapes with G = 1 (the automatic choice up to N = 1024): on = 1 runs
+/* For shapes with G = 1 (with on = 1 also the automatic choice up to N = 1024): on = 1 runs
  * each replica as an annealer warp plus a producer warp that computes the
  * acceptance draws of the coming steps (Philox words as log2 u) into shared
  * memory, one replica per block, rpb ignored; on = 0 (the default) lets the
@@ -271,7 +271,8 @@ typedef struct da_batch_item {
 /* Anneal many instances of different sizes and coupling types together: every
  * replica of every item is one work unit, and warps of one persistent kernel per
  * (coupling type, size class) pull units from a device queue until none are left;
- * all launches and the exact final evaluation form one CUDA graph.  Each item's
+ * the classes run side by side as branches of one CUDA graph with the exact final
+ * evaluation at its end.  Each item's
  * results are identical to da_anneal on that item alone (the random numbers are
  * keyed by the item's seed and replica index).  Each class's configuration is
  * chosen by an autotuner that times short probes (1024 steps) of the class's own

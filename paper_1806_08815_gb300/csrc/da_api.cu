@@ -2,12 +2,16 @@
 // asynchronous anneal, PTDA, exact energies and the field recompute.
 //
 // Runtime layout in HBM (per call, in the context's workspace):
-//   h      [R][npad]   int32 / fp32 fields between step launches
-//   xs     [2R][nw]    current states, then best states (adjacent, so the
-//                      final exact evaluation treats them as 2R states)
-//   sc     [R]         ReplicaScalars (tracked E, best E, flips, offset count)
-//   sums   [N/64][2R] 128-bit partial energies of the exact recompute
-//   E_ex   [2R]        exact energies of the final and best states
+//   h       [R][npad]  int32 / fp32 fields between step launches
+//   res     [4R + 1]   results of the call and its error flag, then
+//   xs      [2R][nw]   current states, then best states (adjacent, so the
+//                      final exact evaluation treats them as 2R states; with
+//                      the results before them, one copy to the host), then
+//   sc      [R]        ReplicaScalars (tracked E, best E, flips, offset count), then
+//   arrived            the fused recompute's counters (states, scalars and
+//                      counters are zeroed together)
+//   sums    [N/64][2R] 128-bit partial energies of the exact recompute
+//   E_ex    [2R]       exact energies of the final and best states
 // The instance itself (symmetric W with row pitch ldw, and diag) lives in the
 // context for its whole life.
 #include <algorithm>

@@ -28,7 +28,7 @@ struct alignas(32) ReplicaScalars {
 
 // Launch shape of the parallel-trial step: a group of G warps per replica,
 // V variables per lane, so one replica spans Npad = 32 * V * G variables;
-// lane l of warp w owns i = w*32V + 32v + l (v < V).
+// lane l of warp w owns i = w*32V + l*V + v (v < V).
 struct StepShape {
     int V = 0;
     int G = 0;

@@ -14,21 +14,21 @@
 //       hardware log2 of the draw; trials with |t| within a band of 2^-15,
 //       wider than the error of that estimate, take the exact test with the
 //       library's exponential instead, so every decision equals the exact one;
-//   (c) each lane's acceptance bits are already in index order, so a warp
-//       prefix sum of their popcounts locates the j-th accepted variable,
-//       j = floor(u * count); the chosen x_k flips while every lane adds
-//       +-W[k][i] (16-byte loads of row k, which equals column k, from L2; the
-//       fp32 forms read a copy of W in the warp row order, where each load of a
-//       warp covers 512 contiguous bytes) to its fields.  The next step's
-//       Philox words are computed while that row is in flight.  E_off returns
-//       to 0 on a flip and grows by inc otherwise.
-// A G = 1 group needs no shared memory or barrier.  A G > 1 group publishes
-// its lanes' acceptance and state masks in shared memory behind one named
-// barrier per step; the energy of step t is booked after the barrier of step
-// t + 1, while x still holds the state right after step t.  The best-state
-// test of a launch's last step is left pending (ReplicaScalars::check) so that
-// it sees the energy after any recompute between launches, as Algorithm 2's
-// result is defined after each complete step.
+//   (c) each lane's acceptance bits are already in index order, so the counts of
+//       the lanes below (from votes; shuffles at V = 32) locate the j-th accepted
+//       variable, j = floor(u * count); the chosen x_k flips while every lane
+//       adds +-W[k][i] (16-byte loads of row k, which equals column k, from L2;
+//       the fp32 forms read a copy of W in the warp row order, where each load
+//       of a warp covers 512 contiguous bytes) to its fields.  The next step's
+//       Philox words are computed in the latency of the votes and of that row.
+//       E_off returns to 0 on a flip and grows by inc otherwise.
+// The energy and the best state are not touched by a step: it appends the flip
+// to a log in shared memory, settled 32 flips at a time (settle_log).  A G = 1
+// group needs no barrier.  A G > 1 group publishes its lanes' acceptance and
+// state masks in shared memory behind one named barrier per step.  The
+// best-state test of a launch's last step is left pending
+// (ReplicaScalars::check) so that it sees the energy after any recompute
+// between launches, as Algorithm 2's result is defined after each complete step.
 //
 // Launches cover steps [t0, t1) and keep the state in global memory between
 // launches (the fp32 path recomputes the fields between launches).
@@ -568,10 +568,10 @@ __global__ void __launch_bounds__(64, 7) step_kernel_ws(const __grid_constant__ 
 // One launch of kernel K with the on-chip memory split of prefer_shared; with
 // no blocks (p.R = 0) only the attribute is set, which also loads the kernel.
 template <auto K>
-inline void launch_shared(int blocks, int threads, size_t shm, cudaStream_t st, const StepParams& p)
+inline void launch_shared(int blocks, int threads, cudaStream_t st, const StepParams& p)
 {
     prefer_shared<K>();
-    if (blocks > 0) K<<<blocks, threads, shm, st>>>(p);
+    if (blocks > 0) K<<<blocks, threads, 0, st>>>(p);
 }
 
 // One launch on clusters of C blocks per replica, G warps in each.
@@ -632,11 +632,11 @@ cudaError_t launch_vg(const StepShape& s, const StepParams& p, bool trace, cudaS
         }
         if (blocks > 0 && sizeof(Tw) == 4 && V >= 8 && p.Wc == nullptr) return cudaErrorInvalidValue;
         if (full) {
-            if (trace) launch_shared<step_kernel_g1<Tw, V, true, true>>(blocks, threads, 0, st, p);
-            else launch_shared<step_kernel_g1<Tw, V, true, false>>(blocks, threads, 0, st, p);
+            if (trace) launch_shared<step_kernel_g1<Tw, V, true, true>>(blocks, threads, st, p);
+            else launch_shared<step_kernel_g1<Tw, V, true, false>>(blocks, threads, st, p);
         } else {
-            if (trace) launch_shared<step_kernel_g1<Tw, V, false, true>>(blocks, threads, 0, st, p);
-            else launch_shared<step_kernel_g1<Tw, V, false, false>>(blocks, threads, 0, st, p);
+            if (trace) launch_shared<step_kernel_g1<Tw, V, false, true>>(blocks, threads, st, p);
+            else launch_shared<step_kernel_g1<Tw, V, false, false>>(blocks, threads, st, p);
         }
         return cudaGetLastError();
     } else {
@@ -646,11 +646,11 @@ cudaError_t launch_vg(const StepShape& s, const StepParams& p, bool trace, cudaS
                 return launch_on_clusters<Tw, V / 2, 4, 4>(p, trace, st);
         }
         if (full) {
-            if (trace) launch_shared<step_kernel<Tw, V, G, true, true>>(blocks, threads, 0, st, p);
-            else launch_shared<step_kernel<Tw, V, G, true, false>>(blocks, threads, 0, st, p);
+            if (trace) launch_shared<step_kernel<Tw, V, G, true, true>>(blocks, threads, st, p);
+            else launch_shared<step_kernel<Tw, V, G, true, false>>(blocks, threads, st, p);
         } else {
-            if (trace) launch_shared<step_kernel<Tw, V, G, false, true>>(blocks, threads, 0, st, p);
-            else launch_shared<step_kernel<Tw, V, G, false, false>>(blocks, threads, 0, st, p);
+            if (trace) launch_shared<step_kernel<Tw, V, G, false, true>>(blocks, threads, st, p);
+            else launch_shared<step_kernel<Tw, V, G, false, false>>(blocks, threads, st, p);
         }
         return cudaGetLastError();
     }

@@ -13,13 +13,11 @@ template <> struct Arith<int8_t> {
     using E = long long;  // tracked energy
     static __device__ __forceinline__ H signed_field(H g, uint32_t x) { return x ? -g : g; }
     static __device__ __forceinline__ float to_float(H g) { return __int2float_rn(g); }
-    static __device__ __forceinline__ H apply(H h, int8_t w, bool minus) { return minus ? h - (H)w : h + (H)w; }
     using Sign = int32_t;
     static __device__ __forceinline__ Sign sign(uint32_t xold) { return xold ? -1 : 1; }
     static __device__ __forceinline__ H apply_signed(H h, int8_t w, Sign s) { return h + s * (H)w; }
     static __device__ __forceinline__ E load_e(long long b) { return b; }
     static __device__ __forceinline__ long long store_e(E e) { return e; }
-    static __device__ __forceinline__ E book(E e, H dE) { return e + (E)dE; }
     static constexpr bool kReal = false;
     static __device__ __forceinline__ uint32_t log_bits(H dE) { return (uint32_t)dE; }
     static __device__ __forceinline__ long long log_int(uint32_t b) { return (long long)(int)b; }
@@ -30,13 +28,11 @@ template <> struct Arith<int16_t> {
     using E = long long;
     static __device__ __forceinline__ H signed_field(H g, uint32_t x) { return x ? -g : g; }
     static __device__ __forceinline__ float to_float(H g) { return __int2float_rn(g); }
-    static __device__ __forceinline__ H apply(H h, int16_t w, bool minus) { return minus ? h - (H)w : h + (H)w; }
     using Sign = int32_t;
     static __device__ __forceinline__ Sign sign(uint32_t xold) { return xold ? -1 : 1; }
     static __device__ __forceinline__ H apply_signed(H h, int16_t w, Sign s) { return h + s * (H)w; }
     static __device__ __forceinline__ E load_e(long long b) { return b; }
     static __device__ __forceinline__ long long store_e(E e) { return e; }
-    static __device__ __forceinline__ E book(E e, H dE) { return e + (E)dE; }
     static constexpr bool kReal = false;
     static __device__ __forceinline__ uint32_t log_bits(H dE) { return (uint32_t)dE; }
     static __device__ __forceinline__ long long log_int(uint32_t b) { return (long long)(int)b; }
@@ -49,15 +45,13 @@ template <> struct Arith<float> {
         return __int_as_float(__float_as_int(g) ^ (int)(x << 31));
     }
     static __device__ __forceinline__ float to_float(H g) { return g; }
-    static __device__ __forceinline__ H apply(H h, float w, bool minus) { return minus ? __fsub_rn(h, w) : __fadd_rn(h, w); }
     using Sign = float;
     static __device__ __forceinline__ Sign sign(uint32_t xold) { return xold ? -1.0f : 1.0f; }
     // h + s w with s = +-1: the product is exact, so this is the same single
-    // rounding as __fadd_rn / __fsub_rn
+    // rounding as a correctly rounded addition or subtraction
     static __device__ __forceinline__ H apply_signed(H h, float w, Sign s) { return __fmaf_rn(s, w, h); }
     static __device__ __forceinline__ E load_e(long long b) { return __longlong_as_double(b); }
     static __device__ __forceinline__ long long store_e(E e) { return __double_as_longlong(e); }
-    static __device__ __forceinline__ E book(E e, H dE) { return __dadd_rn(e, (double)dE); }
     static constexpr bool kReal = true;
     static __device__ __forceinline__ uint32_t log_bits(H dE) { return __float_as_uint(dE); }
 };
@@ -79,7 +73,6 @@ template <> struct Arith<f32e> {
     static __device__ __forceinline__ H apply_signed(H h, f32e w, Sign s) { return __fmaf_rn(s, w.f, h); }
     static __device__ __forceinline__ E load_e(long long b) { return b; }
     static __device__ __forceinline__ long long store_e(E e) { return e; }
-    static __device__ __forceinline__ E book(E e, H dE) { return e + (E)__float2int_rn(dE); }
     static constexpr bool kReal = false;
     static __device__ __forceinline__ uint32_t log_bits(H dE) { return __float_as_uint(dE); }
     static __device__ __forceinline__ long long log_int(uint32_t b) { return (long long)__float2int_rn(__uint_as_float(b)); }
@@ -155,7 +148,7 @@ __device__ __forceinline__ int settle_log(const FlipEntry* f, int n, int tested,
                                           typename A::E& best)
 {
     const uint32_t bits = lane < n ? f[lane].dE : 0u;
-    if constexpr (sizeof(typename A::E) == 8 && !A::kReal) {
+    if constexpr (!A::kReal) {
         const long long v = A::log_int(bits);            // |v| < 2^31 each
         const long long neg = warp_sum53(min(v, 0ll));
         int at = -1;
