@@ -39,7 +39,14 @@ namespace step_detail {
 // words per block live in registers, for kernels that have them to spare.
 // COAL: W points at the couplings in the warp row order (row pitch ldw, slices of 32 V0
 // entries; step_uses_coal in da_internal.h) and rows are read with RowCoal.
-template <typename Tw, int V, bool SW = false, bool PRE = false, bool COAL = false, int V0 = V>
+// WIDE: the form of a step whose instructions count for more than its latency, for one warp
+// per replica at V = 32 and, without padding, at V = 16, where the default shapes put one to
+// two warps on a scheduler: counts by shuffles, packed field updates, most of the draws'
+// rounds before the choice, the rare parts out of line.  At V = 16 against the other form:
+// N = 512 with 1024 replicas 0.755 -> 0.717 us per step (int8 0.738 -> 0.714, PTDA 0.774 ->
+// 0.737), with 512 0.586 -> 0.564; with padding it is slower (N = 500 with 512 replicas 0.607 ->
+// 0.626), and so it is at V = 8 (N = 256 with 1024 replicas 0.516 -> 0.554).
+template <typename Tw, int V, bool SW = false, bool PRE = false, bool COAL = false, int V0 = V, bool WIDE = V == 32>
 struct WarpReplica {
     using A = Arith<Tw>;
     using H = typename A::H;
@@ -48,6 +55,8 @@ struct WarpReplica {
     static constexpr int NQ = V / 4;
     static constexpr uint32_t VMASK = V == 32 ? 0xffffffffu : ((1u << V) - 1u);
     static constexpr int P = 32 / V;
+    // The rare parts of a step (exact test, choice draws' refill) out of line.
+    static constexpr bool kRareOut = V != 16 || WIDE;
 
     H h[V];
     float lg[V];      // log2 U of this lane's draws for the current step (lg2_draw)
@@ -124,7 +133,7 @@ struct WarpReplica {
     __device__ __forceinline__ void fill_choice(long long t, const Keys& keys)
     {
         const uint32_t c = (uint32_t)((t & ~127ll) + 4 * lane);
-        if constexpr (kRareOutOfLine<V>) cr = choice_block(c, rep, keys);
+        if constexpr (kRareOut) cr = choice_block(c, rep, keys);
         else cr = philox4x32_10(0u, c, rep, 1u, keys);
     }
     template <class Keys>
@@ -383,16 +392,17 @@ struct WarpReplica {
         __device__ __forceinline__ void rest_flip() { f(); }
         __device__ __forceinline__ void rest_none() { f(); }
     };
-    template <class Keys, int kR0 = V == 32 ? 7 : 5, int kR1 = V == 32 ? 8 : 6, int kR2 = V == 32 ? 8 : 7,
-              int kR3 = V == 32 ? 9 : 8>
+    template <class Keys, int kR0 = WIDE ? 7 : 5, int kR1 = WIDE ? 8 : 6, int kR2 = WIDE ? 8 : 7,
+              int kR3 = WIDE ? 9 : 8>
     struct DrawSlots {     // the next step's draws (PRE)
         WarpReplica& rp;
         const Keys& keys;
         uint32_t tt;
-        // Rounds done after slot 0 .. 3, measured per V: with all of them under the row
-        // load N = 512 takes 0.608 instead of 0.562 us per step, with all of them before
-        // it 0.581 (fp32, 64 replicas); at V = 32 most of them belong before the choice
-        // (5, 6, 7, 7: 1.25 instead of 1.23 us at N = 1024 with 1024 replicas).
+        // Rounds done after slot 0 .. 3, measured per form: all of them under the row load
+        // (3, 3, 3, 3) take N = 512 with 1024 replicas from 0.755 to 0.803 us per step, all of
+        // them before it (10, 10, 10, 10) N = 256 from 0.516 to 0.543; in the wide form most
+        // belong before the choice (5, 6, 7, 7: 1.25 instead of 1.23 us at N = 1024 with 1024
+        // replicas).
         template <int I>
         __device__ __forceinline__ void at()
         {
@@ -456,18 +466,21 @@ struct WarpReplica {
         bool unsure;
         uint32_t accm = decide_log<A, V>(h, xm, Eoff, __fmul_rn(beta, kLog2e), L, unsure);
         const bool any_unsure = __any_sync(0xffffffffu, unsure);
-        // the rare exact test: at V = 32 before the count, below that after a first count
-        // whose votes overlap the vote on the band (one latency less; at V = 32 the second
-        // count's code costs more)
-        constexpr bool kFirst = V == 32;
+        // the rare exact test before the count: a first count beside the vote on the band and a
+        // second one after the test hide one latency, but their code costs more (N = 64 int8
+        // 0.341 -> 0.321 us per step without them, fp32 with 1024 replicas 0.411 -> 0.395;
+        // N = 256 with 2048 replicas, by its registers, 1.013 -> 0.864), except at V = 16 where
+        // the test is inline (N = 500 int8 with 1024 replicas 0.791, 0.813 before the count) and
+        // for integer rows at V = 8 (allocation-free, N = 200 0.429, 0.434 before it)
+        constexpr bool kFirst = kRareOut && !(V == 8 && sizeof(Tw) < 4);
         if (kFirst && any_unsure)
-            accm = decide_exact_out<A, V>(h, xm, Eoff, beta, L, accm, base, (uint32_t)t, rep, keys);
+            accm = decide_exact_out<A, V, kRareOut>(h, xm, Eoff, beta, L, accm, base, (uint32_t)t, rep, keys);
         if constexpr (!FULL) accm &= valid;
         int excl, total;
         count_below(accm, excl, total);
         slots.template at<0>();
         if (!kFirst && any_unsure) {
-            accm = decide_exact_out<A, V>(h, xm, Eoff, beta, L, accm, base, (uint32_t)t, rep, keys);
+            accm = decide_exact_out<A, V, kRareOut>(h, xm, Eoff, beta, L, accm, base, (uint32_t)t, rep, keys);
             if constexpr (!FULL) accm &= valid;
             count_below(accm, excl, total);
         }
@@ -477,16 +490,16 @@ struct WarpReplica {
     // Accepted trials on the lanes below this one, and on all lanes: the bits of the
     // lanes' counts as votes, which are independent of one another (one latency of
     // about 20 cycles, then the population counts), beside the warp reduction of the
-    // total; a five-shuffle prefix sum is a chain of five 32-cycle latencies.  At V = 32
-    // the shuffles are used all the same: a population count takes 8 cycles of the unit
-    // that also makes the 32 log2 of the draws (8 cycles each), and with two warps per
+    // total; a five-shuffle prefix sum is a chain of five 32-cycle latencies.  In the wide
+    // form the shuffles are used all the same: a population count takes 8 cycles of the
+    // unit that also makes the log2 of the draws (8 cycles each), and with two warps per
     // scheduler that counts for more than the chain (1.25 against 1.29 us per step at
     // N = 1024 with 1024 replicas).
     __device__ __forceinline__ void count_below(uint32_t accm, int& excl, int& total) const
     {
         const int cnt = __popc(accm);
         total = (int)__reduce_add_sync(0xffffffffu, (unsigned)cnt);
-        if constexpr (V == 32) {
+        if constexpr (WIDE) {
             int incl = cnt;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -552,7 +565,9 @@ struct WarpReplica {
             const typename A::Sign sg = A::sign(xold);
 #pragma unroll
             for (int v = 0; v < V; v += 2) {
-                if constexpr (sizeof(Tw) == 4 && V == 32) {   // packed: the same roundings, half the instructions
+                // packed: the same roundings, half the instructions; V = 8 only with padding
+                // (N = 200 0.440 -> 0.420 us per step, but N = 256 0.517 -> 0.521)
+                if constexpr (sizeof(Tw) == 4 && (WIDE || (V == 8 && !FULL))) {
                     const float* w = reinterpret_cast<const float*>(&cv[v]);
                     const float2 u = __ffma2_rn(make_float2(sg, sg), make_float2(w[0], w[1]), make_float2(h[v], h[v + 1]));
                     h[v] = u.x;

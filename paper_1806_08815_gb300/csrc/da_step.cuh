@@ -239,12 +239,22 @@ __global__ void __launch_bounds__(32 * G * OccupancyGV<G, V>::rpb, OccupancyGV<G
         bool unsure;
         uint32_t accm = decide_log<A, V>(rp.h, rp.xm, Eoff, __fmul_rn(rp.beta, kLog2e), rp.lg, unsure);
         const bool any_unsure = __any_sync(0xffffffffu, unsure);
+        // the rare exact test: at V = 16 in one block without padding before the count and out
+        // of line (N = 2048 with 32 replicas 0.728 -> 0.720 us per step, with 1024 2.80 -> 2.72),
+        // else after a first count (N = 500 with 128 replicas 0.487, before it 0.494; N = 8192
+        // with 64 1.557, 1.569) and at V = 16 inline (N = 2000 with 64 replicas 0.812, as a call
+        // 0.866; N = 8192 on clusters 1.32, 1.44)
+        constexpr bool kFirst = V == 16 && C == 1 && FULL, kOut = V != 16 || kFirst;
+        auto exact = [&] {
+            accm = decide_exact_out<A, V, kOut>(rp.h, rp.xm, Eoff, rp.beta, rp.lg, accm, rp.base, t, rp.rep, keys);
+        };
+        if (kFirst && any_unsure) exact();
         if constexpr (!FULL) accm &= rp.valid;
         int excl, mine;
         rp.count_below(accm, excl, mine);
         if constexpr (C == 1) slots.template at<0>();
-        if (any_unsure) {
-            accm = decide_exact_out<A, V>(rp.h, rp.xm, Eoff, rp.beta, rp.lg, accm, rp.base, t, rp.rep, keys);
+        if (!kFirst && any_unsure) {
+            exact();
             if constexpr (!FULL) accm &= rp.valid;
             rp.count_below(accm, excl, mine);
         }
@@ -404,7 +414,7 @@ __global__ void __launch_bounds__(32 * OccupancyGV<1, V>::rpb, OccupancyGV<1, V>
     step_kernel_g1(const __grid_constant__ StepParams p)
 {
     constexpr bool kCoal = sizeof(Tw) == 4 && V >= 8;   // float and f32e
-    using R_ = WarpReplica<Tw, V, false, true, kCoal>;
+    using R_ = WarpReplica<Tw, V, false, true, kCoal, V, V == 32 || (V == 16 && FULL)>;
     using H = typename R_::H;
     __shared__ FlipLog<typename R_::E> logs[OccupancyGV<1, V>::rpb];
     if (launch_stopped(p)) return;

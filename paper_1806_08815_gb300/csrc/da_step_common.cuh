@@ -499,10 +499,9 @@ __device__ __forceinline__ uint32_t decide_exact(const typename A::H (&h)[V], ui
 // one piece: with one or two warps per scheduler its instruction fetch is exposed (0.27
 // stall cycles per instruction at V = 8).  Measured per V: N = 1024 with 1024 replicas
 // 1.209 -> 1.182 us per step, with 128 (V = 8) 0.620 -> 0.608, N = 64 0.352 -> 0.347; but
-// V = 16 keeps them inline (N = 512 0.759 -> 0.763, N = 2048 0.728 -> 0.928 as calls).
-template <int V> constexpr bool kRareOutOfLine = V != 16;
+// V = 16 keeps them inline where it is not WIDE (WarpReplica; step_kernel for the other case).
 
-// decide_exact, out of line on copies of the lane's fields and draws made for the call.
+// decide_exact, where OUT out of line on copies of the lane's fields and draws made for the call.
 template <typename A, int V> struct ExactArgs {
     typename A::H h[V];
     float L[V];
@@ -514,12 +513,12 @@ __device__ __noinline__ uint32_t decide_exact_call(const ExactArgs<A, V>& a, uin
 {
     return decide_exact<A, V>(a.h, xm, Eoff, beta, a.L, acc, base, step, rep, keys);
 }
-template <typename A, int V, class Keys>
+template <typename A, int V, bool OUT, class Keys>
 __device__ __forceinline__ uint32_t decide_exact_out(const typename A::H (&h)[V], uint32_t xm, float Eoff, float beta,
                                                      const float (&L)[V], uint32_t acc, int base, uint32_t step,
                                                      uint32_t rep, const Keys& keys)
 {
-    if constexpr (!kRareOutOfLine<V>) {
+    if constexpr (!OUT) {
         return decide_exact<A, V>(h, xm, Eoff, beta, L, acc, base, step, rep, keys);
     } else {
         ExactArgs<A, V> a;
