@@ -9,9 +9,9 @@
 // votes instead of chains of shuffles, the inputs of the next step (draws, choice word,
 // beta) are made in the shadow of this one, and the fp64 energy and the best state are
 // settled 32 flips at a time (FlipLog).  us per step before and after, 64 replicas
-// (1024): fp32 N = 64 0.555 -> 0.350 (0.613 -> 0.41), N = 256 0.670 -> 0.432
-// (0.761 -> 0.535), N = 512 0.781 -> 0.562 (0.918 -> 0.757), N = 1024 0.961 -> 0.89
-// (1.327 -> 1.232).  With two warps per scheduler (the last) the pipes bind as much as
+// (1024): fp32 N = 64 0.555 -> 0.33 (0.613 -> 0.395), N = 256 0.670 -> 0.426
+// (0.761 -> 0.516), N = 512 0.781 -> 0.56 (0.918 -> 0.717), N = 1024 0.961 -> 0.89
+// (1.327 -> 1.182).  With two warps per scheduler (the last) the pipes bind as much as
 // the chain: a 32 x 32 -> 64 bit product holds the integer multiplier for 4 cycles, and
 // 120 of them with the other multiplications are 1400 of the 2550 cycles.
 //
