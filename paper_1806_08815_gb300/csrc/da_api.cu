@@ -505,6 +505,16 @@ size_t instance_W_bytes(int n, int dtype)
 
 StepShape default_shape(int N, int R) { return auto_shape(N, R); }
 
+StepShape one_warp_shape(int N)
+{
+    StepShape s;
+    s.V = 4;
+    s.G = 1;
+    s.rpb = 4;
+    while (32 * s.V < N) s.V *= 2;
+    return s;
+}
+
 void set_last_error(const std::string& msg) { g_err = msg; }
 const TcOperand& ctx_tc_operand(const da_ctx* c) { return c->tc; }
 

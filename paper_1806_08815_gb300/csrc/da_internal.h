@@ -237,6 +237,8 @@ bool build_instance(const void* Q, int n, int dtype, HostInstance& out, std::str
 
 // The default launch shape of the step kernel for N variables and R replicas.
 StepShape default_shape(int N, int R);
+// The one-warp shape of N <= 1024 variables, whatever R.
+StepShape one_warp_shape(int N);
 
 // True when every entry of a host schedule is finite and >= 0 (the kernels'
 // fast Metropolis test relies on beta >= 0).

@@ -601,7 +601,8 @@ da_status da_submit(da_server* s, const da_job* job, da_req** out)
     // a context's launch shape: measured on a mix of concurrent requests it
     // gives more trials per second than the fewest warps per replica
     q->shape = da::default_shape(q->N, job->replicas);
-    q->resident = q->N <= s->resident_max_n && q->shape.G == 1;
+    q->resident = q->N <= s->resident_max_n;
+    if (q->resident) q->shape = da::one_warp_shape(q->N);   // a warp per replica whatever their number
     plan_request(*q);
     if ((int64_t)peak_bytes(*q) > s->budget)
         return sfail(DA_EBUDGET, "request needs " + std::to_string(peak_bytes(*q)) +
