@@ -1151,7 +1151,6 @@ da_status restore_state(const da_ctx* c, const RunBuffers& b, const da_checkpoin
         sc[r].best = in->scalars[4 * r + 1];
         sc[r].flips = in->scalars[4 * r + 2];
         sc[r].m = (uint32_t)in->scalars[4 * r + 3];
-        sc[r].check = 0;
     }
     DA_CU(cudaMemcpyAsync(b.sc(), sc, (size_t)R * sizeof(ReplicaScalars), cudaMemcpyHostToDevice, st));
     return DA_OK;

@@ -183,18 +183,12 @@ __global__ void init_state_kernel(const void* __restrict__ diag, int N, int R, v
 __global__ void best_fixup_kernel(int R, ReplicaScalars* sc, bool int8, const uint32_t* x, uint32_t* bestx, int nw)
 {
     const int r = blockIdx.x;
-    ReplicaScalars s = sc[r];
-    if (!s.check) return;
+    const ReplicaScalars s = sc[r];
     const bool better = int8 ? s.E < s.best : __longlong_as_double(s.E) < __longlong_as_double(s.best);
-    if (better) {
-        for (int w = threadIdx.x; w < nw; w += blockDim.x) bestx[(size_t)r * nw + w] = x[(size_t)r * nw + w];
-    }
+    if (!better) return;
+    for (int w = threadIdx.x; w < nw; w += blockDim.x) bestx[(size_t)r * nw + w] = x[(size_t)r * nw + w];
     __syncthreads();
-    if (threadIdx.x == 0) {
-        if (better) s.best = s.E;
-        s.check = 0;
-        sc[r] = s;
-    }
+    if (threadIdx.x == 0) sc[r].best = s.E;
 }
 
 }  // namespace

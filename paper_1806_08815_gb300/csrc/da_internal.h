@@ -23,7 +23,6 @@ struct alignas(32) ReplicaScalars {
     long long best;    // lowest tracked energy seen
     long long flips;   // accepted flips
     uint32_t m;        // consecutive steps without an accepted flip (E_off = m * inc)
-    uint32_t check;    // 1: the best-state test of the last step is still to be made
 };
 
 // Launch shape of the parallel-trial step: a group of G warps per replica,
