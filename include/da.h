@@ -156,16 +156,19 @@ da_status da_ctx_info(const da_ctx* ctx, int64_t* N, da_dtype* dtype);
  * automatic choice: a group of G warps per replica, V variables per lane
  * (32 * V * G >= N), rpb replicas per thread block.  Supported: G = 1, 2 or 4
  * with V in {4, 8, 16, 32}; G = 8 with V in {8, 16, 32}; rpb <= 4 (G = 1),
- * <= 2 (G = 2), = 1 (G = 4, 8).  V = 0
- * restores the automatic choice.  Results do
+ * <= 2 (G = 2), = 1 (G = 4, 8).  The shape runs as named: only the automatic
+ * choice and da_tune_shape may put a G = 8 replica on a cluster of four blocks
+ * instead of one (N > 2048 and up to 38 replicas; faster alone, slower beside
+ * other launches).  V = 0 restores the automatic choice.  Results do
  * not depend on the shape (the random numbers are keyed by variable index,
  * step and replica).  Errors: DA_EINVAL. */
 da_status da_set_launch_shape(da_ctx* ctx, int32_t V, int32_t G, int32_t rpb);
 
 /* Autotune the step kernel's launch shape for this context's instance and R
  * replicas: every supported shape that covers N (for each G in 1, 2, 4, 8 the
- * narrowest lane width V, every allowed rpb, and for G = 1 the producer-warp
- * form) runs probe_steps steps from x = 0 with beta = 0 (every step flips), the
+ * narrowest lane width V, every allowed rpb, for G = 1 the producer-warp form
+ * and for G = 8 with up to 38 replicas the cluster form, which is reported as
+ * its V and G = 8) runs probe_steps steps from x = 0 with beta = 0 (every step flips), the
  * fastest (CUDA events, best of two runs) is written to *V, *G, *rpb,
  * *draw_warp (each may be NULL) and kept in a process-wide cache keyed by
  * (device, coupling type, N, R) that every context's later anneals use unless
@@ -488,6 +491,13 @@ int64_t da_static_pitch(int64_t N);
  * Errors: DA_EINVAL (negative arguments). */
 da_status da_diag_fail_alloc(int32_t after, int32_t count);
 da_status da_diag_live_allocations(int64_t* count, int64_t* bytes, int64_t* injected_failures);
+
+/* The launch shape of an anneal with `replicas` replicas: on context ctx (its
+ * fixed shape, its tuned one or the automatic choice), or with ctx = NULL the
+ * automatic choice for N variables, without a device (N is read only then).
+ * shape5 = V, G, rpb, 1 with a producer warp, blocks per replica (1, or 4 on a
+ * cluster).  Errors: DA_EINVAL. */
+da_status da_diag_launch_shape(da_ctx* ctx, int64_t N, int32_t replicas, int32_t* shape5);
 
 /* Read bandwidth of the device buffer buf[bytes] (device, 16-byte aligned,
  * bytes a multiple of 16): one untimed pass, then `passes` timed passes of

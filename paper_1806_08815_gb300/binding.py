@@ -105,6 +105,8 @@ def lib() -> ctypes.CDLL:
     L.da_req_free.restype = None
     L.da_diag_read_bandwidth.argtypes = [_P, i64, i32, ctypes.POINTER(ctypes.c_double)]
     L.da_diag_read_bandwidth.restype = ctypes.c_int
+    L.da_diag_launch_shape.argtypes = [_P, i64, i32, ctypes.POINTER(i32)]
+    L.da_diag_launch_shape.restype = ctypes.c_int
     L.da_cancel.argtypes = [_P]
     L.da_cancel.restype = ctypes.c_int
     L.da_diag_fail_alloc.argtypes = [i32, i32]
@@ -591,6 +593,14 @@ def da_diag_live_allocations() -> dict:
     a, b, c = ctypes.c_int64(), ctypes.c_int64(), ctypes.c_int64()
     _check(lib().da_diag_live_allocations(ctypes.byref(a), ctypes.byref(b), ctypes.byref(c)))
     return dict(count=a.value, bytes=b.value, injected=c.value)
+
+
+def da_diag_launch_shape(ctx: Context | None, replicas: int, N: int = 0) -> tuple:
+    """(V, G, replicas per block, producer warp, blocks per replica) of an anneal on ctx, or with
+    ctx None the automatic choice for N variables (no device needed)."""
+    v = (ctypes.c_int32 * 5)()
+    _check(lib().da_diag_launch_shape(ctx.handle if ctx is not None else None, int(N), int(replicas), v))
+    return tuple(v)
 
 
 def da_diag_read_bandwidth(buf_dev, passes: int) -> float:

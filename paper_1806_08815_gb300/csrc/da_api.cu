@@ -96,6 +96,17 @@ const void* step_W(const da_ctx* c) { return c->Wf ? c->Wf : c->W; }
 //   N = 2048: R = 304 - / 1.294 / .978 / 1.195, R = 512 - / 1.633 / 1.666 / 2.283,
 //             R = 1024 - / 3.237 / 2.850 / 3.958;
 //   N = 4096: R = 152 - / - / 1.354 / 1.141, R = 256 - / - / 1.678 / 2.132.
+//
+// Up to kClusterReplicas the widest shapes (8 warps of V = 16 or 32, N > 2048) run on
+// clusters of 4 blocks of 4 warps with half the V, which spreads a replica's decisions,
+// draws and row over four SMs: as many as give every block an SM.  us per step at 32
+// replicas: N = 3000 int8 1.04 -> 0.91, N = 4096 fp32 1.00 -> 0.93, N = 8192 fp32 1.60 ->
+// 1.36, int16 1.65 -> 1.26; at 64 replicas, two blocks to an SM, N = 4096 1.00 -> 1.03 and
+// N = 8192 1.60 -> 1.56.  They lose beside other launches: the request loop's burst of mixed
+// requests ran at 2.9e11 trials/s with clusters, 3.4e11 without, so it has none, and a
+// context whose anneals overlap others can fix the (V, 8) shape, which runs as named.
+constexpr int kClusterReplicas = 38;
+
 StepShape auto_shape(int N, int R)
 {
     constexpr int kSMs = 152;
@@ -110,6 +121,7 @@ StepShape auto_shape(int N, int R)
     s.V = G == 8 ? 8 : 4;
     while (32 * s.V * G < N) s.V *= 2;
     s.rpb = G == 1 ? 4 : 1;
+    if (G == 8 && s.V >= 16 && R <= kClusterReplicas) s.cluster = 4;
     return s;
 }
 
@@ -503,7 +515,12 @@ size_t instance_W_bytes(int n, int dtype)
     return ((size_t)n * align_up((size_t)n, 128) + 8192) * esz;
 }
 
-StepShape default_shape(int N, int R) { return auto_shape(N, R); }
+StepShape default_shape(int N, int R, bool beside)
+{
+    StepShape s = auto_shape(N, R);
+    if (beside) s.cluster = 1;
+    return s;
+}
 
 StepShape one_warp_shape(int N)
 {
@@ -1065,6 +1082,10 @@ extern "C" da_status da_tune_shape(da_ctx* c, int32_t R, int64_t probe_steps, in
             s.rpb = r;
             if (!da::step_shape_supported(s)) continue;
             cands.push_back(s);
+            if (g == 8 && s.V >= 16 && R <= kClusterReplicas) {
+                cands.push_back(s);
+                cands.back().cluster = 4;
+            }
         }
         if (g == 1) {
             s.rpb = 1;
@@ -1256,5 +1277,21 @@ extern "C" da_status da_anneal_segment(da_ctx* c, const float* beta, int64_t tot
         res->elapsed_s = ms * 1e-3;
         unpack_results(c, b, host.data(), res);
     }
+    return DA_OK;
+}
+
+extern "C" da_status da_diag_launch_shape(da_ctx* c, int64_t N, int32_t R, int32_t* shape5)
+{
+    g_err.clear();
+    if (!shape5 || R < 1 || (!c && (N < 1 || N > 8192))) return fail(DA_EINVAL, "need shape5, R >= 1 and 1 <= N <= 8192");
+    StepShape s;
+    if (c) {
+        std::lock_guard<std::mutex> lk(c->mu);
+        s = shape_for(c, R);
+    } else {
+        s = auto_shape((int)N, R);
+    }
+    const int32_t v[5] = {s.V, s.G, s.rpb, s.ws ? 1 : 0, s.cluster};
+    std::copy(v, v + 5, shape5);
     return DA_OK;
 }

@@ -33,6 +33,7 @@ struct StepShape {
     int G = 0;
     int rpb = 0;  // replicas (groups) per block
     bool ws = false;  // G = 1 only: one replica per block, with a producer warp for its draws
+    int cluster = 1;  // 4, for G = 8 and V >= 16 only: a replica on a cluster of 4 blocks of 4 warps of V / 2
     int npad() const { return 32 * V * G; }
     int nwords() const { return V * G; }
 };
@@ -234,8 +235,9 @@ cudaError_t launch_expand_instance(const void* Q, int n, int ldw, int dtype, voi
                                    cudaStream_t st);
 bool build_instance(const void* Q, int n, int dtype, HostInstance& out, std::string& why);
 
-// The default launch shape of the step kernel for N variables and R replicas.
-StepShape default_shape(int N, int R);
+// The default launch shape of the step kernel for N variables and R replicas; `beside`:
+// for launches that run beside others (the request loop), which stay off clusters.
+StepShape default_shape(int N, int R, bool beside = false);
 // The one-warp shape of N <= 1024 variables, whatever R.
 StepShape one_warp_shape(int N);
 

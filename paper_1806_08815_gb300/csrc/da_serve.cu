@@ -600,7 +600,7 @@ da_status da_submit(da_server* s, const da_job* job, da_req** out)
     if (!da::build_instance(job->Q, q->N, job->dtype, q->inst, why)) return sfail(DA_EINVAL, why);
     // a context's launch shape: measured on a mix of concurrent requests it
     // gives more trials per second than the fewest warps per replica
-    q->shape = da::default_shape(q->N, job->replicas);
+    q->shape = da::default_shape(q->N, job->replicas, true);
     q->resident = q->N <= s->resident_max_n;
     if (q->resident) q->shape = da::one_warp_shape(q->N);   // a warp per replica whatever their number
     plan_request(*q);

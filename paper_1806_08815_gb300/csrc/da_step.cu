@@ -21,7 +21,8 @@ bool step_shape_supported(const StepShape& s)
     default: vg = false;
     }
     const int max_rpb = s.G == 1 ? 4 : s.G == 2 ? 2 : 1;
-    return vg && s.rpb >= 1 && s.rpb <= max_rpb;
+    const bool cluster = s.cluster == 1 || (s.cluster == 4 && s.G == 8 && s.V >= 16);
+    return vg && cluster && s.rpb >= 1 && s.rpb <= max_rpb;
 }
 
 cudaError_t launch_step(int wtype, const StepShape& s, const StepParams& p, bool trace, cudaStream_t st)

@@ -161,7 +161,8 @@ __device__ __forceinline__ bool cluster_await(uint32_t bar, uint32_t parity)
 // N = 1024 (G = 4, V = 8) 1.015 -> 0.611, N = 2048 (G = 4, V = 16) 1.168 -> 0.755,
 // N = 4096 (G = 8, V = 16) 1.564 -> 1.000, N = 8192 (G = 8, V = 32) 2.712 -> 1.606
 // (there the rows of W come from HBM).  16 warps in one block are no faster: N = 2048
-// 0.978, N = 4096 1.314, N = 8192 1.955; on several SMs they are (kClusterReplicas).
+// 0.978, N = 4096 1.314, N = 8192 1.955; on several SMs they are (kClusterReplicas in
+// da_api.cu).
 // C > 1: the replica on the C blocks of a cluster, G warps in each (warp w of block c is
 // warp c G + w); published to every block, the cluster's barrier in the place of the
 // block's.
@@ -611,16 +612,6 @@ cudaError_t launch_on_clusters(const StepParams& p, bool trace, cudaStream_t st)
                  : launch_cluster<step_kernel<Tw, V, G, false, false, C>>(C, 32 * G, st, p);
 }
 
-// The replicas up to which the widest shapes (8 warps of V = 16 or 32, N > 2048) run on
-// clusters of 4 blocks of 4 warps with half the V, which spreads a replica's decisions,
-// draws and row over four SMs: as many as give every block an SM.  us per step at 32
-// replicas: N = 3000 int8 1.04 -> 0.91, N = 4096 fp32 1.00 -> 0.93, N = 8192 fp32 1.60 ->
-// 1.36, int16 1.65 -> 1.26; at 64 replicas, two blocks to an SM, N = 4096 1.00 -> 1.03 and
-// N = 8192 1.60 -> 1.56.  Not for the request loop's launches (those with a stop flag),
-// which run beside others: its burst of mixed requests ran at 2.9e11 trials/s with
-// clusters, 3.4e11 without.
-constexpr int kClusterReplicas = 38;
-
 template <typename Tw, int V, int G>
 cudaError_t launch_vg(const StepShape& s, const StepParams& p, bool trace, cudaStream_t st)
 {
@@ -651,8 +642,10 @@ cudaError_t launch_vg(const StepShape& s, const StepParams& p, bool trace, cudaS
     } else {
         if (blocks > 0 && sizeof(Tw) == 4 && V >= 8 && p.Wc == nullptr) return cudaErrorInvalidValue;
         if constexpr (G == 8 && V >= 16) {
-            if (p.R > 0 && p.R <= kClusterReplicas && p.stop == nullptr)
-                return launch_on_clusters<Tw, V / 2, 4, 4>(p, trace, st);
+            if (s.cluster > 1) {                    // its blocks do not look at a stop flag
+                if (p.R > 0 && p.stop) return cudaErrorInvalidValue;
+                return p.R > 0 ? launch_on_clusters<Tw, V / 2, 4, 4>(p, trace, st) : cudaSuccess;
+            }
         }
         if (full) {
             if (trace) launch_shared<step_kernel<Tw, V, G, true, true>>(blocks, threads, st, p);
