@@ -142,9 +142,12 @@ StepShape shape_for(const da_ctx* c, int R)
         auto f = g_shape_cache.find(std::make_tuple(c->device, step_wtype(c), c->N, R));
         if (f != g_shape_cache.end()) return f->second;
     }
-    StepShape s = auto_shape(c->N, c->draw_warp ? 1 << 30 : R);   // the producer-warp form is a one-warp shape
-    s.ws = s.G == 1 && c->draw_warp;
-    return s;
+    if (c->draw_warp && c->N <= 1024) {   // the producer-warp form is a one-warp shape
+        StepShape s = da::one_warp_shape(c->N);
+        s.ws = true;
+        return s;
+    }
+    return auto_shape(c->N, R);
 }
 
 da_status ensure_ws(da_ctx* c, size_t bytes)
