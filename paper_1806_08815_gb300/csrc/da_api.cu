@@ -394,7 +394,8 @@ da_status run_anneal(da_ctx* c, const RunBuffers& b, const float* beta_dev, long
         if (rec && p.t1 % recompute_every == 0) {
             DA_CU(da::launch_recompute_tc(false, c->tc, c->diag, c->N, c->S, b.x(), b.s.nwords(), b.R, b.h(),
                                           b.s.npad(), reinterpret_cast<long long*>(b.sc()),
-                                          (int)(sizeof(ReplicaScalars) / 8), st, b.sums(), b.arrived()));
+                                          (int)(sizeof(ReplicaScalars) / 8), st, b.sums(), b.arrived(),
+                                          &b.sc()->check));
         }
     }
     DA_CU(da::launch_best_fixup(b.R, b.sc(), is_int(c), b.x(), b.bestx(), b.s.nwords(), st));
@@ -1175,6 +1176,7 @@ da_status restore_state(const da_ctx* c, const RunBuffers& b, const da_checkpoin
         sc[r].best = in->scalars[4 * r + 1];
         sc[r].flips = in->scalars[4 * r + 2];
         sc[r].m = (uint32_t)in->scalars[4 * r + 3];
+        sc[r].check = 0;
     }
     DA_CU(cudaMemcpyAsync(b.sc(), sc, (size_t)R * sizeof(ReplicaScalars), cudaMemcpyHostToDevice, st));
     return DA_OK;

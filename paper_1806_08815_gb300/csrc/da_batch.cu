@@ -127,6 +127,7 @@ __device__ __forceinline__ void run_unit(UnitShared<Tw>& u, int r, const Tw* W, 
         s.best = A::store_e(u.log.head.best);
         s.flips = u.log.head.flips;
         s.m = rp.m;
+        s.check = 0;
         it.sc[r] = s;
     }
     __syncwarp();           // every lane is done with the item before the next one takes its place

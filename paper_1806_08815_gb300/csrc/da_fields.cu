@@ -153,15 +153,17 @@ __global__ void __launch_bounds__(kWarps * 32) recompute_kernel(const void* __re
 }
 
 // E[r] = (sum over row tiles of the partial sums) / 2^(S+1), exact for int8,
-// rounded once to fp64 for fp32.
+// rounded once to fp64 for fp32; check (optional) is set beside it.
 template <bool INT8>
-__global__ void energy_kernel(const I128* __restrict__ part, int tiles, int R, int S, long long* E, int Estride)
+__global__ void energy_kernel(const I128* __restrict__ part, int tiles, int R, int S, long long* E, int Estride,
+                              uint32_t* check)
 {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= R) return;
     I128 s = {0ull, 0ll};
     for (int b = 0; b < tiles; ++b) s = i128_add(s, part[(size_t)b * R + r]);
     E[(size_t)r * Estride] = energy_of_sum<INT8>(s.lo, s.hi, S);
+    if (check) check[(size_t)r * Estride * 2] = 1u;
 }
 
 // g[r][i] = diag[i] for i < N, 0 on the padding (MODE 0: int32 diag and
@@ -183,12 +185,18 @@ __global__ void init_state_kernel(const void* __restrict__ diag, int N, int R, v
 __global__ void best_fixup_kernel(int R, ReplicaScalars* sc, bool int8, const uint32_t* x, uint32_t* bestx, int nw)
 {
     const int r = blockIdx.x;
-    const ReplicaScalars s = sc[r];
+    ReplicaScalars s = sc[r];
+    if (!s.check) return;
     const bool better = int8 ? s.E < s.best : __longlong_as_double(s.E) < __longlong_as_double(s.best);
-    if (!better) return;
-    for (int w = threadIdx.x; w < nw; w += blockDim.x) bestx[(size_t)r * nw + w] = x[(size_t)r * nw + w];
+    if (better) {
+        for (int w = threadIdx.x; w < nw; w += blockDim.x) bestx[(size_t)r * nw + w] = x[(size_t)r * nw + w];
+    }
     __syncthreads();
-    if (threadIdx.x == 0) sc[r].best = s.E;
+    if (threadIdx.x == 0) {
+        if (better) s.best = s.E;
+        s.check = 0;
+        sc[r] = s;
+    }
 }
 
 }  // namespace
@@ -355,17 +363,17 @@ cudaError_t launch_init_state(bool is_int8, const void* diag, int N, int R, void
 }
 
 cudaError_t launch_energy_sum(bool is_int8, const long long* part, int tiles, int R, int S, long long* E, int Estride,
-                              cudaStream_t st)
+                              cudaStream_t st, uint32_t* check)
 {
     if (R <= 0) return cudaSuccess;
     const int tb = 128;
     const I128* pp = reinterpret_cast<const I128*>(part);
     if (is_int8) {
         prefer_shared<energy_kernel<true>>();
-        energy_kernel<true><<<(R + tb - 1) / tb, tb, 0, st>>>(pp, tiles, R, S, E, Estride);
+        energy_kernel<true><<<(R + tb - 1) / tb, tb, 0, st>>>(pp, tiles, R, S, E, Estride, check);
     } else {
         prefer_shared<energy_kernel<false>>();
-        energy_kernel<false><<<(R + tb - 1) / tb, tb, 0, st>>>(pp, tiles, R, S, E, Estride);
+        energy_kernel<false><<<(R + tb - 1) / tb, tb, 0, st>>>(pp, tiles, R, S, E, Estride, check);
     }
     return cudaGetLastError();
 }

@@ -23,6 +23,7 @@ struct alignas(32) ReplicaScalars {
     long long best;    // lowest tracked energy seen
     long long flips;   // accepted flips
     uint32_t m;        // consecutive steps without an accepted flip (E_off = m * inc)
+    uint32_t check;    // 1: the best-state test of the state is still to be made
 };
 
 // Launch shape of the parallel-trial step: a group of G warps per replica,
@@ -132,9 +133,9 @@ cudaError_t launch_recompute_w(int wtype, const void* W, const void* diag, int N
 
 // E[r * Estride] from the 128-bit partial sums part[tiles][R] of a recompute:
 // the energy sum / 2^(S+1) (int64, or the fp64 bit pattern of its single
-// rounding for fp32) (da_fields.cu).
+// rounding for fp32) (da_fields.cu); check (optional): check[2 Estride r] = 1.
 cudaError_t launch_energy_sum(bool is_int8, const long long* part, int tiles, int R, int S, long long* E, int Estride,
-                              cudaStream_t st);
+                              cudaStream_t st, uint32_t* check = nullptr);
 
 // Tensor-core form of the same recompute (da_mma.cu), bit-identical to
 // launch_recompute.  The operand holds the instance's couplings on the
@@ -164,10 +165,12 @@ size_t tc_partial_bytes(int rows, int R);
 // Arguments as launch_recompute (is_int8: integer couplings of either width,
 // int32 fields); with E, scratch must hold tc_partial_bytes(rows, R) bytes.  arrived
 // (optional): ceil(R / kTcStates) counters, 0 before the call and left 0 by it, not shared
-// with another call in flight: the kernel then sums the partial energies itself.
+// with another call in flight: the kernel then sums the partial energies itself.  check
+// (optional, with E inside ReplicaScalars): the states' check flags, set to 1.
 cudaError_t launch_recompute_tc(bool is_int8, const TcOperand& op, const void* diag, int N, int S,
                                 const uint32_t* xs, int nw, int R, void* hout, int npad, long long* E, int Estride,
-                                cudaStream_t st, long long* scratch, unsigned* arrived = nullptr);
+                                cudaStream_t st, long long* scratch, unsigned* arrived = nullptr,
+                                uint32_t* check = nullptr);
 constexpr int kTcStates = 128;   // states per tile of the kernel
 
 // PT exchange (da_pt.cu).

@@ -178,6 +178,7 @@ struct TcParams {
                             // of a state tile that comes last sums the partial energies itself
     long long* E;           // with arrived: E[r Estride] as launch_energy_sum writes it
     int Estride;
+    uint32_t* check;        // or null: check[r 2 Estride] = 1 with every E[r Estride]
     int* err;
     int N, S, bits, limbs, kchunks, nw, R, npad;
     uint32_t ncols;         // tensor-memory columns allocated
@@ -425,6 +426,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) recompute_tc_kernel(cons
 #pragma unroll
             for (int g = 1; g < kThreads / kBM; ++g) i128_add2(t, s_part[g][m]);
             p.E[(size_t)r * p.Estride] = energy_of_sum<INT8>(t.lo, t.hi, p.S);
+            if (p.check) p.check[(size_t)r * p.Estride * 2] = 1u;
         }
     }
 }
@@ -572,7 +574,7 @@ cudaError_t prepare_tc_kernels()
 
 cudaError_t launch_recompute_tc(bool is_int8, const TcOperand& op, const void* diag, int N, int S,
                                 const uint32_t* xs, int nw, int R, void* hout, int npad, long long* E, int Estride,
-                                cudaStream_t st, long long* scratch, unsigned* arrived)
+                                cudaStream_t st, long long* scratch, unsigned* arrived, uint32_t* check)
 {
     if (R <= 0) return cudaSuccess;
     // the dynamic shared-memory limit of each kernel form, set once per device
@@ -608,6 +610,7 @@ cudaError_t launch_recompute_tc(bool is_int8, const TcOperand& op, const void* d
     p.arrived = E ? arrived : nullptr;
     p.E = E;
     p.Estride = Estride;
+    p.check = check;
     p.err = op.err;
     p.N = N;
     p.S = S;
@@ -627,7 +630,7 @@ cudaError_t launch_recompute_tc(bool is_int8, const TcOperand& op, const void* d
         recompute_tc_kernel<false><<<grid, kThreads, smem, st>>>(p);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || !E || arrived) return e;
-    return launch_energy_sum(is_int8, scratch, itiles, R, S, E, Estride, st);
+    return launch_energy_sum(is_int8, scratch, itiles, R, S, E, Estride, st, check);
 }
 
 }  // namespace da

@@ -337,7 +337,7 @@ bool admit(da_server* s, Req& q, long long& launches)
         if (P > 0 && p.t1 % P == 0) {
             if (!cu_ok(da::launch_recompute_tc(false, q.tc, diag, q.N, q.inst.S, xs, sh.nwords(), R, h, sh.npad(),
                                                reinterpret_cast<long long*>(sc), (int)(sizeof(da::ReplicaScalars) / 8),
-                                               st, part),
+                                               st, part, nullptr, &sc->check),
                        q, "recompute"))
                 return false;
             launches += 2;

@@ -26,11 +26,11 @@
 // to a log in shared memory, settled 32 flips at a time (settle_log).  A G = 1
 // group needs no barrier.  A G > 1 group publishes its lanes' acceptance and
 // state masks in shared memory behind one named barrier per step.  The
-// best-state test of a launch's last step is left to the start of the next one
-// (or best_fixup_kernel), so that it sees the energy after any recompute
-// between launches, as Algorithm 2's result is defined after each complete step:
-// a recompute can lower the tracked energy below the best one although the step
-// before it flipped nothing.
+// best-state test of a launch's last step is left pending
+// (ReplicaScalars::check) so that it sees the energy after any recompute
+// between launches, as Algorithm 2's result is defined after each complete step;
+// a recompute sets it too, for it can lower the energy below the best one
+// although the step before it flipped nothing.
 //
 // Launches cover steps [t0, t1) and keep the state in global memory between
 // launches (the fp32 path recomputes the fields between launches).
@@ -218,8 +218,8 @@ __global__ void __launch_bounds__(32 * G * OccupancyGV<G, V>::rpb, OccupancyGV<G
     const bool per_rep = p.betas != nullptr;
     rp.begin(p.t0, p.t1, per_rep ? nullptr : p.beta, per_rep ? p.betas[p.temp_of[r]] : 0.f, A::load_e(sc.E),
              A::load_e(sc.best), sc.flips, keys);
-    bool held = false;               // the last step flipped: its best-state test is left to what follows
-    if (p.t0 < p.t1) rp.test_current();
+    bool held = sc.check != 0;
+    if (held && p.t0 < p.t1) rp.test_current();
     if constexpr (kPre) {
         rp.prep_draws(keys);
         if (p.t0 < p.t1) rp.draw_pre((uint32_t)p.t0, keys);
@@ -405,6 +405,7 @@ __global__ void __launch_bounds__(32 * G * OccupancyGV<G, V>::rpb, OccupancyGV<G
         sc.best = A::store_e(rp.head->best);
         sc.flips = rp.head->flips;
         sc.m = rp.m;
+        sc.check = held ? 1u : 0u;
         p.sc[r] = sc;
     }
 }
@@ -436,8 +437,8 @@ __global__ void __launch_bounds__(32 * OccupancyGV<1, V>::rpb, OccupancyGV<1, V>
     const bool per_rep = p.betas != nullptr;
     rp.begin(p.t0, p.t1, per_rep ? nullptr : p.beta, per_rep ? p.betas[p.temp_of[r]] : 0.f, Arith<Tw>::load_e(sc.E),
              Arith<Tw>::load_e(sc.best), sc.flips, keys);
-    bool held = false;               // the last step flipped: its best-state test is left to what follows
-    if (p.t0 < p.t1) rp.test_current();
+    bool held = sc.check != 0;       // the best-state test of the last step is still to be made
+    if (held && p.t0 < p.t1) rp.test_current();
     rp.prep_draws(keys);
     if (p.t0 < p.t1) rp.draw_pre((uint32_t)p.t0, keys);
     for (uint32_t t = (uint32_t)p.t0; t < (uint32_t)p.t1; ++t) {
@@ -456,6 +457,7 @@ __global__ void __launch_bounds__(32 * OccupancyGV<1, V>::rpb, OccupancyGV<1, V>
         sc.best = Arith<Tw>::store_e(rp.head->best);
         sc.flips = rp.head->flips;
         sc.m = rp.m;
+        sc.check = held ? 1u : 0u;
         p.sc[r] = sc;
     }
 }
@@ -532,8 +534,8 @@ __global__ void __launch_bounds__(64, 7) step_kernel_ws(const __grid_constant__ 
     const bool per_rep = p.betas != nullptr;
     rp.begin(p.t0, p.t1, per_rep ? nullptr : p.beta, per_rep ? p.betas[p.temp_of[r]] : 0.f, Arith<Tw>::load_e(sc.E),
              Arith<Tw>::load_e(sc.best), sc.flips, keys);
-    bool held = false;               // the last step flipped: its best-state test is left to what follows
-    if (p.t0 < p.t1) rp.test_current();
+    bool held = sc.check != 0;       // the best-state test of the last step is still to be made
+    if (held && p.t0 < p.t1) rp.test_current();
 
     float L[V];
     bool ok = true;
@@ -571,6 +573,7 @@ __global__ void __launch_bounds__(64, 7) step_kernel_ws(const __grid_constant__ 
         sc.best = Arith<Tw>::store_e(rp.head->best);
         sc.flips = rp.head->flips;
         sc.m = rp.m;
+        sc.check = held ? 1u : 0u;
         p.sc[r] = sc;
     }
 }
