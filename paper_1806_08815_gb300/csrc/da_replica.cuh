@@ -46,7 +46,13 @@ namespace step_detail {
 // N = 512 with 1024 replicas 0.755 -> 0.717 us per step (int8 0.738 -> 0.714, PTDA 0.774 ->
 // 0.737), with 512 0.586 -> 0.564; with padding it is slower (N = 500 with 512 replicas 0.607 ->
 // 0.626), and so it is at V = 8 (N = 256 with 1024 replicas 0.516 -> 0.554).
-template <typename Tw, int V, bool SW = false, bool PRE = false, bool COAL = false, int V0 = V, bool WIDE = V == 32>
+// RARE_OUT: the rare parts of a step (exact test, choice draws' refill) out of line.
+// SLACK: lanes wholly beyond N load their part of a row too, and leave it: a load under a
+// condition stays before the code that follows it, its registers live throughout, where an
+// unconditional one moves down to its use.  W in the plain order has the room for it
+// (instance_W_bytes).
+template <typename Tw, int V, bool SW = false, bool PRE = false, bool COAL = false, int V0 = V, bool WIDE = V == 32,
+          bool RARE_OUT = V != 16 || WIDE, bool SLACK = false>
 struct WarpReplica {
     using A = Arith<Tw>;
     using H = typename A::H;
@@ -55,8 +61,6 @@ struct WarpReplica {
     static constexpr int NQ = V / 4;
     static constexpr uint32_t VMASK = V == 32 ? 0xffffffffu : ((1u << V) - 1u);
     static constexpr int P = 32 / V;
-    // The rare parts of a step (exact test, choice draws' refill) out of line.
-    static constexpr bool kRareOut = V != 16 || WIDE;
 
     H h[V];
     float lg[V];      // log2 U of this lane's draws for the current step (lg2_draw)
@@ -133,7 +137,7 @@ struct WarpReplica {
     __device__ __forceinline__ void fill_choice(long long t, const Keys& keys)
     {
         const uint32_t c = (uint32_t)((t & ~127ll) + 4 * lane);
-        if constexpr (kRareOut) cr = choice_block(c, rep, keys);
+        if constexpr (RARE_OUT) cr = choice_block(c, rep, keys);
         else cr = philox4x32_10(0u, c, rep, 1u, keys);
     }
     template <class Keys>
@@ -472,15 +476,15 @@ struct WarpReplica {
         // N = 256 with 2048 replicas, by its registers, 1.013 -> 0.864), except at V = 16 where
         // the test is inline (N = 500 int8 with 1024 replicas 0.791, 0.813 before the count) and
         // for integer rows at V = 8 (allocation-free, N = 200 0.429, 0.434 before it)
-        constexpr bool kFirst = kRareOut && !(V == 8 && sizeof(Tw) < 4);
+        constexpr bool kFirst = RARE_OUT && !(V == 8 && sizeof(Tw) < 4);
         if (kFirst && any_unsure)
-            accm = decide_exact_out<A, V, kRareOut>(h, xm, Eoff, beta, L, accm, base, (uint32_t)t, rep, keys);
+            accm = decide_exact_out<A, V, RARE_OUT>(h, xm, Eoff, beta, L, accm, base, (uint32_t)t, rep, keys);
         if constexpr (!FULL) accm &= valid;
         int excl, total;
         count_below(accm, excl, total);
         slots.template at<0>();
         if (!kFirst && any_unsure) {
-            accm = decide_exact_out<A, V, kRareOut>(h, xm, Eoff, beta, L, accm, base, (uint32_t)t, rep, keys);
+            accm = decide_exact_out<A, V, RARE_OUT>(h, xm, Eoff, beta, L, accm, base, (uint32_t)t, rep, keys);
             if constexpr (!FULL) accm &= valid;
             count_below(accm, excl, total);
         }
@@ -556,7 +560,7 @@ struct WarpReplica {
         const H gk = select_slot<H, V>(h, vk);
         const int k = own * V + vk;
         Tw cv[V];
-        if (FULL || base < N) load_row(W + (size_t)k * ldw + rowoff, cv);
+        if (FULL || SLACK || base < N) load_row(W + (size_t)k * ldw + rowoff, cv);
         if (lane == own) log[n] = FlipEntry{A::log_bits(A::signed_field(gk, xold)), k};
         ++n;
         slots.rest_flip();

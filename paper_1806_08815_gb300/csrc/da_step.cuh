@@ -471,6 +471,12 @@ __global__ void __launch_bounds__(32 * OccupancyGV<1, V>::rpb, OccupancyGV<1, V>
 // handshakes are mbarriers whose waits are bounded (a wait that gives up
 // sets *p.err and ends the launch; the replica's results are then invalid,
 // and later launches that see the flag leave at once).
+//
+// Seven blocks per SM, so that 1024 replicas run in one wave, leave 128 registers; at V = 32
+// the exact test is inline and the row load unconditional (SLACK) to fit them: 32 bytes of
+// spills without padding and 40 with it, 300 and 440 with the test out of line and the load
+// under its condition.  us per step with 128 (1024) replicas, fp32: N = 1024 0.99 (1.63), 1.00 (1.83) before,
+// N = 1000 1.02 (1.63), 1.44 (2.59) before.
 constexpr int kWsRing = 4;
 constexpr uint32_t kWsWaitPolls = 1u << 26;
 constexpr uint64_t kWsWaitNs = 2000000000ull;
@@ -478,7 +484,7 @@ constexpr uint64_t kWsWaitNs = 2000000000ull;
 template <typename Tw, int V, bool FULL, bool TRACE>
 __global__ void __launch_bounds__(64, 7) step_kernel_ws(const __grid_constant__ StepParams p)
 {
-    using R_ = WarpReplica<Tw, V>;
+    using R_ = WarpReplica<Tw, V, false, false, false, V, V == 32, (V < 16), V == 32>;
     using H = typename R_::H;
     constexpr int NQ = V / 4;
     __shared__ float4 ring[kWsRing][NQ][32];
