@@ -152,6 +152,14 @@ __device__ __forceinline__ bool cluster_await(uint32_t bar, uint32_t parity)
     return false;
 }
 
+// After a wait that gave up: time for asynchronous stores on their way to this block, before
+// its shared memory goes to another (they take about a microsecond).
+__device__ __forceinline__ void cluster_drain()
+{
+    const uint64_t t0 = tc::global_ns();
+    for (uint32_t i = 0; i < (1u << 20) && tc::global_ns() - t0 < 1000000ull; ++i) {}
+}
+
 // G > 1 warps per replica: warp w owns the slice [32 V w, 32 V (w + 1)) of the variables.
 // One barrier per step: every lane publishes its mask, state bits and in-warp prefix
 // count, every warp its total; after the barrier each warp finds the owner warp from the
@@ -391,7 +399,10 @@ __global__ void __launch_bounds__(32 * G * OccupancyGV<G, V>::rpb, OccupancyGV<G
         __syncwarp();
         cluster_arrive();                           // no block leaves while another may still store to it
         cluster_wait();
-        if (lost) return;
+        if (lost) {                                 // a store sent before that, which no wait here counted, lands
+            cluster_drain();
+            return;
+        }
     } else {
         group_barrier(1 + g, 32 * G);
     }
