@@ -57,8 +57,9 @@ template <typename Tw> struct UnitShared {
 
 // One work unit: replica r of item u.it, all of its steps, by the calling warp;
 // W points at the item's couplings (global memory, row pitch ldw) or at a
-// copy staged in shared memory (SW, row pitch ldw = 32 V).
-template <typename Tw, int V, bool SW, bool COAL = false>
+// copy staged in shared memory (SW, row pitch ldw = 32 V).  TRACE: the flipped index of every
+// step goes to it.trace where the item has one.
+template <typename Tw, int V, bool SW, bool COAL, bool TRACE>
 __device__ __forceinline__ void run_unit(UnitShared<Tw>& u, int r, const Tw* W, int ldw, long long t_limit)
 {
     // The precomputed Philox words and the table of round keys where there are registers for
@@ -90,7 +91,7 @@ __device__ __forceinline__ void run_unit(UnitShared<Tw>& u, int r, const Tw* W, 
     const uint32_t T = (uint32_t)(t_limit > 0 ? std::min(t_limit, it.T) : it.T);   // < 2^32
     rp.begin(0, T, it.beta, 0.f, 0, 0, 0, keys);
     // the steps up to the next point where something else is due: a recompute of the
-    // fp32 fields, a look at the stop flag, the trace of every step, the end
+    // fp32 fields, a look at the stop flag, the end
     uint32_t t = 0;
     while (t < T) {
         // the draws (and their step-invariant words) are made anew after a recompute: dead
@@ -101,14 +102,17 @@ __device__ __forceinline__ void run_unit(UnitShared<Tw>& u, int r, const Tw* W, 
         } else {
             rp.draw(t, keys);
         }
-        long long due = T;
+        uint32_t t1 = T;
         if (kReal && it.recompute_every > 0)
-            due = std::min(due, (t / it.recompute_every + 1) * it.recompute_every);
-        if (it.stop) due = std::min(due, ((long long)t / 1024 + 1) * 1024);
-        if (it.trace) due = t + 1;
+            t1 = (uint32_t)std::min<long long>(t1, (t / it.recompute_every + 1) * it.recompute_every);
+        if (it.stop) t1 = (uint32_t)std::min<long long>(t1, ((long long)t / 1024 + 1) * 1024);
         int k = -1;
-        for (const uint32_t t1 = (uint32_t)due; t < t1; ++t) k = rp.template step<false>(t, true, inc, keys);
-        if (it.trace && lane == 0) it.trace[(size_t)r * it.T + t - 1] = k;
+        for (; t < t1; ++t) {
+            k = rp.template step<false>(t, true, inc, keys);
+            if constexpr (TRACE) {
+                if (it.trace && lane == 0) it.trace[(size_t)r * it.T + t] = k;
+            }
+        }
         if (it.stop && t % 1024 == 0 && *reinterpret_cast<const volatile int*>(it.stop)) break;
         if constexpr (kReal) {
             if (it.recompute_every > 0 && t % it.recompute_every == 0) {
@@ -136,8 +140,9 @@ __device__ __forceinline__ void run_unit(UnitShared<Tw>& u, int r, const Tw* W, 
 // COAL: rows of W from the items' copies in the one-warp row order (it.Wc).
 // Blocks per SM in the launch bounds: registers enough for the step without spills (the
 // compiler's own choice leaves V = 16 with fewer: 0.77 instead of 0.69 ms per 1024 steps
-// of 512 fp32 replicas).
-template <typename Tw, int V, bool COAL = false>
+// of 512 fp32 replicas).  TRACE is a kernel of its own: a test of the item's trace in every
+// step costs launches without one 1 to 5 %.
+template <typename Tw, int V, bool COAL, bool TRACE>
 __global__ void __launch_bounds__(128, V == 4 ? 4 : V == 8 ? 3 : 2)
     batch_kernel(const __grid_constant__ BatchClassParams bp)
 {
@@ -159,15 +164,15 @@ __global__ void __launch_bounds__(128, V == 4 ? 4 : V == 8 ? 3 : 2)
         if (lane == 0) u.it = bp.items[lo];
         __syncwarp();
         const int r = (int)(unit - (unsigned long long)u.it.unit0);
-        if constexpr (COAL) run_unit<Tw, V, false, true>(u, r, static_cast<const Tw*>(u.it.Wc), 32 * V, bp.t_limit);
-        else run_unit<Tw, V, false>(u, r, static_cast<const Tw*>(u.it.W), u.it.ldw, bp.t_limit);
+        if constexpr (COAL) run_unit<Tw, V, false, true, TRACE>(u, r, static_cast<const Tw*>(u.it.Wc), 32 * V, bp.t_limit);
+        else run_unit<Tw, V, false, false, TRACE>(u, r, static_cast<const Tw*>(u.it.W), u.it.ldw, bp.t_limit);
     }
 }
 
 // Shared-memory staging: the block takes group g = (item, r0) from the
 // counter, copies rows 0..N-1 of the item's W into shared memory (row pitch
 // 32 V, zeros beyond column N), and warp w runs replica r0 + w.
-template <typename Tw, int V>
+template <typename Tw, int V, bool TRACE>
 __global__ void __launch_bounds__(512) batch_kernel_smem(const __grid_constant__ BatchClassParams bp)
 {
     extern __shared__ __align__(16) unsigned char wsm_raw[];
@@ -195,7 +200,7 @@ __global__ void __launch_bounds__(512) batch_kernel_smem(const __grid_constant__
         const int r = gi.y + warp;
         if ((threadIdx.x & 31) == 0) shared[warp].it = it;
         __syncwarp();
-        if (r < it.R) run_unit<Tw, V, true>(shared[warp], r, Ws, cols, bp.t_limit);
+        if (r < it.R) run_unit<Tw, V, true, false, TRACE>(shared[warp], r, Ws, cols, bp.t_limit);
     }
 }
 
@@ -204,18 +209,19 @@ typedef void (*BatchKernel)(BatchClassParams);
 // Kernels per step coupling form wk: kWInt8AsF32 (int8 instances, exact fp32
 // couplings), kWFp32, kWInt16 (16-bit couplings, int32 fields; rows from L2
 // only: the staged copy holds 4-byte entries).
+template <bool TRACE>
 BatchKernel smem_kernel_for(int wk, int V)
 {
     if (wk == kWInt16) return nullptr;
     if (wk == kWInt8AsF32) {
         switch (V) {
-        case 4: return batch_kernel_smem<step_detail::f32e, 4>;
-        case 8: return batch_kernel_smem<step_detail::f32e, 8>;
+        case 4: return batch_kernel_smem<step_detail::f32e, 4, TRACE>;
+        case 8: return batch_kernel_smem<step_detail::f32e, 8, TRACE>;
         }
     } else {
         switch (V) {
-        case 4: return batch_kernel_smem<float, 4>;
-        case 8: return batch_kernel_smem<float, 8>;
+        case 4: return batch_kernel_smem<float, 4, TRACE>;
+        case 8: return batch_kernel_smem<float, 8, TRACE>;
         }
     }
     return nullptr;
@@ -223,44 +229,45 @@ BatchKernel smem_kernel_for(int wk, int V)
 
 // The rows-from-L2 kernel of a class; coal: its items carry the row-ordered copies
 // (the fp32 forms at V >= 8).
+template <bool TRACE>
 BatchKernel kernel_for(int wk, int V, bool coal)
 {
     if (coal && wk == kWInt8AsF32) {
         switch (V) {
-        case 8: return batch_kernel<step_detail::f32e, 8, true>;
-        case 16: return batch_kernel<step_detail::f32e, 16, true>;
-        case 32: return batch_kernel<step_detail::f32e, 32, true>;
+        case 8: return batch_kernel<step_detail::f32e, 8, true, TRACE>;
+        case 16: return batch_kernel<step_detail::f32e, 16, true, TRACE>;
+        case 32: return batch_kernel<step_detail::f32e, 32, true, TRACE>;
         }
         return nullptr;
     }
     if (coal && wk == kWFp32) {
         switch (V) {
-        case 8: return batch_kernel<float, 8, true>;
-        case 16: return batch_kernel<float, 16, true>;
-        case 32: return batch_kernel<float, 32, true>;
+        case 8: return batch_kernel<float, 8, true, TRACE>;
+        case 16: return batch_kernel<float, 16, true, TRACE>;
+        case 32: return batch_kernel<float, 32, true, TRACE>;
         }
         return nullptr;
     }
     if (wk == kWInt16) {
         switch (V) {
-        case 4: return batch_kernel<int16_t, 4>;
-        case 8: return batch_kernel<int16_t, 8>;
-        case 16: return batch_kernel<int16_t, 16>;
-        case 32: return batch_kernel<int16_t, 32>;
+        case 4: return batch_kernel<int16_t, 4, false, TRACE>;
+        case 8: return batch_kernel<int16_t, 8, false, TRACE>;
+        case 16: return batch_kernel<int16_t, 16, false, TRACE>;
+        case 32: return batch_kernel<int16_t, 32, false, TRACE>;
         }
     } else if (wk == kWInt8AsF32) {
         switch (V) {
-        case 4: return batch_kernel<step_detail::f32e, 4>;
-        case 8: return batch_kernel<step_detail::f32e, 8>;
-        case 16: return batch_kernel<step_detail::f32e, 16>;
-        case 32: return batch_kernel<step_detail::f32e, 32>;
+        case 4: return batch_kernel<step_detail::f32e, 4, false, TRACE>;
+        case 8: return batch_kernel<step_detail::f32e, 8, false, TRACE>;
+        case 16: return batch_kernel<step_detail::f32e, 16, false, TRACE>;
+        case 32: return batch_kernel<step_detail::f32e, 32, false, TRACE>;
         }
     } else {
         switch (V) {
-        case 4: return batch_kernel<float, 4>;
-        case 8: return batch_kernel<float, 8>;
-        case 16: return batch_kernel<float, 16>;
-        case 32: return batch_kernel<float, 32>;
+        case 4: return batch_kernel<float, 4, false, TRACE>;
+        case 8: return batch_kernel<float, 8, false, TRACE>;
+        case 16: return batch_kernel<float, 16, false, TRACE>;
+        case 32: return batch_kernel<float, 32, false, TRACE>;
         }
     }
     return nullptr;
@@ -338,10 +345,11 @@ struct BatchClass {
     unsigned long long* head;
     int2* groups_dev;            // room for the groups of 2 replicas (the smallest staged group)
     int max_N;
+    bool traced = false;         // an item wants its trace
     BatchConfig cfg;
     std::string probes;          // the tuner's measurements, for da_batch_describe
     size_t staged_bytes() const { return (size_t)max_N * 32 * V * 4; }
-    bool can_stage() const { return smem_kernel_for(wk, V) != nullptr && staged_bytes() <= kMaxStagedBytes; }
+    bool can_stage() const { return smem_kernel_for<false>(wk, V) != nullptr && staged_bytes() <= kMaxStagedBytes; }
     // rows from L2 may come in the one-warp row order (every item carries its copy, Host::Wc)
     bool coal() const { return (wk == kWFp32 || wk == kWInt8AsF32) && V >= 8; }
 };
@@ -365,15 +373,17 @@ cudaError_t launch_class(const BatchClass& c, const std::vector<int>& reps, cons
                          long long t_limit, int sms, cudaStream_t st, bool upload_groups)
 {
     BatchClassParams bp{c.items_dev, c.n_items, units, c.head, t_limit, nullptr, 0, 0};
+    const bool traced = c.traced && t_limit == 0;   // the tuner's probes leave no trace
     if (!cfg.smem) {
-        BatchKernel k = kernel_for(c.wk, c.V, cfg.coal && c.coal());
+        const bool coal = cfg.coal && c.coal();
+        BatchKernel k = traced ? kernel_for<true>(c.wk, c.V, coal) : kernel_for<false>(c.wk, c.V, coal);
         // no more blocks than the units need: the rest of the SMs is left to other classes
         const long long need = (units + cfg.warps_per_block - 1) / cfg.warps_per_block;
         const int blocks = (int)std::min<long long>(blocks_for(k, cfg.warps_per_block, sms, 0), need);
         k<<<blocks, cfg.warps_per_block * 32, 0, st>>>(bp);
         return cudaGetLastError();
     }
-    BatchKernel k = smem_kernel_for(c.wk, c.V);
+    BatchKernel k = traced ? smem_kernel_for<true>(c.wk, c.V) : smem_kernel_for<false>(c.wk, c.V);
     const size_t bytes = c.staged_bytes();
     cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k),
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
@@ -567,6 +577,7 @@ extern "C" da_status da_batch_anneal(const da_batch_item* items, int32_t n, doub
         c.V = hi[i].V;
         c.max_N = std::max(c.max_N, hi[i].N);
         c.item_idx.push_back(i);
+        c.traced = c.traced || (items[i].out && items[i].out->trace);
     }
     const size_t o_desc = off;
     off += da::al((size_t)n * sizeof(BatchItemDev));
@@ -846,7 +857,7 @@ namespace da {
 cudaError_t launch_resident_anneal(int wk, int V, const BatchItemDev* item_dev, unsigned long long* head_dev, int R,
                                    cudaStream_t st)
 {
-    BatchKernel k = kernel_for(wk, V, false);   // a request's item carries no row-ordered copy
+    BatchKernel k = kernel_for<false>(wk, V, false);   // a request's item carries no row-ordered copy
     if (!k) return cudaErrorInvalidValue;
     prefer_shared_fn(reinterpret_cast<const void*>(k));
     cudaError_t e = cudaMemsetAsync(head_dev, 0, sizeof(unsigned long long), st);
@@ -859,7 +870,7 @@ cudaError_t launch_resident_anneal(int wk, int V, const BatchItemDev* item_dev, 
 cudaError_t prepare_resident_kernels()
 {
     for (int wk : {kWInt8AsF32, kWFp32, kWInt16})
-        for (int V : {4, 8, 16, 32}) prefer_shared_fn(reinterpret_cast<const void*>(kernel_for(wk, V, false)));
+        for (int V : {4, 8, 16, 32}) prefer_shared_fn(reinterpret_cast<const void*>(kernel_for<false>(wk, V, false)));
     return cudaGetLastError();
 }
 
