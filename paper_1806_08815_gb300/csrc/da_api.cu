@@ -94,7 +94,9 @@ const void* step_W(const da_ctx* c) { return c->Wf ? c->Wf : c->W; }
 //   N = 500:  R = 304 .622 / .609 / .574, R = 512 .625 / .702 / .811;
 //   N = 1024: R = 304 .917 / .738 / .693, R = 512 .926 / .951 / 1.094;
 //   N = 2048: R = 304 - / 1.294 / .978 / 1.195, R = 512 - / 1.633 / 1.666 / 2.283,
-//             R = 1024 - / 3.237 / 2.850 / 3.958;
+//             R = 1024 - / 3.237 / 2.850 / 3.958; beyond two full waves of four warps (1216
+//             replicas) two warps, two replicas to a block, at R = 1400 - / 3.93 / 4.27,
+//             R = 2048 - / 5.53 / 5.88, R = 8192 - / 19.7 / 22.0;
 //   N = 4096: R = 152 - / - / 1.354 / 1.141, R = 256 - / - / 1.678 / 2.132.
 //
 // Up to kClusterReplicas the widest shapes (8 warps of V = 16 or 32, N > 2048) run on
@@ -113,14 +115,14 @@ StepShape auto_shape(int N, int R)
     int G;
     if (N <= 256) G = 1;
     else if (N <= 1024) G = R <= 2 * kSMs ? 4 : 1;
-    else if (N <= 2048) G = 4;
+    else if (N <= 2048) G = R <= 8 * kSMs ? 4 : 2;
     else if (N <= 4096) G = R <= kSMs ? 8 : 4;
     else G = 8;
     StepShape s;
     s.G = G;
     s.V = G == 8 ? 8 : 4;
     while (32 * s.V * G < N) s.V *= 2;
-    s.rpb = G == 1 ? 4 : 1;
+    s.rpb = G == 1 ? 4 : G == 2 ? 2 : 1;
     if (G == 8 && s.V >= 16 && R <= kClusterReplicas) s.cluster = 4;
     return s;
 }

@@ -25,6 +25,8 @@ def test_automatic_shapes_over_all_sizes(da):
             assert blocks == (4 if N > 2048 and R <= 38 else 1), (N, R)
             if N <= 256:
                 assert G == 1
+            if 1024 < N <= 2048:
+                assert (G, rpb) == ((4, 1) if R <= 1216 else (2, 2))
 
 
 def test_arguments_are_checked(da):
