@@ -330,13 +330,56 @@ da_status finalize(const da_ctx* c, const RunBuffers& b, cudaStream_t st)
     return DA_OK;
 }
 
-// ... and, after `host` = that block and the states have arrived, out of it into `out`.  One
-// copy of all of it: every copy to pageable memory is a round trip of about 10 us, and the
-// three arrays, the flag and the scalars were five of them.
-size_t result_bytes(const RunBuffers& b) { return b.L.sc - b.L.res; }
+// ... and from there to the caller's arrays.  Every copy to pageable memory is a round trip of
+// about 10 us, so up to kStagedResults bytes the results, the flag and the states that are
+// asked for come in one copy and are taken apart on the host; a longer block costs more on
+// that way (its pages, and every byte twice) than the copies it saves.  us a call of one step:
+// N = 1024 with 2048 replicas (576 KB) 146 staged and 170 by array, N = 64 with 16384 replicas
+// and one state each (768 KB) 139 and 123, with 65536 and two (4 MB) 497 and 282.
+constexpr size_t kStagedResults = 3u << 18;
 
-void unpack_results(const da_ctx* c, const RunBuffers& b, const char* host, da_result* out)
+struct HostResults {
+    std::vector<char> staged;
+    int64_t flag = 0;         // the error flag, where nothing is staged
+};
+
+da_status fetch_results(const da_ctx* c, const RunBuffers& b, const da_result* out, cudaStream_t st, HostResults* h)
 {
+    const int R = b.R;
+    const size_t r8 = (size_t)R * 8, words = (size_t)da_words(c->N), nw = (size_t)b.s.nwords();
+    const char* res = b.base + b.L.res;
+    const size_t states = out ? (out->best_x ? 2 : out->final_x ? 1 : 0) : 0;
+    const size_t bytes = b.L.xs - b.L.res + states * R * nw * 4;
+    if (bytes <= kStagedResults) {
+        h->staged.resize(bytes);
+        DA_CU(cudaMemcpyAsync(h->staged.data(), res, bytes, cudaMemcpyDeviceToHost, st));
+        return DA_OK;
+    }
+    DA_CU(cudaMemcpyAsync(&h->flag, res + 4 * r8, sizeof(int), cudaMemcpyDeviceToHost, st));
+    void* const dst[4] = {out ? out->final_E : nullptr, out ? out->best_E : nullptr, out ? out->max_drift : nullptr,
+                          out ? out->flips : nullptr};
+    for (int k = 0; k < 4; ++k)
+        if (dst[k]) DA_CU(cudaMemcpyAsync(dst[k], res + k * r8, r8, cudaMemcpyDeviceToHost, st));
+    for (int k = 0; k < 2; ++k) {
+        uint32_t* x = !out ? nullptr : k ? out->best_x : out->final_x;
+        if (x) DA_CU(cudaMemcpy2DAsync(x, words * 4, k ? b.bestx() : b.x(), nw * 4, words * 4, R, cudaMemcpyDeviceToHost, st));
+    }
+    return DA_OK;
+}
+
+// After the copies have arrived: the error flag, and what was staged into `out`.
+int results_flag(const RunBuffers& b, const HostResults& h)
+{
+    int flag;
+    std::memcpy(&flag, h.staged.empty() ? reinterpret_cast<const char*>(&h.flag) : h.staged.data() + (size_t)4 * b.R * 8,
+                sizeof(int));
+    return flag;
+}
+
+void unpack_results(const da_ctx* c, const RunBuffers& b, const HostResults& h, da_result* out)
+{
+    if (h.staged.empty()) return;
+    const char* host = h.staged.data();
     const int R = b.R;
     const size_t words = (size_t)da_words(c->N), nw = (size_t)b.s.nwords();
     const size_t r8 = (size_t)R * 8;
@@ -758,18 +801,16 @@ da_status da_anneal(da_ctx* c, const float* beta, int64_t steps, float inc, int3
         DA_CU(cudaStreamSynchronize(st));
         return check_kernel_flag(c);
     }
-    std::vector<char> host(result_bytes(b));
-    DA_CU(cudaMemcpyAsync(host.data(), b.base + b.L.res, host.size(), cudaMemcpyDeviceToHost, st));
+    HostResults host;
+    if (da_status e = fetch_results(c, b, out, st, &host)) return e;
     if (want_trace && steps > 0)
         DA_CU(cudaMemcpyAsync(out->trace, b.base + b.L.trace, (size_t)R * steps * 4, cudaMemcpyDeviceToHost, st));
     DA_CU(cudaStreamSynchronize(st));
-    int flag;
-    std::memcpy(&flag, host.data() + (size_t)4 * R * 8, sizeof(int));
-    if (da_status e = report_flag(c, flag)) return e;
+    if (da_status e = report_flag(c, results_flag(b, host))) return e;
     float ms = 0.f;
     DA_CU(cudaEventElapsedTime(&ms, c->ev0, c->ev1));
     out->elapsed_s = ms * 1e-3;
-    unpack_results(c, b, host.data(), out);
+    unpack_results(c, b, host, out);
     return DA_OK;
 }
 
@@ -1268,21 +1309,19 @@ extern "C" da_status da_anneal_segment(da_ctx* c, const float* beta, int64_t tot
     if (da_status e = evaluate(c, b, st)) return e;
     if (da_status e = finalize(c, b, st)) return e;
     DA_CU(cudaEventRecord(c->ev1, st));
-    std::vector<char> host(result_bytes(b));
-    DA_CU(cudaMemcpyAsync(host.data(), b.base + b.L.res, host.size(), cudaMemcpyDeviceToHost, st));
+    HostResults host;
+    if (da_status e = fetch_results(c, b, res, st, &host)) return e;
     const size_t sc_idx = keep.size();
     if (out)
         if (da_status e = save_state(c, b, out, st, keep)) return e;
     DA_CU(cudaStreamSynchronize(st));
-    int flag;
-    std::memcpy(&flag, host.data() + (size_t)4 * R * 8, sizeof(int));
-    if (da_status e = report_flag(c, flag)) return e;
+    if (da_status e = report_flag(c, results_flag(b, host))) return e;
     if (out) finish_saved(c, R, out, out->scalars ? &keep[sc_idx] : nullptr);
     if (res) {
         float ms = 0.f;
         DA_CU(cudaEventElapsedTime(&ms, c->ev0, c->ev1));
         res->elapsed_s = ms * 1e-3;
-        unpack_results(c, b, host.data(), res);
+        unpack_results(c, b, host, res);
     }
     return DA_OK;
 }
