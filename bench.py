@@ -42,7 +42,7 @@ C3 = dict(N=1024, replicas=1024, steps=200_000, recompute_every=1024, beta0=0.1,
 # Warp instructions per replica-step of the step kernel (smsp__inst_executed.sum / (R x steps))
 # from the same capture: the issue-slot roofline of a kernel bound by instruction issue.
 STEP_INST_PER_REPLICA_STEP = 636.8
-STEP_TRAFFIC = {"source_sha256_16": "41c79345f9453bd3", "bytes_per_launch": 8.6321e6}
+STEP_TRAFFIC = {"source_sha256_16": "82f81c567715a5ea", "bytes_per_launch": 8.6321e6}
 
 
 def step_source_sha():

@@ -17,7 +17,7 @@ namespace da {
 constexpr int kWInt8 = 0, kWFp32 = 1, kWInt16 = 2, kWInt8AsF32 = 3;
 
 // Per-replica scalars kept in global memory between kernel launches.
-// E and best hold int64 energies (int8 instances) or fp64 bit patterns (fp32).
+// E and best hold int64 energies (integer couplings) or fp64 bit patterns (fp32).
 struct alignas(32) ReplicaScalars {
     long long E;       // tracked energy after the last completed step
     long long best;    // lowest tracked energy seen

@@ -5,7 +5,7 @@
 // (128 per tile, one per TMEM lane), the variables i the N side (64 per tile)
 // and the couplings j the K side.  Its value is defined exactly (da_fields.cu):
 // every coupling is put on the fixed-point grid, v_ij = round(W_ij 2^S) (the
-// int8 couplings themselves), and summed in integers.  The tensor cores reach
+// integer couplings themselves), and summed in integers.  The tensor cores reach
 // the same integers: v is split into balanced digits of b bits,
 //   v = sum_l d_l 2^(b l),   d_l in [-2^(b-1), 2^(b-1)),
 // every digit is exact in fp16 (|d| <= 2048), and b is chosen so that no
@@ -18,16 +18,17 @@
 // Operands use the tensor core's canonical K-major layout (8-row x 16-byte
 // core matrices, [K chunk][row group][8][8] halves per tile).  The digit planes
 // of the instance are built once per context in that layout in HBM, so a
-// pipeline stage takes them in one contiguous bulk copy; the states are not
-// staged in HBM at all: two warps of the block expand the tile's state bits
+// pipeline stage takes them in contiguous bulk copies; the states are not
+// staged in HBM at all: eight warps of the block expand the tile's state bits
 // (2 words per state and stage) to f16 {0, 1} directly into the stage.
 //
 // Block: 16 warps, 128 states x 64 variables.  Warp 0 allocates tensor memory and
 // issues the digit planes' bulk copies (4 KB a lane) into a 3-stage ring; warps 2-9
 // write the stage's state tile (half a state each, the word of the next chunk loaded
 // while the current one is written); one thread of warp 1 issues the MMAs (4 K-steps of
-// 16 per stage, the digit planes side by side as up to 192 columns of one or two MMAs:
-// one MMA of 64 columns per plane took 1.17 us a stage at 5 planes, this form 0.85) and
+// 16 per stage, the digit planes side by side as the columns of one MMA, up to four planes,
+// or of two: one MMA of 64 columns per plane took 1.17 us a stage at 5 planes, this form
+// 0.85) and
 // commits the stage back to both producers; then all 16 warps read their TMEM lanes
 // (warp w: states 32 (w % 4).., 16 variables from 16 (w / 4)) and write fields and
 // 128-bit partial energies, and the last block of a state tile sums those.
@@ -381,7 +382,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) recompute_tc_kernel(cons
             }
         }
     }
-    // partial energies of the 2 column groups, in the first stage's memory: every bulk
+    // partial energies of the four column groups, in the first stage's memory: every bulk
     // copy has landed and every MMA has read its operands once `done` has completed
     I128 (*s_part)[kBM] = reinterpret_cast<I128 (*)[kBM]>(sm);
     s_part[cg][m] = esum;

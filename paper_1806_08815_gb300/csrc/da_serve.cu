@@ -169,7 +169,7 @@ void plan_request(Req& q)
     size_t o = 0;
     auto take = [&](size_t b) { size_t at = o; o += al256(b); return at; };
     // W in the request's coupling type (what the exact final evaluation reads);
-    // int8 requests anneal on the same couplings held as exact fp32 (Wf)
+    // int8 requests anneal on the same couplings held as exact fp32 (Wf), int16 ones on W
     q.o_W = take(da::instance_W_bytes(q.N, q.dtype));
     if (q.dtype == DA_INT8) q.o_Wf = take(da::instance_W_bytes(q.N, DA_FP32));
     q.o_diag = take((size_t)q.N * 4);

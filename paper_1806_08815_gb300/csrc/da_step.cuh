@@ -172,8 +172,8 @@ __device__ __forceinline__ void cluster_drain()
 // 0.978, N = 4096 1.314, N = 8192 1.955; on several SMs they are (kClusterReplicas in
 // da_api.cu).
 // C > 1: the replica on the C blocks of a cluster, G warps in each (warp w of block c is
-// warp c G + w); published to every block, the cluster's barrier in the place of the
-// block's.
+// warp c G + w); published to every block by asynchronous stores, and the wait for the bytes
+// they bring (await_step) in the place of the block's barrier.
 template <typename Tw, int V, int G, bool FULL, bool TRACE, int C = 1>
 __global__ void __launch_bounds__(32 * G * OccupancyGV<G, V>::rpb, OccupancyGV<G, V>::min_blocks)
     step_kernel(const __grid_constant__ StepParams p)

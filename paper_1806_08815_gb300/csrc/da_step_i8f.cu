@@ -1,5 +1,5 @@
-// da_step_i8f.cu -- the step kernel for DA_INT8 contexts: the int8 couplings
-// held as exact fp32 (f32e in da_step_common.cuh), int64 energies.
+// da_step_i8f.cu -- the step kernel for integer couplings held as exact fp32 (every DA_INT8
+// context, DA_INT16 ones by their row sums; f32e in da_step_common.cuh), int64 energies.
 #include "da_step.cuh"
 
 namespace da {
