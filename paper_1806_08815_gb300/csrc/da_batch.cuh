@@ -70,6 +70,9 @@ __device__ __forceinline__ void run_unit(UnitShared<Tw>& u, int r, const Tw* W, 
     rp.m = 0;
     const std::conditional_t<SW, PhiloxKeys, PhiloxSeed> keys(it.seed);
     const float inc = it.inc;
+    const int* stop = it.stop;
+    // a period beyond any step count never comes
+    const uint32_t period = kReal && it.recompute_every <= 0xffffffffll ? (uint32_t)it.recompute_every : 0u;
     const uint32_t T = (uint32_t)(t_limit > 0 ? std::min(t_limit, it.T) : it.T);   // < 2^32
     rp.begin(0, T, it.beta, 0.f, 0, 0, 0, keys);
     // the steps up to the next point where something else is due: a recompute of the
@@ -85,9 +88,8 @@ __device__ __forceinline__ void run_unit(UnitShared<Tw>& u, int r, const Tw* W, 
             rp.draw(t, keys);
         }
         uint32_t t1 = T;
-        if (kReal && it.recompute_every > 0)
-            t1 = (uint32_t)std::min<long long>(t1, (t / it.recompute_every + 1) * it.recompute_every);
-        if (it.stop) t1 = (uint32_t)std::min<long long>(t1, ((long long)t / 1024 + 1) * 1024);
+        if (period > 0 && period - t % period < t1 - t) t1 = t + (period - t % period);
+        if (stop && 1024 - t % 1024 < t1 - t) t1 = t + (1024 - t % 1024);
         int k = -1;
         for (; t < t1; ++t) {
             k = rp.template step<false>(t, true, inc, keys);
@@ -95,9 +97,9 @@ __device__ __forceinline__ void run_unit(UnitShared<Tw>& u, int r, const Tw* W, 
                 if (it.trace && lane == 0) it.trace[(size_t)r * it.T + t] = k;
             }
         }
-        if (it.stop && t % 1024 == 0 && *reinterpret_cast<const volatile int*>(it.stop)) break;
+        if (stop && t % 1024 == 0 && *reinterpret_cast<const volatile int*>(stop)) break;
         if constexpr (kReal) {
-            if (it.recompute_every > 0 && t % it.recompute_every == 0) {
+            if (period > 0 && t % period == 0) {
                 if (rp.n > 0) rp.settle(k >= 0);
                 rp.recompute(static_cast<const float*>(it.diag), it.S);
                 rp.test_current();
