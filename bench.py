@@ -509,7 +509,7 @@ def profile_case(da, instances, case):
     """Small runs of the library's other kernels for ncu captures: `batched` (a two-class batched
     launch: fp32 N = 1024 from L2, int8 N = 64 staged), `ptda` (SK bimodal N = 512, 32 betas,
     20 sweeps), `plain` (the plain form, 200 steps of the headline workload), `g8` (fp32
-    N = 8192, 32 replicas: the 8-warp step kernel)."""
+    N = 8192, 32 replicas: the step kernel on clusters of four blocks)."""
     if case == "batched":
         T = 2048
         jobs = []
