@@ -131,6 +131,13 @@ std::vector<int2> make_groups(const std::vector<int>& replicas_per_item, int wpb
     return g;
 }
 
+BatchKernel class_kernel(const BatchClass& c, const BatchConfig& cfg, bool traced)
+{
+    if (cfg.smem) return traced ? traced_smem_kernel_for(c.wk, c.V) : smem_kernel_for(c.wk, c.V);
+    const bool coal = cfg.coal && c.coal();
+    return traced ? traced_kernel_for(c.wk, c.V, coal) : kernel_for(c.wk, c.V, coal);
+}
+
 // One launch of a class's kernel in configuration cfg over its first `units`
 // units (all of them for the real run), t_limit steps per unit (0: all).
 cudaError_t launch_class(const BatchClass& c, const std::vector<int>& reps, const BatchConfig& cfg, long long units,
@@ -139,15 +146,14 @@ cudaError_t launch_class(const BatchClass& c, const std::vector<int>& reps, cons
     BatchClassParams bp{c.items_dev, c.n_items, units, c.head, t_limit, nullptr, 0, 0};
     const bool traced = c.traced && t_limit == 0;   // the tuner's probes leave no trace
     if (!cfg.smem) {
-        const bool coal = cfg.coal && c.coal();
-        BatchKernel k = traced ? traced_kernel_for(c.wk, c.V, coal) : kernel_for(c.wk, c.V, coal);
+        BatchKernel k = class_kernel(c, cfg, traced);
         // no more blocks than the units need: the rest of the SMs is left to other classes
         const long long need = (units + cfg.warps_per_block - 1) / cfg.warps_per_block;
         const int blocks = (int)std::min<long long>(blocks_for(k, cfg.warps_per_block, sms, 0), need);
         k<<<blocks, cfg.warps_per_block * 32, 0, st>>>(bp);
         return cudaGetLastError();
     }
-    BatchKernel k = traced ? traced_smem_kernel_for(c.wk, c.V) : smem_kernel_for(c.wk, c.V);
+    BatchKernel k = class_kernel(c, cfg, traced);
     const size_t bytes = c.staged_bytes();
     cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k),
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
@@ -458,6 +464,9 @@ extern "C" da_status da_batch_anneal(const da_batch_item* items, int32_t n, doub
     for (auto& kv : classes) {
         BatchClass& c = kv.second;
         c.cfg = da::tune_class(c, reps[kv.first], dev, sms, st);
+        // the kernel of the real run is loaded here, not by its first launch under capture
+        cudaFuncAttributes fa;
+        DA_B(cudaFuncGetAttributes(&fa, reinterpret_cast<const void*>(da::class_kernel(c, c.cfg, c.traced))));
         desc_text += std::string(desc_text.empty() ? "" : "; ") + (c.wk == da::kWFp32 ? "fp32" : c.wk == da::kWInt16 ? "int16" : "integer as fp32") + " V=" +
                      std::to_string(c.V) + " (N <= " + std::to_string(c.max_N) + ", " + std::to_string(c.n_items) +
                      " instances, " + std::to_string(c.units) + " replicas): " +
